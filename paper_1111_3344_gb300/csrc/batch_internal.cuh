@@ -5,9 +5,9 @@
 namespace bssn {
 
 constexpr int BATCH_MAX = BSSN_BATCH_MAX_MEMBERS;
-// work lists of a batch: every active member (boundary, persistent and TMA
-// stage kernels); float64 members with full tiles and the others (the
-// one-block-per-tile stage kernels, one point function each)
+// work lists of a batch: every active member (boundary, persistent, TMA and
+// float64 or mixed one-block-per-tile stage kernels); double-word members with
+// full tiles and the others (one point function each)
 constexpr int WORK_ALL = 0, WORK_FULL = 1, WORK_REST = 2, NWORK = 3;
 
 // One member as the batched kernels see it: its grid and the arguments of its
@@ -77,15 +77,14 @@ bool batch_tile_is_members(int c);
 // ("members" 16, "members4" 4, "members1" 1; 0 for other configurations)
 int batch_members_streams(int c);
 int batch_default_tile_ff();
-// Whether a float64 member has full tiles under configuration cfg (n0 a
+// Whether a member has full tiles under configuration cfg (n0 a
 // multiple of 32 = the tile's x extent, n1 and n2 of its y and z extents).
 bool batch_tile_full(int cfg, const Grid& g);
 // Stage kernel over the tiles of one work list.  Persistent and TMA-staged
 // configurations: grid = resident blocks, every member (WORK_ALL).
-// One-block-per-tile configurations: grid = ntiles, the list's tile count;
-// full selects the full-block float64 point function (WORK_FULL).  err: device
-// error word (a bounded wait of the TMA kernel gave up).
-cudaError_t launch_batch_stage(int cfg, bool mixed, bool full, const MemberDev* mem, const BatchWork* wk,
+// One-block-per-tile configurations: grid = ntiles, the list's tile count.
+// err: device error word (a bounded wait of the TMA kernel gave up).
+cudaError_t launch_batch_stage(int cfg, bool mixed, const MemberDev* mem, const BatchWork* wk,
                                unsigned ntiles, int stage, int* err, cudaStream_t s);
 // TMA-staged forms (k_batch_tma.cu), variant v: 0 = 32x4x1 tiles with 8
 // staged fields, 1 = 32x8x1 tiles with 11; batch_tma_variant(cfg): the

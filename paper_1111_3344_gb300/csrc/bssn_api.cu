@@ -326,7 +326,7 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
     ctx->ks64 = p->ksum_fp64 ? (double*)(ctx->mem + c.ks64) : nullptr;
   }
   ctx->shadow_valid = false;
-  ctx->tile = p->precision == BSSN_FF ? ff_cfg_index(0) : 0;
+  ctx->tile = p->precision == BSSN_FF ? ff_cfg_index(0) : (p->precision == BSSN_FP64 ? fp64_default_tile() : 0);
   ctx->part = (double*)(ctx->mem + c.part);
   ctx->out16 = (double*)(ctx->mem + c.out16);
   ctx->t = 0.0;

@@ -409,9 +409,9 @@ cudaError_t launch_members(bssn_batch* b, int s0, int s1, bool bc) {
 }
 
 // The stage launches of one RK4 stage under configuration cfg: persistent and
-// TMA-staged kernels, one launch over every member; one-block-per-tile
-// kernels, one launch per float64 list (members with full tiles, the others),
-// or one over every member (mixed).
+// TMA-staged and float64 or mixed one-block-per-tile kernels, one launch over
+// every member; double-word kernels, one launch per list (members with full
+// tiles, the others).
 cudaError_t launch_stage_lists(bssn_batch* b, int cfg, int stage) {
   if (batch_tile_is_members(cfg)) return launch_members(b, stage, stage + 1, false);
   const bool mixed = b->precision == BSSN_MIXED;
@@ -424,15 +424,8 @@ cudaError_t launch_stage_lists(bssn_batch* b, int cfg, int stage) {
                                 b->stream);
     return e;
   }
-  if (!batch_tile_is_per_tile(cfg) || mixed)
-    return launch_batch_stage(cfg, mixed, false, b->d_mem, b->d_work + WORK_ALL, b->h_work[WORK_ALL].total_tiles,
-                              stage, b->d_err, b->stream);
-  cudaError_t e = launch_batch_stage(cfg, false, true, b->d_mem, b->d_work + WORK_FULL,
-                                     b->h_work[WORK_FULL].total_tiles, stage, b->d_err, b->stream);
-  if (e == cudaSuccess)
-    e = launch_batch_stage(cfg, false, false, b->d_mem, b->d_work + WORK_REST, b->h_work[WORK_REST].total_tiles,
-                           stage, b->d_err, b->stream);
-  return e;
+  return launch_batch_stage(cfg, mixed, b->d_mem, b->d_work + WORK_ALL, b->h_work[WORK_ALL].total_tiles, stage,
+                            b->d_err, b->stream);
 }
 
 cudaError_t capture(bssn_batch* b) {

@@ -46,6 +46,7 @@ struct Grid {
   // precisions (a float64 division or conversion costs a slot of the slow
   // float64 pipe on every thread that would otherwise compute it)
   double i12h, i12h2, i144h2, kos, i2h;  // 1/(12h), 1/(12h^2), 1/(144h^2), eps/(64h), 1/(2h)
+  double h12;  // 12 h
   float i12hf, i12h2f, i144h2f, kosf, i2hf, w_floorf, etaf, hf;
   // the float remainders d - (double)f of the same constants (the low words
   // of their double-word forms)
@@ -58,6 +59,7 @@ struct Grid {
 
 // Host-side fill of the derived constants of a Grid.
 inline void grid_constants(Grid& g) {
+  g.h12 = 12.0 * g.h;
   g.i12h = 1.0 / (12.0 * g.h);
   g.i12h2 = 1.0 / (12.0 * g.h * g.h);
   g.i144h2 = 1.0 / (144.0 * g.h * g.h);
@@ -304,6 +306,7 @@ cudaError_t launch_stage_fp64(const Grid& g, const StageArgs& a, cudaStream_t s,
 cudaError_t launch_stage_mixed(const Grid& g, const StageArgsMixed& a, cudaStream_t s, int cfg = 0);
 cudaError_t launch_stage_mixed_ks64(const Grid& g, const StageArgsMixed& a, cudaStream_t s);
 int tile_config_count();
+int fp64_default_tile();  // of a new float64 context
 bool tile_config_has_fp64(int c);  // false for the mixed-only configurations
 const char* tile_config_name(int c);
 // TMA-staged mixed stage kernel (k_stage_tma.cu); map describes the float

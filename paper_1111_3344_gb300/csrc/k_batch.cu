@@ -67,13 +67,9 @@ __global__ void __launch_bounds__(TX * TY * TZ, MINB)
 
 // Float64 persistent stage: the body of one tile is a call of its own
 // (__noinline__), so that it gets the register allocation of a one-tile
-// kernel.  Inlined into the loop over tiles, the float64 stage spills
-// 1.2-1.8 KB per thread whether its arguments sit in shared memory or in the
-// member table; behind the call, about 330 B (full tiles, 255 registers).  The callee reads the member's grid and
-// stage arguments from the read-only member table.  FULL: the member has full
-// tiles (every warp a full x-row, every thread of the block inside the grid),
-// which the caller decides uniformly over the block.
-template <int TY, int TZ, bool FULL>
+// kernel; the callee reads the member's grid and stage arguments from the
+// read-only member table.
+template <int TY, int TZ>
 __device__ __noinline__ void batch_fp64_tile(const MemberDev* __restrict__ mem, int sid, unsigned lt, int stage) {
   const MemberDev& M = mem[sid];
   const int bx = (int)(lt % (unsigned)M.tiles[0]);
@@ -81,41 +77,34 @@ __device__ __noinline__ void batch_fp64_tile(const MemberDev* __restrict__ mem, 
   const int by = (int)(lt % (unsigned)M.tiles[1]);
   const int bz = (int)(lt / (unsigned)M.tiles[1]);
   const int ii = bx * 32 + threadIdx.x, jj = by * TY + threadIdx.y, kk = bz * TZ + threadIdx.z;
-  if constexpr (FULL)
-    stage_point_fp64<32, TY, TZ>(M.g, M.a64[stage], ii, jj, kk);
-  else if (ii < M.g.n0 && jj < M.g.n1 && kk < M.g.n2)
-    stage_point_fp64<0>(M.g, M.a64[stage], ii, jj, kk);
+  if (ii < M.g.n0 && jj < M.g.n1 && kk < M.g.n2) stage_point_fp64(M.g, M.a64[stage], ii, jj, kk);
 }
 
 template <int TY, int TZ, int MINB>
 __global__ void __launch_bounds__(32 * TY * TZ, MINB)
     batch_stage_fp64_kernel(const MemberDev* __restrict__ mem, const BatchWork* __restrict__ wk, int stage) {
-  __shared__ int sid, sfull;
+  __shared__ int sid;
   __shared__ unsigned slocal;
   const int tid = threadIdx.x + 32 * (threadIdx.y + TY * threadIdx.z);
   const unsigned total = wk->total_tiles;
   const int count = wk->count;
   // thread 0: the member of the block's current tile and its tile range
   unsigned t_lo = 1u, t_hi = 0u;
-  int cur = 0, full = 0;
+  int cur = 0;
   for (unsigned t = blockIdx.x; t < total; t += gridDim.x) {
-    __syncthreads();  // the previous tile is done with sid, sfull, slocal
+    __syncthreads();  // the previous tile is done with sid, slocal
     if (tid == 0) {
       if (t < t_lo || t >= t_hi) {
         const int slot = find_member(wk->tile_base, count, t);
         cur = wk->member[slot];
-        const Grid& g = mem[cur].g;
-        full = g.n0 % 32 == 0 && g.n1 % TY == 0 && g.n2 % TZ == 0;
         t_lo = wk->tile_base[slot];
         t_hi = wk->tile_base[slot + 1];
       }
       sid = cur;
-      sfull = full;
       slocal = t - t_lo;
     }
     __syncthreads();
-    if (sfull) batch_fp64_tile<TY, TZ, true>(mem, sid, slocal, stage);
-    else batch_fp64_tile<TY, TZ, false>(mem, sid, slocal, stage);
+    batch_fp64_tile<TY, TZ>(mem, sid, slocal, stage);
   }
 }
 
@@ -123,10 +112,8 @@ __global__ void __launch_bounds__(32 * TY * TZ, MINB)
 // block looks up its member once and runs one point function.  Against the
 // persistent kernel above this trades the resident-block loop for a launch
 // over all tiles; the compiler then allocates registers as for a single-grid
-// stage (about 200 B of spills per thread for float64, against 1.2-1.8 KB in
-// the loop).  FULL (float64): every member of the list has full tiles, so every
-// warp is a full x-row and every thread of a block is inside the grid.
-template <int TX, int TY, int TZ, int MINB, bool MIXED, bool FULL>
+// stage.
+template <int TX, int TY, int TZ, int MINB, bool MIXED>
 __global__ void __launch_bounds__(TX * TY * TZ, MINB)
     batch_tile_kernel(const MemberDev* __restrict__ mem, const BatchWork* __restrict__ wk, int stage) {
   __shared__ int sid;
@@ -150,10 +137,8 @@ __global__ void __launch_bounds__(TX * TY * TZ, MINB)
   if (ii < M.g.n0 && jj < M.g.n1 && kk < M.g.n2) {
     if constexpr (MIXED)
       stage_point_mixed(M.g, M.amx[stage], ii, jj, kk);
-    else if constexpr (FULL && TX == 32)
-      stage_point_fp64<32, TY, TZ>(M.g, M.a64[stage], ii, jj, kk);
     else
-      stage_point_fp64<0>(M.g, M.a64[stage], ii, jj, kk);
+      stage_point_fp64(M.g, M.a64[stage], ii, jj, kk);
   }
 }
 
@@ -205,9 +190,10 @@ struct BatchCfg {
   const void* kmx;
 };
 
+// float64 forms: 16 warps per SM (see stage_fp64_kernel)
 #define BCFG(TX, TY, TZ, MINB)                                                       \
   { #TX "x" #TY "x" #TZ "/" #MINB, TX, TY, TZ,                                      \
-    (const void*)batch_stage_fp64_kernel<TY, TZ, MINB>,                             \
+    (const void*)batch_stage_fp64_kernel<TY, TZ, 512 / (32 * TY * TZ)>,             \
     (const void*)batch_stage_kernel<TX, TY, TZ, MINB> }
 static const BatchCfg k_bcfg[] = {
     BCFG(32, 8, 1, 1), BCFG(32, 2, 2, 2), BCFG(32, 4, 1, 3), BCFG(32, 4, 2, 1),
@@ -218,15 +204,13 @@ static const BatchCfg k_bcfg[] = {
 struct TileCfgB {
   const char* name;
   int tx, ty, tz;
-  const void* k64full;
   const void* k64;
   const void* kmx;
 };
 #define TCFG(TX, TY, TZ, MINB)                                                      \
   { "tiles" #TX "x" #TY "x" #TZ "/" #MINB, TX, TY, TZ,                            \
-    (const void*)batch_tile_kernel<TX, TY, TZ, MINB, false, true>,                \
-    (const void*)batch_tile_kernel<TX, TY, TZ, MINB, false, false>,               \
-    (const void*)batch_tile_kernel<TX, TY, TZ, MINB, true, false> }
+    (const void*)batch_tile_kernel<TX, TY, TZ, 512 / (TX * TY * TZ), false>,      \
+    (const void*)batch_tile_kernel<TX, TY, TZ, MINB, true> }
 static const TileCfgB k_tcfg[] = {TCFG(32, 4, 1, 2), TCFG(32, 8, 1, 1)};
 #undef TCFG
 
@@ -304,41 +288,31 @@ bool batch_tile_full(int cfg, const Grid& g) {
   return tx == 32 && g.n0 % 32 == 0 && g.n1 % ty == 0 && g.n2 % tz == 0;
 }
 
-cudaError_t launch_batch_stage(int cfg, bool mixed, bool full, const MemberDev* mem, const BatchWork* wk,
+cudaError_t launch_batch_stage(int cfg, bool mixed, const MemberDev* mem, const BatchWork* wk,
                                unsigned ntiles, int stage, int* err, cudaStream_t s) {
   if (batch_tma_variant(cfg) >= 0 && mixed) return launch_batch_stage_tma(batch_tma_variant(cfg), mem, wk, stage, err, s);
   if (batch_tile_is_per_tile(cfg) && batch_ff_variant(cfg) < 0) {
     const TileCfgB& c = k_tcfg[cfg - N_FUSED];
     if (ntiles == 0) return cudaSuccess;
-    full = full && !mixed;
-    const void* fn = mixed ? c.kmx : (full ? c.k64full : c.k64);
-    const size_t smem = full ? rows_block_smem(c.ty, c.tz, true) : 0;
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const void* fn = mixed ? c.kmx : c.k64;
     dim3 block(c.tx, c.ty, c.tz);
     void* args[] = {(void*)&mem, (void*)&wk, (void*)&stage};
-    return cudaLaunchKernel(fn, dim3(ntiles), block, args, smem, s);
+    return cudaLaunchKernel(fn, dim3(ntiles), block, args, 0, s);
   }
   if (cfg < 0 || cfg >= N_FUSED) cfg = 0;
   const BatchCfg& c = k_bcfg[cfg];
   const void* fn = mixed ? c.kmx : c.k64;
   const int threads = c.tx * c.ty * c.tz;
-  // float64 full-block tiles exchange first differences through shared memory
-  const size_t smem = (!mixed && c.tx == 32) ? rows_block_smem(c.ty, c.tz, true) : 0;
   int dev = 0, sms = 0, per = 0;
-  cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                                   : cudaSuccess;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, 0);
   if (e != cudaSuccess) return e;
   if (per < 1) per = 1;
   dim3 block(c.tx, c.ty, c.tz);
   dim3 grid((unsigned)(sms * per));
   void* args[] = {(void*)&mem, (void*)&wk, (void*)&stage};
-  return cudaLaunchKernel(fn, grid, block, args, smem, s);
+  return cudaLaunchKernel(fn, grid, block, args, 0, s);
 }
 
 cudaError_t launch_batch_boundary(bool mixed, const MemberDev* mem, const BatchWork* wk, int stage,

@@ -113,7 +113,7 @@ cudaError_t launch_batch_stage_ff(int v, bool full, const MemberDev* mem, const 
   if (ntiles == 0) return cudaSuccess;
   const FfBatchCfg& c = k_ffcfg[v];
   const void* fn = full ? c.kfull : c.krest;
-  const size_t smem = full ? rows_block_smem(c.ty, c.tz, false) : 0;
+  const size_t smem = full ? rows_block_smem(c.ty, c.tz) : 0;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

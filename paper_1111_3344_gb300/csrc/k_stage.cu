@@ -26,14 +26,32 @@
 
 namespace bssn {
 
-// One thread per interior point; TX x TY x TZ points per block.
+// Float64: one thread per interior point, blocks of TX x TY x TZ points where
+// these divide the grid; else (flat) blocks of as many consecutive points of
+// the interior in x-y-z order, so that no thread and no warp but the last is
+// without a point (75 x 53 x 61: 5.9 against 8.1 thousand warps of 32 x 4 tiles).
+// MINB keeps 16 warps per SM resident (128 registers, spills of some 700 B per
+// thread): the stencils wait on loads and integer chains, the algebra on the
+// float64 pipe, and only other warps fill either's gaps.  At 128^3 a step takes
+// 19.1 ms with 16 warps, 20.2 with 12, 25.3 with 8.
 template <int TX, int TY, int TZ, int MINB>
-__global__ void __launch_bounds__(TX * TY * TZ, MINB) stage_fp64_kernel(Grid g, StageArgs a) {
-  const int ii = blockIdx.x * TX + threadIdx.x;
-  const int jj = blockIdx.y * TY + threadIdx.y;
-  const int kk = blockIdx.z * TZ + threadIdx.z;
-  if (ii >= g.n0 || jj >= g.n1 || kk >= g.n2) return;
-  stage_point_fp64<0>(g, a, ii, jj, kk);
+__global__ void __launch_bounds__(TX * TY * TZ, MINB) stage_fp64_kernel(Grid g, StageArgs a, bool flat) {
+  int ii, jj, kk;
+  if (flat) {
+    const unsigned tid = threadIdx.x + TX * (threadIdx.y + TY * threadIdx.z);
+    const unsigned long long q = (unsigned long long)blockIdx.x * (TX * TY * TZ) + tid;
+    const unsigned pl = (unsigned)g.n0 * (unsigned)g.n1;
+    kk = (int)(q / pl);
+    const unsigned r = (unsigned)(q - (unsigned long long)kk * pl);
+    jj = (int)(r / (unsigned)g.n0);
+    ii = (int)(r - (unsigned)jj * (unsigned)g.n0);
+    if (kk >= g.n2) return;
+  } else {
+    ii = blockIdx.x * TX + threadIdx.x;
+    jj = blockIdx.y * TY + threadIdx.y;
+    kk = blockIdx.z * TZ + threadIdx.z;
+  }
+  stage_point_fp64(g, a, ii, jj, kk);
 }
 
 template <int TX, int TY, int TZ, int MINB, bool KS64 = false>
@@ -45,23 +63,19 @@ __global__ void __launch_bounds__(TX * TY * TZ, MINB) stage_mixed_kernel(Grid g,
   stage_point_mixed<KS64>(g, a, ii, jj, kk);
 }
 
-// float64 full-row variants, defined in k_stage_shfl.cu
-template <int TY, int TZ, int MINB>
-cudaError_t launch_fp64_rows(const Grid& g, const StageArgs& a, cudaStream_t s);
-extern template cudaError_t launch_fp64_rows<8, 1, 1>(const Grid&, const StageArgs&, cudaStream_t);
-extern template cudaError_t launch_fp64_rows<4, 1, 1>(const Grid&, const StageArgs&, cudaStream_t);
-extern template cudaError_t launch_fp64_rows<4, 2, 1>(const Grid&, const StageArgs&, cudaStream_t);
-extern template cudaError_t launch_fp64_rows<2, 2, 2>(const Grid&, const StageArgs&, cudaStream_t);
-
 // ------------------------------------------------------ tile configurations
 // Candidate block shapes (points per block along x, y, z) and the minimum
 // resident blocks per SM handed to the compiler (which caps registers and so
 // trades spills for occupancy).  The autotuner times them on the live state.
 template <int TX, int TY, int TZ, int MINB>
 static cudaError_t launch_fp64_t(const Grid& g, const StageArgs& a, cudaStream_t s) {
-  dim3 block(TX, TY, TZ);
-  dim3 grid((g.n0 + TX - 1) / TX, (g.n1 + TY - 1) / TY, (g.n2 + TZ - 1) / TZ);
-  stage_fp64_kernel<TX, TY, TZ, MINB><<<grid, block, 0, s>>>(g, a);
+  constexpr int MB = MINB > 512 / (TX * TY * TZ) ? MINB : 512 / (TX * TY * TZ);  // 16 warps per SM
+  const bool flat = g.n0 % TX || g.n1 % TY || g.n2 % TZ;
+  const unsigned long long pts = (unsigned long long)g.n0 * g.n1 * g.n2;
+  const dim3 block(TX, TY, TZ);
+  const dim3 grid = flat ? dim3((unsigned)((pts + TX * TY * TZ - 1) / (TX * TY * TZ)))
+                         : dim3(g.n0 / TX, g.n1 / TY, g.n2 / TZ);
+  stage_fp64_kernel<TX, TY, TZ, MB><<<grid, block, 0, s>>>(g, a, flat);
   return cudaGetLastError();
 }
 template <int TX, int TY, int TZ, int MINB>
@@ -76,30 +90,26 @@ struct TileCfg {
   const char* name;
   cudaError_t (*fp64)(const Grid&, const StageArgs&, cudaStream_t);
   cudaError_t (*mixed)(const Grid&, const StageArgsMixed&, cudaStream_t);
-  // float64 variant whose warps are full 32-point x-rows sharing first
-  // differences (k_stage_shfl.cu); used when n0 is a multiple of 32
-  cudaError_t (*fp64_rows)(const Grid&, const StageArgs&, cudaStream_t);
 };
 
 #define TILE(TX, TY, TZ, MINB)                                                  \
   { #TX "x" #TY "x" #TZ "/" #MINB, launch_fp64_t<TX, TY, TZ, MINB>,            \
-    launch_mixed_t<TX, TY, TZ, MINB>, nullptr }
-#define TILE_ROWS(TY, TZ, MINB)                                                 \
-  { "32x" #TY "x" #TZ "/" #MINB, launch_fp64_t<32, TY, TZ, MINB>,              \
-    launch_mixed_t<32, TY, TZ, MINB>, launch_fp64_rows<TY, TZ, MINB> }
+    launch_mixed_t<TX, TY, TZ, MINB> }
 // mixed only: registers capped for four or six resident blocks per SM (more
 // warps to cover the load latency, more spills)
 #define TILE_MX(TX, TY, TZ, MINB) \
-  { #TX "x" #TY "x" #TZ "/" #MINB, nullptr, launch_mixed_t<TX, TY, TZ, MINB>, nullptr }
+  { #TX "x" #TY "x" #TZ "/" #MINB, nullptr, launch_mixed_t<TX, TY, TZ, MINB> }
 static const TileCfg k_tiles[] = {
-    TILE_ROWS(8, 1, 1), TILE_ROWS(4, 1, 1), TILE_ROWS(4, 2, 1), TILE(64, 4, 1, 1),
-    TILE(16, 8, 2, 1), TILE_ROWS(2, 2, 2), TILE(32, 8, 1, 2), TILE(32, 4, 1, 3),
+    TILE(32, 8, 1, 1), TILE(32, 4, 1, 1), TILE(32, 4, 2, 1), TILE(64, 4, 1, 1),
+    TILE(16, 8, 2, 1), TILE(32, 2, 2, 2), TILE(32, 8, 1, 2), TILE(32, 4, 1, 3),
     TILE_MX(32, 4, 1, 4), TILE_MX(32, 4, 1, 6),
 };
 #undef TILE_MX
 #undef TILE
-#undef TILE_ROWS
 
+// 32 x 4 x 1 blocks: 19.1 ms a step at 128^3 against 20.1 for 32 x 8 x 1
+// (smaller blocks leave together more evenly)
+int fp64_default_tile() { return 1; }
 int tile_config_count() { return (int)(sizeof(k_tiles) / sizeof(k_tiles[0])); }
 bool tile_config_has_fp64(int c) { return c >= 0 && c < tile_config_count() && k_tiles[c].fp64 != nullptr; }
 const char* tile_config_name(int c) {
@@ -108,7 +118,6 @@ const char* tile_config_name(int c) {
 
 cudaError_t launch_stage_fp64(const Grid& g, const StageArgs& a, cudaStream_t s, int cfg) {
   if (!tile_config_has_fp64(cfg)) cfg = 0;
-  if (k_tiles[cfg].fp64_rows && g.n0 % 32 == 0) return k_tiles[cfg].fp64_rows(g, a, s);
   return k_tiles[cfg].fp64(g, a, s);
 }
 

@@ -3,9 +3,9 @@
 // phi, gt, At, Gt with m = 1 in vacuum; Ricci pieces Rt_ij and Rphi_ij; 1+log
 // / harmonic / geodesic slicing; Gamma-driver shift with q(r)).
 //
-// Formulation (same discrete operator as the statement in the paper; the
-// arrangement is chosen to cut float64 instructions, the binding resource on
-// GB300):
+// Float and double-word forms (the float64 one is rhs_fx.cuh).  Formulation
+// (same discrete operator as the statement in the paper; the arrangement is
+// chosen to cut instructions):
 //  - symmetric tensors held as 6 components; gt^{ij} by cofactors over det;
 //  - second derivatives are consumed as they are produced (the
 //    gt^{kl} d_k d_l contractions are accumulated pair by pair) to keep the
@@ -107,10 +107,8 @@ __device__ __forceinline__ T dmu(const A& acc, int f, const P* p, long long sa, 
 // consecutive x points of one row: v is this point's first difference along b
 // (already formed, scaled by 1/(12h)); the lanes x-1, x+1, x-2, x+2 hold
 // theirs, so only the two lanes at each end of the row form one more
-// (at x -+ 2), and the mixed difference costs 3 float64 operations instead
-// of 15.  Same stencil as dmu (D1 along x applied to D1 along b); the result
+// (at x -+ 2), and the mixed difference costs 3 operations instead of 15.  Same stencil as dmu (D1 along x applied to D1 along b); the result
 // is 12 h times the mixed derivative (v already carries 1/(12h)).
-__device__ __forceinline__ double shflT(double v, int src, int W) { return __shfl_sync(0xffffffffu, v, src, W); }
 __device__ __forceinline__ ff shflT(ff v, int src, int W) {
   return ff(__shfl_sync(0xffffffffu, v.hi, src, W), __shfl_sync(0xffffffffu, v.lo, src, W));
 }
@@ -132,45 +130,11 @@ __device__ __forceinline__ T dmx_shfl(const A& acc, int f, const P* p, long long
   const T vp2 = lane <= W - 3 ? sp2 : ve;
   return fmaT<T>(T(8), vp1 - vm1, -(vp2 - vm2));
 }
-// The same mixed difference with the four first differences past the ends of
-// the row already formed (float64 full blocks): xe[0..3] hold them at
-// x_0 - 2, x_0 - 1, x_{W-1} + 1, x_{W-1} + 2, in shared memory.
-template <int W, typename T>
-__device__ __forceinline__ T dmx_pre(T v, const T* xe) {
-  const int lane = threadIdx.x & (W - 1);
-  const T sm2 = shflT(v, lane - 2, W);
-  const T sm1 = shflT(v, lane - 1, W);
-  const T sp1 = shflT(v, lane + 1, W);
-  const T sp2 = shflT(v, lane + 2, W);
-  // indices clamped to 0..3 on every lane, so that no lane reads past xe
-  const T vm2 = lane >= 2 ? sm2 : xe[lane < 2 ? lane : 0];
-  const T vm1 = lane >= 1 ? sm1 : xe[1];
-  const T vp1 = lane <= W - 2 ? sp1 : xe[2];
-  const T vp2 = lane <= W - 3 ? sp2 : xe[lane >= W - 2 ? lane - W + 4 : 3];
-  return fmaT<T>(T(8), vp1 - vm1, -(vp2 - vm2));
-}
-
-// x-mixed difference of the q-th of the 11 twice-differenced fields (gt_ij,
-// phi|W, alpha, beta^i) along axis b (1 or 2): from the staged end-of-row
-// values on float64 full blocks, else with the end lanes forming their own.
-// (Double-word blocks keep the end lanes' own: the 88 values per warp cost
-// them shared memory that their register spills use as L1, and the stage
-// measured 3 % slower, 30 % in the batch.)
-template <int W, int YROWS, typename T, typename A, typename P>
-__device__ __forceinline__ T dmx_row(const A& acc, int f, const P* p, long long sb, T v, T i12h, const T* xep,
-                                     int b, int q) {
-  if constexpr (YROWS > 0 && is_f64<T>) return dmx_pre<W>(v, xep + ((b == 2 ? 11 : 0) + q) * 4);
-  else return dmx_shfl<W>(acc, f, p, sb, v, i12h);
-}
-
-// Dynamic shared memory of a float64 or double-word full-block stage (32 x ty
-// x tz points; 8-byte values): the first differences along z of 11 fields
-// over the block's rows and two halo rows on each side, then, for float64
-// (ends), per warp the 88 first differences along y and z past the ends of
-// its row (dmx_pre).
-static_assert(sizeof(ff) == sizeof(double), "double-word values take 8-byte slots");
-__host__ __device__ constexpr size_t rows_block_smem(int ty, int tz, bool ends) {
-  return ((size_t)11 * (ty + 4) * tz * 32 + (ends ? (size_t)ty * tz * 88 : 0)) * sizeof(double);
+// Dynamic shared memory of a double-word full-block stage (32 x ty x tz
+// points): the first differences along z of 11 fields over the block's rows
+// and two halo rows on each side.
+__host__ __device__ constexpr size_t rows_block_smem(int ty, int tz) {
+  return (size_t)11 * (ty + 4) * tz * 32 * sizeof(ff);
 }
 
 // the same helpers over the plain read-only global path (one field)
@@ -224,13 +188,13 @@ __host__ __device__ __forceinline__ double background(const Grid& g, int f) {
 // Right-hand side of all 24 fields at interior point (i, j, k) with linear
 // index id, reading the state register st (field stride g.fstride).  DEV: the
 // register holds X - X0 (mixed-path float buffers) instead of X.
-// XSEG = 32: the calling warp is one full x-row of 32 points (float64 only);
+// XSEG = 32: the calling warp is one full x-row of 32 points (double-word only);
 // the mixed second differences involving x then share first differences
 // across lanes (dmx_shfl).  XSEG = 0: every stencil evaluated by the thread.
 // YROWS > 0 (with XSEG = 32): the block is 32 x YROWS x ZS points, every
 // thread inside the grid, and D_y D_z takes the neighbouring rows' first
 // differences along z from shared memory (11 fields x (YROWS + 4) rows x ZS x
-// 32 doubles of dynamic shared memory; one barrier).
+// 32 values of dynamic shared memory; one barrier).
 template <typename T, typename S, bool DEV, typename A, int XSEG = 0, int YROWS = 0, int ZS = 1>
 __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i, int j, int k,
                                               T out[NF]) {
@@ -315,9 +279,8 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
 
   // ---- D_y D_z through shared memory (full blocks of full rows)
   [[maybe_unused]] T dyz[11];  // gt_ij (6), phi|W, alpha, beta^i (3)
-  [[maybe_unused]] const T* xep = nullptr;  // this warp's 88 end-of-row first differences (float64)
   if constexpr (YROWS > 0 && XSEG == 32 && !is_f32<T>) {
-    extern __shared__ double yz_smem[];  // 8-byte slots: float64 or double-word values
+    extern __shared__ float2 yz_smem[];
     T* yz = reinterpret_cast<T*>(yz_smem);
     constexpr int ROWS = YROWS + 4;
     const int ty = threadIdx.y, tz = threadIdx.z, lane = threadIdx.x;
@@ -336,28 +299,6 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
     if (ty >= YROWS - 2) {  // rows y0+YROWS, y0+YROWS+1 above it
 #pragma unroll
       for (int q = 0; q < 11; q++) at(q, ty + 4) = d1u<T>(acc, field_of(q), PF(field_of(q)) + 2 * sy, sz) * i12h;
-    }
-    if constexpr (is_f64<T>) {
-      // The x-mixed differences need, for each of the 11 fields and for y
-      // and z, the first differences at the four points past the ends of
-      // this warp's row: 88 values.  All 32 lanes form them, three rounds of
-      // one value each, into shared memory (item 4 p + e: pair p = field
-      // q + 11 (0 for y, 1 for z), point e = x_0 - 2, x_0 - 1, x_0 + 32,
-      // x_0 + 33), rather than the two lanes at each end of the row with the
-      // other 30 lanes of every such instruction idle.  Same arithmetic.
-      T* xe = yz + 11 * ROWS * ZS * 32 + (tz * YROWS + ty) * 88;
-#pragma unroll
-      for (int r = 0; r < 3; r++) {
-        const int idx = r * 32 + lane;
-        if (idx < 88) {
-          const int pr = idx >> 2, e = idx & 3;
-          const int q = pr < 11 ? pr : pr - 11;
-          const int f = field_of(q);
-          const int dx = (e < 2 ? e - 2 : 30 + e) - lane;  // x offset from this lane's point (unit stride)
-          xe[idx] = d1u<T>(acc, f, PF(f) + dx, pr < 11 ? sy : sz) * i12h;
-        }
-      }
-      xep = xe;
     }
     __syncthreads();
 #pragma unroll
@@ -408,13 +349,12 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
           const bool y = pb == 1;
 #pragma unroll
           for (int m = 0; m < 6; m++)
-            dd[m] = dmx_row<XSEG, YROWS>(acc, F_GT + m, PF(F_GT + m), sb, y ? dgt[1][m] : dgt[2][m], i12h, xep, pb, m);
-          vchi = dmx_row<XSEG, YROWS>(acc, F_CHI, PF(F_CHI), sb, y ? dchi[1] : dchi[2], i12h, xep, pb, 6) * i12h;
-          valp = dmx_row<XSEG, YROWS>(acc, F_ALP, PF(F_ALP), sb, y ? dalp[1] : dalp[2], i12h, xep, pb, 7);
+            dd[m] = dmx_shfl<XSEG>(acc, F_GT + m, PF(F_GT + m), sb, y ? dgt[1][m] : dgt[2][m], i12h);
+          vchi = dmx_shfl<XSEG>(acc, F_CHI, PF(F_CHI), sb, y ? dchi[1] : dchi[2], i12h) * i12h;
+          valp = dmx_shfl<XSEG>(acc, F_ALP, PF(F_ALP), sb, y ? dalp[1] : dalp[2], i12h);
 #pragma unroll
           for (int a = 0; a < 3; a++)
-            vb[a] = dmx_row<XSEG, YROWS>(acc, F_BETA + a, PF(F_BETA + a), sb, y ? db[1][a] : db[2][a], i12h, xep,
-                                         pb, 8 + a);
+            vb[a] = dmx_shfl<XSEG>(acc, F_BETA + a, PF(F_BETA + a), sb, y ? db[1][a] : db[2][a], i12h);
         }
       } else if (YROWS > 0 && pa == 1) {  // (1, 2) from the rows' differences along z
         sc = i12h;
@@ -473,9 +413,9 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
             sc = i12h;
 #pragma unroll
             for (int m = 0; m < 6; m++)
-              dd[m] = dmx_row<XSEG, YROWS>(acc, F_GT + m, PF(F_GT + m), SD(F_GT + m, pb), dgt[pb][m], i12h, xep, pb, m);
-            ddchi[pq] = dmx_row<XSEG, YROWS>(acc, F_CHI, PF(F_CHI), SD(F_CHI, pb), dchi[pb], i12h, xep, pb, 6) * i12h;
-            ddalp[pq] = dmx_row<XSEG, YROWS>(acc, F_ALP, PF(F_ALP), SD(F_ALP, pb), dalp[pb], i12h, xep, pb, 7);
+              dd[m] = dmx_shfl<XSEG>(acc, F_GT + m, PF(F_GT + m), SD(F_GT + m, pb), dgt[pb][m], i12h);
+            ddchi[pq] = dmx_shfl<XSEG>(acc, F_CHI, PF(F_CHI), SD(F_CHI, pb), dchi[pb], i12h) * i12h;
+            ddalp[pq] = dmx_shfl<XSEG>(acc, F_ALP, PF(F_ALP), SD(F_ALP, pb), dalp[pb], i12h);
           } else if constexpr (YROWS > 0) {  // (1, 2)
             sc = i12h;
 #pragma unroll
@@ -510,8 +450,7 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
             v = d2u<T>(acc, F_BETA + a, PF(F_BETA + a), SD(F_BETA + a, pa), beta[a]);
           } else if constexpr (XSEG > 0 && !is_f32<T>) {
             if (pa == 0)
-              v = dmx_row<XSEG, YROWS>(acc, F_BETA + a, PF(F_BETA + a), SD(F_BETA + a, pb), db[pb][a], i12h, xep,
-                                       pb, 8 + a);
+              v = dmx_shfl<XSEG>(acc, F_BETA + a, PF(F_BETA + a), SD(F_BETA + a, pb), db[pb][a], i12h);
             else if constexpr (YROWS > 0)
               v = dyz[8 + a];
             else

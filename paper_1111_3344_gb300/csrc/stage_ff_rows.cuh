@@ -2,10 +2,8 @@
 // x points (n0 a multiple of 32): the mixed second differences D1_x D1_y and
 // D1_x D1_z take the neighbouring points' first differences from the
 // neighbouring lanes and, when n1 and n2 fill the blocks, D1_y D1_z takes the
-// neighbouring rows' from shared memory -- the float64 path's arrangement
-// (k_stage_shfl.cu) in double-word arithmetic.  Instantiated for several
-// register caps in k_stage_ff_rows.cu and k_stage_ff_rows_occ.cu (compiled in
-// parallel).
+// neighbouring rows' from shared memory.  Instantiated for several register
+// caps in k_stage_ff_rows.cu and k_stage_ff_rows_occ.cu (compiled in parallel).
 #pragma once
 #include "stage_point.cuh"
 
@@ -39,7 +37,7 @@ cudaError_t launch_ff_rows(const Grid& g, const StageArgsFF& a, cudaStream_t s) 
   dim3 block(32, TY, TZ);
   dim3 grid(g.n0 / 32, (g.n1 + TY - 1) / TY, (g.n2 + TZ - 1) / TZ);
   if (g.n1 % TY == 0 && g.n2 % TZ == 0 && TY >= 2) {
-    constexpr int smem = (int)rows_block_smem(TY, TZ, false);
+    constexpr int smem = (int)rows_block_smem(TY, TZ);
     if constexpr (smem > 48 * 1024) {  // above the default limit: opt in once per device
       static std::atomic<unsigned> done{0};
       cudaError_t e = smem_optin(stage_ff_blocks_kernel<TY, TZ, MINB>, smem, done);

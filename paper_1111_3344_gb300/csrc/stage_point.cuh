@@ -3,6 +3,7 @@
 // (k_batch.cu) so that an evolution computes the same bits in either.
 #pragma once
 #include "bssn_internal.cuh"
+#include "rhs_fx.cuh"
 #include "rhs_point.cuh"
 
 namespace bssn {
@@ -12,39 +13,27 @@ __device__ __forceinline__ bool on_shell(const Grid& g, int ii, int jj, int kk) 
 }
 
 // Fused stage at interior point (ii, jj, kk) (interior indices), float64.
-// XSEG = 32: the calling warp is one full row of 32 x points (see dmx_shfl);
-// YROWS > 0: also every thread of the block is inside the grid (D_y D_z
-// through shared memory, see rhs_point_acc).
-template <int XSEG = 0, int YROWS = 0, int ZS = 1>
-__device__ __forceinline__ void stage_point_fp64(const Grid& g, const StageArgs& a, int ii, int jj,
-                                                 int kk) {
+__device__ __forceinline__ void stage_point_fp64(const Grid& g, const StageArgs& a, int ii, int jj, int kk) {
   const int i = ii + GH, j = jj + GH, k = kk + GH;
   const long long id = lin(g, i, j, k);
   double r[NF];
-  rhs_point<double, double, false, XSEG, YROWS, ZS>(g, a.src, id, i, j, k, r);
+  rhs_fx(g, a.src, id, i, j, k, r);
   const long long fs = g.fstride;
-  if (a.mode == MODE_RHS) {
-#pragma unroll
-    for (int f = 0; f < NF; f++) a.rhs[f * fs + id] = r[f];
-    return;
-  }
-  if (a.kshell && on_shell(g, ii, jj, kk)) {
-#pragma unroll
-    for (int f = 0; f < NF; f++) a.kshell[f * fs + id] = r[f];
-  }
-  if (a.mode == MODE_LAST) {
-#pragma unroll
-    for (int f = 0; f < NF; f++) {
-      const long long o = f * fs + id;
-      a.yn[o] = fma(a.b_dt, a.ksum[o] + r[f], a.yn[o]);
-    }
-    return;
-  }
-#pragma unroll
+  const bool anchor = a.mode != MODE_RHS && a.kshell && on_shell(g, ii, jj, kk);
+#pragma unroll 4
   for (int f = 0; f < NF; f++) {
     const long long o = f * fs + id;
-    a.out0[o] = fma(a.a_dt, r[f], a.src0[o]);
-    a.ksum[o] = a.mode == MODE_FIRST ? r[f] : fma(2.0, r[f], a.ksum[o]);
+    if (a.mode == MODE_RHS) {
+      a.rhs[o] = r[f];
+      continue;
+    }
+    if (anchor) a.kshell[o] = r[f];
+    if (a.mode == MODE_LAST) {
+      a.yn[o] = fma(a.b_dt, a.ksum[o] + r[f], a.yn[o]);
+    } else {
+      a.out0[o] = fma(a.a_dt, r[f], a.src0[o]);
+      a.ksum[o] = a.mode == MODE_FIRST ? r[f] : fma(2.0, r[f], a.ksum[o]);
+    }
   }
 }
 

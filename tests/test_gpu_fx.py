@@ -1,0 +1,88 @@
+"""The float64 right-hand side with integer-summed stencils (csrc/fx.cuh,
+csrc/rhs_fx.cuh) where it can go wrong: grids that whole tiles fill and grids
+that flat blocks cover, values of very different magnitude inside one stencil,
+signed zeros, and stencils outside the integer range (huge, tiny, not finite).
+
+Bar: 1e-12 max(S_f, M_pf) as everywhere (cases.rounding_aware_errors).  A
+stencil's alignment error is at most 192 2^-54 of its largest value (1.1e-14),
+its rounding 2^-53; the some 400 operations of a field's equation add 4e-14 M,
+so the bar holds with a factor of 15 to spare."""
+import numpy as np
+import pytest
+
+import cases as T
+import oracle as O
+from paper_1111_3344_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _rhs(c, st):
+    from paper_1111_3344_gb300.bssn import Evolution
+    evo = Evolution(T.gpu_params(c))
+    out = evo.register_to_numpy(evo.rhs(evo.numpy_to_register(st)))
+    evo.close()
+    return out
+
+
+def _case(n, seed, **kw):
+    c = dict(n=n, xmin=(-0.9, -1.1, -0.7), h=0.11, boundary="sommerfeld", **kw)
+    return c, inputs.random_state(seed, n, c["xmin"], c["h"], amp=0.05)
+
+
+SMALL = [7, 8, 10, 13, 14, 16, 19, 20, 22, 23]  # fields that may take any size
+
+
+@pytest.mark.parametrize("n", [(4, 4, 4), (32, 4, 5), (33, 5, 4), (24, 7, 9), (64, 8, 4), (31, 13, 6)])
+@pytest.mark.parametrize("conformal", ["W", "phi"])
+def test_wide_range_of_magnitudes(n, conformal):
+    """Neighbouring values from 1 down to 1e-25, of both signs, and exact zeros of both signs."""
+    c, st = _case(n, 3, conformal=conformal)
+    rng = np.random.default_rng(17)
+    if conformal == "phi":
+        st[0] = -0.5 * np.log(st[0])
+    for f in SMALL:
+        st[f] = 0.05 * rng.uniform(-1, 1, st[f].shape) * 10.0 ** rng.integers(-25, 1, st[f].shape)
+        st[f][rng.random(st[f].shape) < 0.1] = -0.0
+    cfg = T.oracle_cfg(c)
+    want, mag = O.rhs_mag(cfg, st)
+    got = _rhs(c, st)
+    assert T.rounding_aware_errors(got, want, mag).max() <= 1.0
+
+
+@pytest.mark.parametrize("scale", [1e-300, 1e-270, 5e-324, 1e300])
+def test_stencils_outside_the_integer_range(scale):
+    """B^i and Gt^x of such size: their own right-hand sides by the float64 sums."""
+    c, st = _case((12, 9, 8), 5)
+    st[21:24] *= scale
+    want, mag = O.rhs_mag(T.oracle_cfg(c), st)
+    got = _rhs(c, st)
+    assert T.rounding_aware_errors(got, want, mag).max() <= 1.0
+    if scale < 1.0:  # a stencil of subnormals is not flushed: B's advection is of its size
+        st2 = st.copy()
+        st2[21:24] = 0.0
+        keep = [f for f in range(24) if f not in (21, 22, 23)]
+        assert np.abs(got[keep] - _rhs(c, st2)[keep]).max() <= 10 * scale
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("f", [0, 3, 7, 9, 15, 17, 19, 22])
+def test_not_finite_values_spread_with_the_stencils(f, bad):
+    """One such value: every point whose dissipation stencil holds it is not
+    finite in that field, and nothing is where the oracle is finite.  (The
+    oracle also multiplies it by the zero coefficients of its stencils, so
+    its own set may be larger.)"""
+    c, st = _case((16, 9, 8), 7)
+    at = (7, 8, 9)
+    st[(f,) + at] = bad
+    with np.errstate(all="ignore"):
+        want = O.rhs(T.oracle_cfg(c), st)
+    got = _rhs(c, st)
+    inner = np.s_[:, 3:-3, 3:-3, 3:-3]
+    assert not (np.isfinite(want[inner]) & ~np.isfinite(got[inner])).any()
+    for d in range(3):
+        for m in range(-3, 4):
+            q = list(at)
+            q[d] += m
+            if all(3 <= q[e] < st.shape[1 + e] - 3 for e in range(3)):
+                assert not np.isfinite(got[(f,) + tuple(q)])
