@@ -313,6 +313,8 @@ bssn_status bssn_set_staging(bssn_ctx* ctx, void* d_mem, size_t bytes);
  * as well (eleven fields, 173 KB of shared memory, one block of 32x8 points
  * per SM); "split32x4x1/B" (B = 2, 3, 4) run the stencils as one
  * pass per field into a derivative register and the algebra as a second pass.
+ * A new context starts on the fastest measured configuration of its precision
+ * (mixed: "tma11_32x8x1/1").
  * Every configuration evaluates the same per-point arithmetic, so results agree
  * to rounding and each configuration is reproducible bit for bit. */
 int32_t bssn_tile_count(void);

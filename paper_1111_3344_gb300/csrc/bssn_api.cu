@@ -343,6 +343,11 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
     for (int v = 0; v < 2 && ok; v++)
       for (int q = 0; q < 3 && ok; q++) ok = make_stage_tensor_map(g, ctx->m32[q], &ctx->tmap[v][q], v) == cudaSuccess;
     ctx->tmap_ok = ok;
+    // the 11-field TMA stage: the same bits as the fused kernels and the
+    // fastest configuration at every size measured (one step, against the fused
+    // 32x8x1: 24^3 0.128 against 0.145 ms, 48^3 0.40 / 0.48, 100x70x50 1.07 /
+    // 1.41, 128^3 4.23 / 5.37, 256^3 31.2 / 43.2)
+    if (ok) ctx->tile = tile_config_count() + 2;
   }
   ctx->cstream = ctx->istream = nullptr;
   ctx->ev_out_ready = ctx->ev_out_done = ctx->ev_in_ready = ctx->ev_in_free = ctx->ev_out_free = nullptr;
