@@ -473,6 +473,30 @@ cudaError_t after_state(bssn_batch* b, Member& M) {
   return e;
 }
 
+// A member's state to or from the host layout: repacked on the device through
+// a stage buffer that holds nothing between steps, and copied as contiguous
+// blocks of whole fields.  (A pitched copy moves the rows one by one: 1.1 GB/s
+// from or to pageable memory.)
+cudaError_t copy_member(bssn_batch* b, const Member& M, double* host, bool to_device) {
+  const Grid& g = M.g;
+  const size_t per = (size_t)g.sx * g.sy * g.sz;
+  double* yn = (double*)mptr(b, M, M.L.yn);
+  double* area = (double*)mptr(b, M, b->precision == BSSN_FP64 ? M.L.s1 : (b->precision == BSSN_FF ? M.L.f2[1] : M.L.m32[1]));
+  const int chunk = b->precision == BSSN_MIXED ? NF / 2 : NF;  // 24 floats a point are 12 doubles
+  cudaError_t e = cudaSuccess;
+  for (int f0 = 0; f0 < NF && e == cudaSuccess; f0 += chunk) {
+    const size_t bytes = per * chunk * sizeof(double);
+    if (to_device) {
+      e = cudaMemcpyAsync(area, host + per * f0, bytes, cudaMemcpyHostToDevice, b->stream);
+      if (e == cudaSuccess) e = launch_repack(g, area, yn, f0, chunk, true, b->stream);
+    } else {
+      e = launch_repack(g, area, yn, f0, chunk, false, b->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(host + per * f0, area, bytes, cudaMemcpyDeviceToHost, b->stream);
+    }
+  }
+  return e;
+}
+
 bool member_ok(bssn_batch* b, int id) { return b && id >= 0 && id < b->maxm && b->m[id].used; }
 
 bool tile_usable(const bssn_batch* b, int c) {
@@ -691,10 +715,7 @@ bssn_status bssn_batch_set_state(bssn_batch* b, int32_t id, const double* host, 
   std::lock_guard<std::mutex> lk(b->mu);
   if (!member_ok(b, id)) return bfail(BSSN_ENOTFOUND, "no such member");
   Member& M = b->m[id];
-  const Grid& g = M.g;
-  double* yn = (double*)mptr(b, M, M.L.yn);
-  cudaError_t e = cudaMemcpy2DAsync(yn, (size_t)g.pitch * 8, host, (size_t)g.sx * 8, (size_t)g.sx * 8,
-                                    (size_t)NF * g.sz * g.sy, cudaMemcpyHostToDevice, b->stream);
+  cudaError_t e = copy_member(b, M, const_cast<double*>(host), true);
   if (e == cudaSuccess) e = after_state(b, M);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bcuda(e, "batch set_state");
@@ -709,10 +730,7 @@ bssn_status bssn_batch_get_state(bssn_batch* b, int32_t id, double* host, double
   std::lock_guard<std::mutex> lk(b->mu);
   if (!member_ok(b, id)) return bfail(BSSN_ENOTFOUND, "no such member");
   Member& M = b->m[id];
-  const Grid& g = M.g;
-  const double* yn = (const double*)mptr(b, M, M.L.yn);
-  cudaError_t e = cudaMemcpy2DAsync(host, (size_t)g.sx * 8, yn, (size_t)g.pitch * 8, (size_t)g.sx * 8,
-                                    (size_t)NF * g.sz * g.sy, cudaMemcpyDeviceToHost, b->stream);
+  cudaError_t e = copy_member(b, M, host, false);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bcuda(e, "batch get_state");
   if (bssn_status es = check_batch_err(b)) return es;
