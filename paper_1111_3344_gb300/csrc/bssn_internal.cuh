@@ -373,8 +373,8 @@ cudaError_t launch_adm_integrals(const Grid& g, const double* y, const Punct& pu
                                  double* partials, int nblocks, double* dout8, cudaStream_t s);
 // Weyl scalar Psi4 at interior points into out (2 fields of the register
 // layout: real, imaginary) (k_psi4.cu).
-cudaError_t launch_psi4(const Grid& g, const double* y, double* out, cudaStream_t s,
-                        double* adm_scratch = nullptr);
+// (adm_scratch: 12 * fstride doubles, as launch_constraints')
+cudaError_t launch_psi4(const Grid& g, const double* y, double* out, cudaStream_t s, double* adm_scratch);
 // One Euler step of the puncture positions dpunct (rows {m, x, y, z}) from the
 // shift of y (k_track.cu).
 cudaError_t launch_track(const Grid& g, const double* y, double* dpunct, int np, double dt, cudaStream_t s);

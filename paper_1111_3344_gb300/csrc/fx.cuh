@@ -76,4 +76,86 @@ __device__ __forceinline__ double fx_to(long long s, int E) {
   return __hiloint2double((int)hi, (int)(unsigned)r);
 }
 
+// 144 h^2 d_a d_b of the field at p (strides sa, sb; a != b) times 2^up, up 0 or -1.
+__device__ __forceinline__ double fx_mixed(const double* p, long long sa, long long sb, int up) {
+  double v[16];  // (m, q), m, q in -2, -1, 1, 2
+#pragma unroll
+  for (int m = 0; m < 4; m++)
+#pragma unroll
+    for (int q = 0; q < 4; q++) v[4 * m + q] = __ldg(p + (m < 2 ? m - 2 : m - 1) * sa + (q < 2 ? q - 2 : q - 1) * sb);
+  const unsigned top = fx_top(v);
+  if (fx_ok(top)) {
+    const int E = (int)(top >> 20);
+    long long l[4];
+#pragma unroll
+    for (int m = 0; m < 4; m++)
+      l[m] = 8 * (fx_from(v[4 * m + 2], E) - fx_from(v[4 * m + 1], E)) - (fx_from(v[4 * m + 3], E) - fx_from(v[4 * m], E));
+    // half of 8 (l1 - l-1) - (l2 - l-2): the whole may pass 2^63
+    return fx_to(4 * (l[2] - l[1]) - ((l[3] - l[0]) >> 1), E + 1 + up);
+  }
+  if (fx_zero(v)) return 0.0;
+  double l[4];
+#pragma unroll
+  for (int m = 0; m < 4; m++) l[m] = fma(8.0, v[4 * m + 2] - v[4 * m + 1], -(v[4 * m + 3] - v[4 * m]));
+  return (up ? 0.5 : 1.0) * fma(8.0, l[2] - l[1], -(l[3] - l[0]));
+}
+
+// The three mixed second derivatives (xy, xz, yz), one copy of the code.
+__device__ __forceinline__ void fx_mixed3(const double* p, long long sy, long long sz, int up, double dd[3]) {
+  double t[3];
+#pragma unroll 1
+  for (int m = 0; m < 3; m++) t[m] = fx_mixed(p, m < 2 ? 1 : sy, m == 0 ? sy : sz, up);
+  dd[0] = t[0];
+  dd[1] = t[1];
+  dd[2] = t[2];
+}
+
+// 12 h d f along stride s times 2^up.
+__device__ __forceinline__ double fx_d1(const double* p, long long s, int up) {
+  const double v[4] = {__ldg(p - 2 * s), __ldg(p - s), __ldg(p + s), __ldg(p + 2 * s)};
+  const unsigned top = fx_top(v);
+  if (fx_ok(top)) {
+    const int E = (int)(top >> 20);
+    return fx_to(8 * (fx_from(v[2], E) - fx_from(v[1], E)) - (fx_from(v[3], E) - fx_from(v[0], E)), E + up);
+  }
+  if (fx_zero(v)) return 0.0;
+  return (up ? 0.5 : 1.0) * fma(8.0, v[2] - v[1], -(v[3] - v[0]));
+}
+
+// 12 h d_d f and, SECOND, 144 h^2 d_d d_d f, d = x, y, z, times 2^up.
+template <bool SECOND>
+__device__ __forceinline__ void fx_axes(const double* p, long long sy, long long sz, int up, double d1[3],
+                                        double d2[3]) {
+  double v[13];
+  v[0] = SECOND ? __ldg(p) : 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    const long long s = d == 0 ? 1 : (d == 1 ? sy : sz);
+    v[1 + 4 * d] = __ldg(p - 2 * s);
+    v[2 + 4 * d] = __ldg(p - s);
+    v[3 + 4 * d] = __ldg(p + s);
+    v[4 + 4 * d] = __ldg(p + 2 * s);
+  }
+  const unsigned top = fx_top(v);
+  if (fx_ok(top)) {
+    const int E = (int)(top >> 20);
+    const long long f0 = SECOND ? fx_from(v[0], E) : 0;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+      const long long a = fx_from(v[1 + 4 * d], E), b = fx_from(v[2 + 4 * d], E), c = fx_from(v[3 + 4 * d], E),
+                      e = fx_from(v[4 + 4 * d], E);
+      d1[d] = fx_to(8 * (c - b) - (e - a), E + up);
+      if (SECOND) d2[d] = fx_to(3 * (16 * (c + b) - (e + a) - 30 * f0), E + 2 + up);
+    }
+    return;
+  }
+  const double sc = fx_zero(v) ? 0.0 : (up ? 0.5 : 1.0);
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    const double a = v[1 + 4 * d], b = v[2 + 4 * d], c = v[3 + 4 * d], e = v[4 + 4 * d];
+    d1[d] = sc * fma(8.0, c - b, -(e - a));
+    if (SECOND) d2[d] = 12.0 * sc * fma(-30.0, v[0], fma(16.0, c + b, -(e + a)));
+  }
+}
+
 }  // namespace bssn

@@ -12,12 +12,16 @@
 // sums h^3 sum over interior points, over all of them and over the points
 // farther than r_excise from every puncture.  Float64 in every precision mode.
 //
-// One thread per interior point; per block a warp-shuffle tree in each warp
-// and over the warp results (fixed order) into 8 partial sums, then one block
-// folds the partials the same way, so the result does not depend on
-// scheduling.
-#include "rhs_point.cuh"
-#include "ricci3.cuh"
+// Formulation: only the trace of Rt_ij is formed,
+//   Rt = -1/2 gt^ij gt^kl d_k d_l gt_ij + d_k Gt^k - 1/2 gt^ab d_k gt_ab d_l gt^lk
+//        + 2 Gt^k_li Gt^i_k^l + Gt_klj Gt^klj,
+// with integer-summed stencils (fx.cuh): about 450 float64 operations a point.
+//
+// One thread per interior point; per block a halving exchange in each warp and
+// a serial sum over the warps (fixed order) into 8 partial sums (slot-major),
+// then one block per result folds the partials, so the result does not depend
+// on scheduling.
+#include "curv3.cuh"
 
 namespace bssn {
 
@@ -26,126 +30,88 @@ namespace {
 constexpr int AB = 256;  // threads per block
 constexpr int NQ = 8;    // M, J_x, J_y, J_z; full then excised
 
-__device__ void adm_density(const Grid& g, const double* __restrict__ y, long long id, double x[3],
-                            double out[4]) {
-  const GlobalAcc<double> acc(g, y, id);
-  const double i12h = g.i12h, i12h2 = g.i12h2, i144h2 = g.i144h2;
-#define PF(f) acc.ptr(f)
-#define SD(f, d) acc.s((f), (d))
-  const double chi = __ldg(PF(F_CHI));
-  const double trK = __ldg(PF(F_TRK));
-  double gt[6], At[6];
+__device__ __forceinline__ void adm_density(const Grid& g, const double* __restrict__ y, long long id,
+                                            const double x[3], double out[4]) {
+  const long long fs = g.fstride, sy = g.pitch, sz = g.plane;
+  const double* p = y + id;
+  MetricD M;
+  metric_stencils(p + F_GT * fs, fs, sy, sz, M);
+  double dK[3];  // 12h d_d K
+  fx_axes<false>(p + F_TRK * fs, sy, sz, 0, dK, nullptr);
+  double dG = 0.0;  // 12h d_k Gt^k
+#pragma unroll 1
+  for (int a = 0; a < 3; a++) dG += fx_d1(p + (F_GAM + a) * fs, a == 0 ? 1 : (a == 1 ? sy : sz), 0);
+  const double chi = __ldg(p + F_CHI * fs);
+  const double trK = __ldg(p + F_TRK * fs);
+  double gt[6], At[6], gu[6], g2u[6], G1[3][6], G2[3][6];
 #pragma unroll
   for (int m = 0; m < 6; m++) {
-    gt[m] = __ldg(PF(F_GT + m));
-    At[m] = __ldg(PF(F_AT + m));
+    gt[m] = __ldg(p + (F_GT + m) * fs);
+    At[m] = __ldg(p + (F_AT + m) * fs);
   }
-  double gu[6];
+  inverse3(gt, gu);
+#pragma unroll
+  for (int m = 0; m < 6; m++) g2u[m] = (m == 0 || m == 3 || m == 5) ? gu[m] : 2.0 * gu[m];
+  christoffel_h(M.hg, gu, G1, G2);
+  // Rt, times 144 h^2
+  double Rtr = 0.0;
   {
-    const double c00 = gt[3] * gt[5] - gt[4] * gt[4];
-    const double c01 = gt[2] * gt[4] - gt[1] * gt[5];
-    const double c02 = gt[1] * gt[4] - gt[2] * gt[3];
-    const double idet = 1.0 / (gt[0] * c00 + gt[1] * c01 + gt[2] * c02);
-    gu[0] = c00 * idet;
-    gu[1] = c01 * idet;
-    gu[2] = c02 * idet;
-    gu[3] = (gt[0] * gt[5] - gt[2] * gt[2]) * idet;
-    gu[4] = (gt[1] * gt[2] - gt[0] * gt[4]) * idet;
-    gu[5] = (gt[0] * gt[3] - gt[1] * gt[1]) * idet;
-  }
-  double dgt[3][6], dG[3][3], dK[3];
+    double s = 0.0;  // 72 h^2 gt^ij gt^kl d_k d_l gt_ij
 #pragma unroll
-  for (int d = 0; d < 3; d++) {
+    for (int m = 0; m < 6; m++) {
+      double t = 0.0;
 #pragma unroll
-    for (int m = 0; m < 6; m++) dgt[d][m] = d1u<double>(acc, F_GT + m, PF(F_GT + m), SD(F_GT + m, d)) * i12h;
-#pragma unroll
-    for (int a = 0; a < 3; a++) dG[d][a] = d1u<double>(acc, F_GAM + a, PF(F_GAM + a), SD(F_GAM + a, d)) * i12h;
-    dK[d] = d1u<double>(acc, F_TRK, PF(F_TRK), SD(F_TRK, d)) * i12h;
-  }
-  // -1/2 gt^{kl} d_k d_l gt_ij, accumulated pair by pair
-  double Rdd[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll
-  for (int pa = 0; pa < 3; pa++)
-#pragma unroll
-    for (int pb = pa; pb < 3; pb++) {
-      const int pq = sym(pa, pb);
-      const double w = (pa == pb) ? -0.5 * gu[pq] : -gu[pq];
-#pragma unroll
-      for (int m = 0; m < 6; m++) {
-        const double dd = (pa == pb)
-                              ? d2u<double>(acc, F_GT + m, PF(F_GT + m), SD(F_GT + m, pa), gt[m]) * i12h2
-                              : dmu<double>(acc, F_GT + m, PF(F_GT + m), SD(F_GT + m, pa), SD(F_GT + m, pb)) * i144h2;
-        Rdd[m] = fma(w, dd, Rdd[m]);
-      }
+      for (int q = 0; q < 6; q++) t = fma(g2u[q], M.hdd[m][q], t);
+      s = fma(g2u[m], t, s);
     }
-#undef PF
-#undef SD
-  // Christoffel symbols of gt (ricci3.cuh: the terms that cancel left out)
-  double G1[3][6], G2[3][6];
-  christoffel3(gu, dgt, G1, G2);
-  double dgu[3];
-  {
+    Rtr = fma(g.h12, dG, -s);
+    // V[k] = 6h gt^{kb} gt^{la} d_l gt_ab = -6h d_l gt^{lk}; tr[k] = 6h gt^ab d_k gt_ab
     double Tb[3];
 #pragma unroll
     for (int b = 0; b < 3; b++) {
-      double s = 0.0;
+      double t = 0.0;
 #pragma unroll
       for (int l = 0; l < 3; l++)
 #pragma unroll
-        for (int a = 0; a < 3; a++) s = fma(gu[sym(l, a)], dgt[l][sym(a, b)], s);
-      Tb[b] = s;
+        for (int a = 0; a < 3; a++) t = fma(gu[sym(l, a)], M.hg[sym(a, b)][l], t);
+      Tb[b] = t;
     }
+    double q3 = 0.0;
 #pragma unroll
-    for (int kk = 0; kk < 3; kk++)
-      dgu[kk] = -(gu[sym(kk, 0)] * Tb[0] + gu[sym(kk, 1)] * Tb[1] + gu[sym(kk, 2)] * Tb[2]);
-  }
-  // Rt_ij and its trace gt^ij Rt_ij
-  double Rtr = 0.0;
-  {
-    double G1u[3][3][3];
+    for (int k = 0; k < 3; k++) {
+      const double V = gu[sym(k, 0)] * Tb[0] + gu[sym(k, 1)] * Tb[1] + gu[sym(k, 2)] * Tb[2];
+      double t = 0.0;
 #pragma unroll
-    for (int jj = 0; jj < 3; jj++)
+      for (int m = 0; m < 6; m++) t = fma(g2u[m], M.hg[m][k], t);
+      q3 = fma(t, V, q3);
+    }
+    Rtr = fma(2.0, q3, Rtr);
+    // H[i][k][l] = Gt^i_k^l; 2 Gt^k_li H[i][k][l] + Gt_k,lj Gt^k,lj
+    double H[3][3][3];
 #pragma unroll
-      for (int kk = 0; kk < 3; kk++)
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int k = 0; k < 3; k++)
 #pragma unroll
         for (int l = 0; l < 3; l++)
-          G1u[jj][kk][l] = gu[sym(l, 0)] * G1[jj][sym(kk, 0)] + gu[sym(l, 1)] * G1[jj][sym(kk, 1)] +
-                           gu[sym(l, 2)] * G1[jj][sym(kk, 2)];
+          H[i][k][l] = gu[sym(l, 0)] * G2[i][sym(k, 0)] + gu[sym(l, 1)] * G2[i][sym(k, 1)] + gu[sym(l, 2)] * G2[i][sym(k, 2)];
+    double q1 = 0.0, q2 = 0.0;
 #pragma unroll
-    for (int a = 0; a < 3; a++)
+    for (int k = 0; k < 3; k++) {
 #pragma unroll
-      for (int b = a; b < 3; b++) {
-        const int ab = sym(a, b);
-        double s = Rdd[ab], t = 0.0;
+      for (int l = 0; l < 3; l++)
 #pragma unroll
-        for (int kk = 0; kk < 3; kk++) {
-          t = fma(gt[sym(kk, a)], dG[b][kk], t);
-          t = fma(gt[sym(kk, b)], dG[a][kk], t);
-          t = fma(-dgt[kk][ab], dgu[kk], t);  // Gt_akb + Gt_bka = d_k gt_ab
+        for (int i = 0; i < 3; i++) q1 = fma(G2[k][sym(l, i)], H[i][k][l], q1);
+#pragma unroll
+      for (int l = 0; l < 3; l++)
+#pragma unroll
+        for (int j = l; j < 3; j++) {
+          const double W = gu[sym(l, 0)] * H[k][0][j] + gu[sym(l, 1)] * H[k][1][j] + gu[sym(l, 2)] * H[k][2][j];
+          if (l == j) Rtr = fma(G1[k][sym(l, j)], W, Rtr);
+          else q2 = fma(G1[k][sym(l, j)], W, q2);
         }
-        s = fma(0.5, t, s);
-        if (a == b) {  // the first two quadratic terms coincide
-          double q = 0.0;
-#pragma unroll
-          for (int kk = 0; kk < 3; kk++)
-#pragma unroll
-            for (int l = 0; l < 3; l++) {
-              q = fma(G2[kk][sym(l, a)], G1u[a][kk][l], q);
-              s = fma(G2[kk][sym(a, l)], G1u[kk][a][l], s);
-            }
-          s = fma(2.0, q, s);
-        } else {
-#pragma unroll
-          for (int kk = 0; kk < 3; kk++)
-#pragma unroll
-            for (int l = 0; l < 3; l++) {
-              s = fma(G2[kk][sym(l, a)], G1u[b][kk][l], s);
-              s = fma(G2[kk][sym(l, b)], G1u[a][kk][l], s);
-              s = fma(G2[kk][sym(a, l)], G1u[kk][b][l], s);
-            }
-        }
-        Rtr = fma(a == b ? gu[ab] : 2.0 * gu[ab], s, Rtr);
-      }
+    }
+    Rtr = fma(2.0, q1 + q2, Rtr) * g.i144h2;
   }
   // e^{phi} and its powers
   double ephi;
@@ -170,11 +136,12 @@ __device__ void adm_density(const Grid& g, const double* __restrict__ y, long lo
 #pragma unroll
     for (int b = a; b < 3; b++)
       Au[sym(a, b)] = Am[a][0] * gu[sym(0, b)] + Am[a][1] * gu[sym(1, b)] + Am[a][2] * gu[sym(2, b)];
-  double AA = 0.0;
+  double Au2[6], AA = 0.0;
 #pragma unroll
-  for (int a = 0; a < 3; a++)
-#pragma unroll
-    for (int b = 0; b < 3; b++) AA = fma(At[sym(a, b)], Au[sym(a, b)], AA);
+  for (int m = 0; m < 6; m++) {
+    Au2[m] = (m == 0 || m == 3 || m == 5) ? Au[m] : 2.0 * Au[m];
+    AA = fma(At[m], Au2[m], AA);
+  }
   // matter: E and S_k (zero in vacuum)
   double Em = 0.0, Sk[3] = {0.0, 0.0, 0.0};
   if (g.tmunu) {
@@ -185,103 +152,74 @@ __device__ void adm_density(const Grid& g, const double* __restrict__ y, long lo
     matter_at<double>(g, id, alp, beta, Em, Sk, Sij);
   }
   out[0] = (e5 * (16.0 * M_PI * Em + AA - (2.0 / 3.0) * trK * trK) - ephi * Rtr) * (1.0 / (16.0 * M_PI));
-  // At_ln d_k gt^{ln} = -At^{ab} d_k gt_ab
-  double AdG[3];
+  // w[k] = (2/3) d_k K - (1/2) At_ln d_k gt^{ln} + 8 pi S_k, At_ln d_k gt^{ln} = -At^{ab} d_k gt_ab
+  double w[3];
 #pragma unroll
-  for (int kk = 0; kk < 3; kk++) {
-    double s = 0.0;
+  for (int k = 0; k < 3; k++) {
+    double t = (2.0 / 3.0) * dK[k];
 #pragma unroll
-    for (int a = 0; a < 3; a++)
-#pragma unroll
-      for (int b = 0; b < 3; b++) s = fma(Au[sym(a, b)], dgt[kk][sym(a, b)], s);
-    AdG[kk] = -s;
+    for (int m = 0; m < 6; m++) t = fma(Au2[m], M.hg[m][k], t);
+    w[k] = fma(g.i12h, t, (8.0 * M_PI) * Sk[k]);
   }
-  double v[3][3];  // v[j][k] = At^j_k + x^j ((2/3) d_k K - (1/2) At_ln d_k gt^{ln})
-#pragma unroll
-  for (int jj = 0; jj < 3; jj++)
-#pragma unroll
-    for (int kk = 0; kk < 3; kk++)
-      v[jj][kk] = fma(x[jj], (2.0 / 3.0) * dK[kk] - 0.5 * AdG[kk] + 8.0 * M_PI * Sk[kk], Am[jj][kk]);
   const double c = e6 * (1.0 / (8.0 * M_PI));
-  out[1] = c * (v[1][2] - v[2][1]);
-  out[2] = c * (v[2][0] - v[0][2]);
-  out[3] = c * (v[0][1] - v[1][0]);
-}
-
-// Fixed-order block sum of NQ values per thread: shuffle tree in each warp,
-// then over the warp results in warp 0; thread 0 returns the sums in v.
-__device__ __forceinline__ void block_sum(double v[NQ]) {
-  __shared__ double wsum[NQ][AB / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-    for (int q = 0; q < NQ; q++) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < NQ; q++) wsum[q][warp] = v[q];
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int q = 0; q < NQ; q++) v[q] = lane < AB / 32 ? wsum[q][lane] : 0.0;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-      for (int q = 0; q < NQ; q++) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
+  for (int i = 0; i < 3; i++) {  // eps_ijk (At^j_k + x^j w_k)
+    const int j = (i + 1) % 3, k = (i + 2) % 3;
+    out[1 + i] = c * ((Am[j][k] - Am[k][j]) + (x[j] * w[k] - x[k] * w[j]));
   }
 }
 
-__global__ void __launch_bounds__(AB) adm_integrals_kernel(Grid g, const double* __restrict__ y, Punct pu,
-                                                           double* __restrict__ dens,
-                                                           double* __restrict__ partials) {
-  const long long npts = (long long)g.n0 * g.n1 * g.n2;
-  const long long tid = (long long)blockIdx.x * AB + threadIdx.x;
+__global__ void __launch_bounds__(AB, 2) adm_integrals_kernel(Grid g, const double* __restrict__ y, Punct pu,
+                                                              double* __restrict__ dens,
+                                                              double* __restrict__ partials) {
+  __shared__ double wsum[NQ][AB / 32];
+  const unsigned npts = (unsigned)g.n0 * g.n1 * g.n2;
+  const unsigned t = blockIdx.x * AB + threadIdx.x;
   double v[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; q++) v[q] = 0.0;
-  if (tid < npts) {
-    const int ii = (int)(tid % g.n0);
-    const int jj = (int)((tid / g.n0) % g.n1);
-    const int kk = (int)(tid / ((long long)g.n0 * g.n1));
-    const int i = ii + GH, j = jj + GH, k = kk + GH;
-    const long long id = lin(g, i, j, k);
-    double x[3] = {cell_coord(g.xmin0, ii, g.h), cell_coord(g.xmin1, jj, g.h), cell_coord(g.xmin2, kk, g.h)};
+  if (t < npts) {
+    const unsigned row = t / (unsigned)g.n0;
+    const int ii = (int)(t - row * g.n0), kk = (int)(row / (unsigned)g.n1), jj = (int)(row - (unsigned)kk * g.n1);
+    const long long id = lin(g, ii + GH, jj + GH, kk + GH);
+    const double x[3] = {cell_coord(g.xmin0, ii, g.h), cell_coord(g.xmin1, jj, g.h), cell_coord(g.xmin2, kk, g.h)};
     double o[4];
     adm_density(g, y, id, x, o);
     if (dens) {
 #pragma unroll
       for (int q = 0; q < 4; q++) dens[q * g.fstride + id] = o[q];
     }
-    bool outside = true;
-    for (int a = 0; a < pu.n; a++) {
-      const double dx = x[0] - pu.p[a][1], dy = x[1] - pu.p[a][2], dz = x[2] - pu.p[a][3];
-      if (sqrt(dx * dx + dy * dy + dz * dz) <= pu.r_ex) outside = false;
-    }
+    const bool outside = outside_punctures(pu, x[0], x[1], x[2]);
 #pragma unroll
     for (int q = 0; q < 4; q++) {
       v[q] = o[q];
       v[4 + q] = outside ? o[q] : 0.0;
     }
   }
-  block_sum(v);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int q = 0; q < NQ; q++) partials[(long long)blockIdx.x * NQ + q] = v[q];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double s = warp_sums<NQ>(v);
+  if ((lane & 3) == 0) wsum[lane >> 2][warp] = s;
+  __syncthreads();
+  if (threadIdx.x < NQ) {
+    double r = 0.0;
+    for (int w = 0; w < AB / 32; w++) r += wsum[threadIdx.x][w];
+    partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = r;
+  }
 }
 
+// block q: result q, threads striding over its partials, then a fixed tree
 __global__ void __launch_bounds__(AB) adm_integrals_finalize(const double* __restrict__ partials, int nblocks,
                                                              double vol, double* __restrict__ out) {
-  double v[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; q++) v[q] = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += AB) {
-#pragma unroll
-    for (int q = 0; q < NQ; q++) v[q] += partials[(long long)b * NQ + q];
+  __shared__ double a[AB];
+  const double* p = partials + (size_t)blockIdx.x * nblocks;
+  double v = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += AB) v += p[b];
+  a[threadIdx.x] = v;
+  for (int w = AB / 2; w > 0; w >>= 1) {
+    __syncthreads();
+    if (threadIdx.x < w) a[threadIdx.x] += a[threadIdx.x + w];
   }
-  block_sum(v);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int q = 0; q < NQ; q++) out[q] = v[q] * vol;
+  if (threadIdx.x == 0) out[blockIdx.x] = a[0] * vol;
 }
 
 }  // namespace
@@ -296,7 +234,7 @@ cudaError_t launch_adm_integrals(const Grid& g, const double* y, const Punct& pu
   adm_integrals_kernel<<<nblocks, AB, 0, s>>>(g, y, pu, dens, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  adm_integrals_finalize<<<1, AB, 0, s>>>(partials, nblocks, g.h * g.h * g.h, dout8);
+  adm_integrals_finalize<<<NQ, AB, 0, s>>>(partials, nblocks, g.h * g.h * g.h, dout8);
   return cudaGetLastError();
 }
 

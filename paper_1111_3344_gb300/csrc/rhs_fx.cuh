@@ -33,31 +33,6 @@
 
 namespace bssn {
 
-// Half of D1_a D1_b of the field at p (strides sa, sb), in units of 72 h^2:
-// returned as 144 h^2 d_a d_b f times 2^up.
-__device__ __forceinline__ double fx_mixed(const double* p, long long sa, long long sb, int up) {
-  double v[16];  // (m, q), m, q in -2, -1, 1, 2
-#pragma unroll
-  for (int m = 0; m < 4; m++)
-#pragma unroll
-    for (int q = 0; q < 4; q++) v[4 * m + q] = __ldg(p + (m < 2 ? m - 2 : m - 1) * sa + (q < 2 ? q - 2 : q - 1) * sb);
-  const unsigned top = fx_top(v);
-  if (fx_ok(top)) {
-    const int E = (int)(top >> 20);
-    long long l[4];
-#pragma unroll
-    for (int m = 0; m < 4; m++)
-      l[m] = 8 * (fx_from(v[4 * m + 2], E) - fx_from(v[4 * m + 1], E)) - (fx_from(v[4 * m + 3], E) - fx_from(v[4 * m], E));
-    // half of 8 (l1 - l-1) - (l2 - l-2): the whole may pass 2^63
-    return fx_to(4 * (l[2] - l[1]) - ((l[3] - l[0]) >> 1), E + 1 + up);
-  }
-  if (fx_zero(v)) return 0.0;
-  double l[4];
-#pragma unroll
-  for (int m = 0; m < 4; m++) l[m] = fma(8.0, v[4 * m + 2] - v[4 * m + 1], -(v[4 * m + 3] - v[4 * m]));
-  return (up ? 0.5 : 1.0) * fma(8.0, l[2] - l[1], -(l[3] - l[0]));
-}
-
 // Advection and dissipation weights of a point: bh = |beta| / (24h), neg the
 // signs of beta as masks, kap = eps / (64h).
 struct FxAdv {
@@ -121,16 +96,6 @@ __device__ __forceinline__ double fx_axes(const double* p, long long sy, long lo
     r = fma(w.kap, k, r);
   }
   return r;
-}
-
-// The three mixed second derivatives (xy, xz, yz), one copy of the code.
-__device__ __forceinline__ void fx_mixed3(const double* p, long long sy, long long sz, int up, double dd[3]) {
-  double t[3];
-#pragma unroll 1
-  for (int m = 0; m < 3; m++) t[m] = fx_mixed(p, m < 2 ? 1 : sy, m == 0 ? sy : sz, up);
-  dd[0] = t[0];
-  dd[1] = t[1];
-  dd[2] = t[2];
 }
 
 // The stencils' results at a point, in local memory (indexed by the field loop).

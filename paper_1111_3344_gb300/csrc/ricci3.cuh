@@ -1,8 +1,7 @@
 // Christoffel symbols and Ricci tensor of a 3-metric g_ij from its first and
-// second differences, float64, for the analysis kernels (constraints and Psi4:
-// Ricci tensor of gamma_ij; ADM integrals: Christoffel symbols of gt_ij;
-// arXiv:1111.3344, Sec. "Other analysis modules", Sec. "Masses and Momenta",
-// Sec. "Gravitational Waves").
+// second differences, float64, for the constraint norms of a caller's state,
+// whose ADM fields are formed at every stencil point (arXiv:1111.3344, Sec.
+// "Other analysis modules"); the other analysis kernels use curv3.cuh.
 //
 //   Gamma_kij   = (d_i g_kj + d_j g_ki - d_k g_ij) / 2,   Gamma^k_ij = g^ks Gamma_sij
 //   R_ij = 1/2 g^kl (d_k d_j g_il + d_i d_l g_kj - d_k d_l g_ij - d_i d_j g_kl)

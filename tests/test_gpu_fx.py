@@ -86,3 +86,22 @@ def test_not_finite_values_spread_with_the_stencils(f, bad):
             q[d] += m
             if all(3 <= q[e] < st.shape[1 + e] - 3 for e in range(3)):
                 assert not np.isfinite(got[(f,) + tuple(q)])
+
+
+@pytest.mark.parametrize("n", [(4, 4, 4), (5, 7, 33), (32, 8, 8), (17, 15, 1 + 8)])
+@pytest.mark.parametrize("r_excise", [0.3, 50.0])
+def test_norms_at_block_edges(n, r_excise):
+    """Blocks of 256 points with a ragged end, an excised set that is empty
+    (r_excise past the grid) or not; the bar of the norms' parity tests."""
+    from paper_1111_3344_gb300.bssn import Evolution
+    c, st = _case(n, 11, r_excise=r_excise, punctures=[(1.0, 0.02, -0.01, 0.03)])
+    evo = Evolution(T.gpu_params(c))
+    evo.set_punctures(c["punctures"])
+    evo.set_state(st)
+    want = O.constraints(T.oracle_cfg(c), st)[0]
+    assert np.allclose(evo.constraints(), want, rtol=1e-12, atol=0)
+    st[7, 4, 5, 4] = np.nan  # a NaN shows in the sums and the maxima of both sets that hold it
+    evo.set_state(st)
+    got = evo.constraints()
+    assert np.isnan(got[:8]).any() and (r_excise > 10 or np.isnan(got[8:]).any())
+    evo.close()
