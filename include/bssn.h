@@ -314,7 +314,8 @@ bssn_status bssn_set_staging(bssn_ctx* ctx, void* d_mem, size_t bytes);
  * per SM); "split32x4x1/B" (B = 2, 3, 4) run the stencils as one
  * pass per field into a derivative register and the algebra as a second pass.
  * A new context starts on the fastest measured configuration of its precision
- * (mixed: "tma11_32x8x1/1").
+ * (mixed: "tma11_32x8x1/1"; float64: "32x4x1/1", whose float64 form stages boxes of
+ * 8x4x4 points in shared memory by tensor loads where these fit the grid).
  * Every configuration evaluates the same per-point arithmetic, so results agree
  * to rounding and each configuration is reproducible bit for bit. */
 int32_t bssn_tile_count(void);
@@ -489,7 +490,8 @@ bssn_status bssn_profile(bssn_ctx* ctx, int32_t enable, double out[4]);
  * the next synchronising call (bssn_get_state, bssn_wait_state,
  * bssn_constraints) returns BSSN_ETIMEOUT and clears the error word; the
  * context stays usable.  polls in [0, 2^20]; 0 (the default) restores normal
- * operation.  Affects only the TMA-staged configurations of mixed contexts. */
+ * operation.  Affects only the TMA-staged configurations of mixed contexts
+ * (the float64 tiles' waits have the same limit and report the same way). */
 bssn_status bssn_test_stall_tma(bssn_ctx* ctx, int32_t polls);
 
 /* Measured arithmetic peak of the current GPU (no counterpart in the paper:

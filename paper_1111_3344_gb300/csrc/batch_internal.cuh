@@ -18,8 +18,9 @@ struct MemberDev {
   StageArgsMixed amx[4];
   StageArgsFF aff[4];  // double-word batches
   int tiles[3];  // stage tiles per axis for the batch's current tile shape
-  // mixed: tensor map of each stage's input float buffer (TMA-staged batch
-  // kernel); 64-byte aligned, as the tensor loads require
+  // tensor map of each stage's input (mixed: the float buffer, TMA-staged batch
+  // kernel; float64: the tile form of the per-member launches); 64-byte
+  // aligned, as the tensor loads require
   CUtensorMap tmap[4];
 };
 

@@ -183,6 +183,8 @@ struct bssn_ctx {
   int tile;  // stage-kernel tile configuration (see bssn_autotune)
   CUtensorMap tmap[2][3];  // mixed: tensor maps of the float stage buffers, per TMA box (tma_map)
   bool tmap_ok;
+  CUtensorMap fmap[3];  // float64: tensor maps of y_n, s1, s2 (tile form of the stage)
+  bool fmap_ok;
   int* err;             // device error word (bounded waits that gave up)
   int stall_polls;      // test hook of the TMA-staged kernels (bssn_test_stall_tma)
   double* part;
@@ -338,6 +340,9 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
   ctx->tracking = false;
   ctx->trk_stale = false;
   ctx->tmap_ok = false;
+  ctx->fmap_ok = p->precision == BSSN_FP64 && make_fx_tensor_map(g, ctx->yn, &ctx->fmap[0]) == cudaSuccess &&
+                 make_fx_tensor_map(g, ctx->s1, &ctx->fmap[1]) == cudaSuccess &&
+                 make_fx_tensor_map(g, ctx->s2, &ctx->fmap[2]) == cudaSuccess;
   if (p->precision == BSSN_MIXED) {
     bool ok = true;
     for (int v = 0; v < 2 && ok; v++)
@@ -508,6 +513,12 @@ bssn_status bssn_get_punctures(bssn_ctx* ctx, double* out, int32_t* npunct) {
   return BSSN_OK;
 }
 
+// tensor map of one of a float64 context's own registers (null: none)
+static const CUtensorMap* fx_map(const bssn_ctx* ctx, const double* src) {
+  if (!ctx->fmap_ok) return nullptr;
+  return src == ctx->yn ? &ctx->fmap[0] : (src == ctx->s1 ? &ctx->fmap[1] : (src == ctx->s2 ? &ctx->fmap[2] : nullptr));
+}
+
 bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs) {
   if (!ctx || !d_rhs) return fail(BSSN_EINVAL, "NULL argument");
   if (cudaError_t ed = drain_out(ctx)) return cuda_fail(ed, "wait for the state read-back");
@@ -523,7 +534,11 @@ bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs) {
     a.src = src;
     a.rhs = out;
     a.mode = MODE_RHS;
-    e = launch_stage_fp64(ctx->g, a, ctx->stream, ctx->tile);
+    // a caller's register is described here, where its address allows it
+    CUtensorMap made;
+    const CUtensorMap* map = fx_map(ctx, src);
+    if (!map && (uintptr_t)src % 16 == 0 && make_fx_tensor_map(ctx->g, src, &made) == cudaSuccess) map = &made;
+    e = launch_stage_fp64(ctx->g, a, ctx->stream, ctx->tile, map, ctx->err);
     if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs interior");
     if (!ctx->g.periodic) {
       e = launch_sommerfeld(ctx->g, a, nullptr, ctx->stream);
@@ -588,7 +603,7 @@ static bssn_status run_stage(bssn_ctx* ctx, const double* src, int mode, double*
   a.mode = mode;
   cudaError_t e;
   if (ctx->prof && (e = prof_mark(ctx, ctx->ev_stage)) != cudaSuccess) return cuda_fail(e, "profile");
-  e = launch_stage_fp64(ctx->g, a, ctx->stream, ctx->tile);
+  e = launch_stage_fp64(ctx->g, a, ctx->stream, ctx->tile, fx_map(ctx, src), ctx->err);
   if (e != cudaSuccess) return cuda_fail(e, "stage");
   if (ctx->prof && (e = prof_mark(ctx, ctx->ev_stage)) != cudaSuccess) return cuda_fail(e, "profile");
   if (ctx->prof && (e = prof_mark(ctx, ctx->ev_bc)) != cudaSuccess) return cuda_fail(e, "profile");
@@ -1070,7 +1085,7 @@ bssn_status bssn_autotune(bssn_ctx* ctx, int32_t reps, int32_t* best, double* ms
         a.src = second ? ctx->s1 : ctx->yn; a.src0 = ctx->yn; a.yn = ctx->yn;
         a.out0 = second ? ctx->s2 : ctx->s1; a.ksum = ctx->ks;
         a.a_dt = 0.5 * ctx->p.dt; a.mode = second ? MODE_MID : MODE_FIRST;
-        return launch_stage_fp64(ctx->g, a, ctx->stream, c);
+        return launch_stage_fp64(ctx->g, a, ctx->stream, c, fx_map(ctx, a.src), ctx->err);
       }
       const int q = second ? 1 : 0, o = second ? 2 : 1;
       StageArgsMixed a{};

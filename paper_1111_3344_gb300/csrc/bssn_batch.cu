@@ -128,6 +128,7 @@ MemberLayout member_layout(const bssn_params* p, const Grid& g) {
 
 struct Member {
   bool used = false, active = false;
+  bool fmap_ok = false;  // float64: the tensor maps of its stage inputs are made
   bool held = false;  // resident but left out of the steps (bssn_batch_hold)
   bssn_params p{};
   Grid g{};
@@ -195,6 +196,7 @@ void fill_member_dev(bssn_batch* b, int id) {
     double* s2 = (double*)mptr(b, M, M.L.s2);
     double* src[4] = {yn, s1, s2, s1};
     double* out[4] = {s1, s2, s1, nullptr};
+    M.fmap_ok = true;
     for (int s = 0; s < 4; s++) {
       StageArgs& a = D.a64[s];
       a.src = src[s];
@@ -206,6 +208,7 @@ void fill_member_dev(bssn_batch* b, int id) {
       a.a_dt = a_dt[s];
       a.b_dt = b_dt[s];
       a.mode = mode[s];
+      if (make_fx_tensor_map(M.g, a.src, &D.tmap[s]) != cudaSuccess) M.fmap_ok = false;
     }
   } else if (b->precision == BSSN_FF) {
     const int src[4] = {0, 1, 2, 1}, out[4] = {1, 2, 1, 0};
@@ -307,13 +310,6 @@ cudaError_t rebuild_work(bssn_batch* b) {
 
 // ---- per-member configuration
 // the single-grid configurations it launches (looked up by name once)
-int single_fp64_cfg() {
-  static int c = -1;
-  if (c < 0)
-    for (int q = 0; q < tile_config_count(); q++)
-      if (!strcmp(tile_config_name(q), "32x4x1/1")) c = q;
-  return c < 0 ? 0 : c;
-}
 int single_ff_cfg() {
   static int c = -1;
   if (c < 0)
@@ -356,7 +352,8 @@ cudaError_t member_stage(bssn_batch* b, int id, int stage, cudaStream_t s) {
   const MemberDev& D = b->h_mem[id];
   if (b->precision == BSSN_MIXED) return launch_stage_mixed_tma(D.g, D.amx[stage], D.tmap[stage], b->d_err, s, 2);
   if (b->precision == BSSN_FF) return launch_stage_ff(D.g, D.aff[stage], s, single_ff_cfg());
-  return launch_stage_fp64(D.g, D.a64[stage], s, single_fp64_cfg());
+  return launch_stage_fp64(D.g, D.a64[stage], s, fp64_default_tile(), b->m[id].fmap_ok ? &D.tmap[stage] : nullptr,
+                           b->d_err);
 }
 
 // member id's boundary after a stage, with the single-grid boundary kernels

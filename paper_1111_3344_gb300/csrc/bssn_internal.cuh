@@ -302,7 +302,14 @@ struct Punct {
 };
 
 // Launch wrappers (defined in the .cu files); all return cudaError_t of the launch.
-cudaError_t launch_stage_fp64(const Grid& g, const StageArgs& a, cudaStream_t s, int cfg = 0);
+// map (may be null): tensor map of a.src made by make_fx_tensor_map, with which
+// fp64_default_tile() runs the tile form (k_stage_fx.cu) where that is the faster
+// one; err: device error word (a bounded wait gave up)
+cudaError_t launch_stage_fp64(const Grid& g, const StageArgs& a, cudaStream_t s, int cfg = 0,
+                              const CUtensorMap* map = nullptr, int* err = nullptr);
+bool fx_tile_fits(const Grid& g);
+cudaError_t make_fx_tensor_map(const Grid& g, const double* base, CUtensorMap* out);
+cudaError_t launch_stage_fx(const Grid& g, const StageArgs& a, const CUtensorMap& map, int* err, cudaStream_t s);
 cudaError_t launch_stage_mixed(const Grid& g, const StageArgsMixed& a, cudaStream_t s, int cfg = 0);
 cudaError_t launch_stage_mixed_ks64(const Grid& g, const StageArgsMixed& a, cudaStream_t s);
 int tile_config_count();
@@ -311,6 +318,9 @@ bool tile_config_has_fp64(int c);  // false for the mixed-only configurations
 const char* tile_config_name(int c);
 // TMA-staged mixed stage kernel (k_stage_tma.cu); map describes the float
 // stage buffer that is the stencil source.
+// Tensor map of a register as [field][z][y][x] (elem bytes: 4 float, 8 float64)
+// with a box of bx x by x bz points of one field.
+cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out);
 // Tensor map of a float stage buffer for TMA-staged variant v (0: 32 x 4 x 1
 // tiles, 1: 32 x 8 x 1; the box is the tile plus three ghost layers).
 cudaError_t make_stage_tensor_map(const Grid& g, const float* base, CUtensorMap* out, int variant = 0);

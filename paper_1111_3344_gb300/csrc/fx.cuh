@@ -45,24 +45,39 @@ __device__ __forceinline__ bool fx_zero(const double (&v)[N]) {
   for (int q = 0; q < N; q++) m |= ((unsigned)__double2hiint(v[q]) & 0x7fffffffu) | (unsigned)__double2loint(v[q]);
   return m == 0;
 }
-// biased exponents 128 .. 2026: every value below 2^-64 of the largest shifts
+// biased exponents 256 .. 1900: every value below 2^-64 of the largest shifts
 // out whole (so a subnormal's missing leading bit never shows), and no result
-// overflows or underflows
-__device__ __forceinline__ bool fx_ok(unsigned top) { return (top >> 20) - 128u <= 2026u - 128u; }
+// overflows or underflows, products with weights (FxWeights) included
+__device__ __forceinline__ bool fx_ok(unsigned top) { return (top >> 20) - 256u <= 1900u - 256u; }
 
-// v in units of 2^(E - 1075 - FX_BITS), E the biased exponent of top
+// v in units of 2^(E - 1075 - BITS), E the biased exponent of top
+template <int BITS = FX_BITS>
 __device__ __forceinline__ long long fx_from(double v, int E) {
   const int hi = __double2hiint(v), lo = __double2loint(v);
   const int sh = E - ((hi >> 20) & 0x7ff);
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
-  const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)lo) << FX_BITS;
+  const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)lo) << BITS;
   unsigned long long r;
   asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(sh));  // shifts of 64 and more give 0
   const long long s = hi >> 31;
   return (long long)((r ^ (unsigned long long)s) - (unsigned long long)s);
 }
 
-// s 2^(E - 1075 - FX_BITS + up), rounded to the nearest float64
+// v in the same units, rounded to the nearest
+template <int BITS>
+__device__ __forceinline__ long long fx_near(double v, int E) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const int sh = E - ((hi >> 20) & 0x7ff);
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)lo) << (BITS + 1);
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(sh));
+  r = (r + 1) >> 1;
+  const long long s = hi >> 31;
+  return (long long)((r ^ (unsigned long long)s) - (unsigned long long)s);
+}
+
+// s 2^(E - 1075 - FX_BITS), rounded to the nearest float64
 __device__ __forceinline__ double fx_to(long long s, int E) {
   const int neg = (int)(s >> 63);
   const unsigned long long a = (unsigned long long)((s ^ (long long)neg) - (long long)neg);
@@ -74,6 +89,40 @@ __device__ __forceinline__ double fx_to(long long s, int E) {
   const unsigned ex = (unsigned)(E + 10 - FX_BITS - n) << 20;
   const unsigned hi = a ? ((unsigned)(r >> 32) + ex) | ((unsigned)neg & 0x80000000u) : 0u;
   return __hiloint2double((int)hi, (int)(unsigned)r);
+}
+
+// Weights of a point (float64) for sums over stencil results: fixed point in
+// units of 2^(E - 1083), the largest in [2^60, 2^61).
+template <int N>
+struct FxWeights {
+  long long w[N];
+  int E;
+  bool ok;  // exponent within 2^-50 .. 2^60 (or all zero)
+};
+template <int N>
+__device__ __forceinline__ FxWeights<N> fx_weights(const double (&v)[N]) {
+  FxWeights<N> r;
+  const unsigned top = fx_top(v);
+  r.E = top ? (int)(top >> 20) : 1023;
+  r.ok = (unsigned)(r.E - 973) <= 110u;
+#pragma unroll
+  for (int q = 0; q < N; q++) r.w[q] = top ? fx_from<8>(v[q], r.E) : 0;
+  return r;
+}
+
+// sum_q a[q] w[q], a in units of 2^(Ea - 1075 - FX_BITS): the a are shifted up
+// together to their full width, so each truncated product is off by at most
+// 2^-60 of the largest a times the largest weight.
+template <int N>
+__device__ __forceinline__ double fx_dot(const long long (&a)[N], int Ea, const FxWeights<N>& w) {
+  unsigned long long m = 0;
+#pragma unroll
+  for (int q = 0; q < N; q++) m |= (unsigned long long)(a[q] ^ (a[q] >> 63));
+  const int n = __clzll((long long)m) - 1;  // |a| < 2^63: n >= 0
+  long long s = 0;
+#pragma unroll
+  for (int q = 0; q < N; q++) s += __mul64hi(a[q] << n, w.w[q]);
+  return fx_to(s, Ea - n + w.E - 1019);
 }
 
 // 144 h^2 d_a d_b of the field at p (strides sa, sb; a != b) times 2^up, up 0 or -1.

@@ -30,7 +30,7 @@ namespace bssn {
 // these divide the grid; else (flat) blocks of as many consecutive points of
 // the interior in x-y-z order, so that no thread and no warp but the last is
 // without a point (75 x 53 x 61: 5.9 against 8.1 thousand warps of 32 x 4 tiles).
-// MINB keeps 16 warps per SM resident (128 registers, spills of some 700 B per
+// (Where the tile form of k_stage_fx.cu does not apply.)  MINB keeps 16 warps per SM resident (128 registers, spills of some 700 B per
 // thread): the stencils wait on loads and integer chains, the algebra on the
 // float64 pipe, and only other warps fill either's gaps.  At 128^3 a step takes
 // 19.1 ms with 16 warps, 20.2 with 12, 25.3 with 8.
@@ -107,8 +107,10 @@ static const TileCfg k_tiles[] = {
 #undef TILE_MX
 #undef TILE
 
-// 32 x 4 x 1 blocks: 19.1 ms a step at 128^3 against 20.1 for 32 x 8 x 1
-// (smaller blocks leave together more evenly)
+// 32x4x1/1: float64 registers with a tensor map run in tiles of 8 x 4 x 4 points
+// (k_stage_fx.cu; also blocks of 128 threads), the fastest; without one, and
+// where tiles fit the grid badly, one point at a time in 32 x 4 x 1 blocks (19.1 ms a
+// step at 128^3 against 20.1 for 32 x 8 x 1: smaller blocks leave together more evenly)
 int fp64_default_tile() { return 1; }
 int tile_config_count() { return (int)(sizeof(k_tiles) / sizeof(k_tiles[0])); }
 bool tile_config_has_fp64(int c) { return c >= 0 && c < tile_config_count() && k_tiles[c].fp64 != nullptr; }
@@ -116,8 +118,10 @@ const char* tile_config_name(int c) {
   return (c >= 0 && c < tile_config_count()) ? k_tiles[c].name : "";
 }
 
-cudaError_t launch_stage_fp64(const Grid& g, const StageArgs& a, cudaStream_t s, int cfg) {
+cudaError_t launch_stage_fp64(const Grid& g, const StageArgs& a, cudaStream_t s, int cfg, const CUtensorMap* map,
+                              int* err) {
   if (!tile_config_has_fp64(cfg)) cfg = 0;
+  if (cfg == fp64_default_tile() && map && fx_tile_fits(g)) return launch_stage_fx(g, a, *map, err, s);
   return k_tiles[cfg].fp64(g, a, s);
 }
 

@@ -64,7 +64,7 @@ namespace {
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 }
 
-cudaError_t make_stage_tensor_map(const Grid& g, const float* base, CUtensorMap* out, int variant) {
+cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out) {
   // the encoding is a driver call and needs a current context: a thread whose
   // first CUDA call this is has none until a runtime call binds the primary
   // context of its device (cudaFree(nullptr) does, and frees nothing)
@@ -77,16 +77,20 @@ cudaError_t make_stage_tensor_map(const Grid& g, const float* base, CUtensorMap*
     if (e != cudaSuccess) return e;
     if (q != cudaDriverEntryPointSuccess || !g_encode) return cudaErrorNotSupported;
   }
-  const int by = variant >= 1 ? TmaShape<8>::BY : TmaShape<4>::BY;
-  const int bz = TmaShape<4>::BZ;
   cuuint64_t dims[4] = {(cuuint64_t)g.pitch, (cuuint64_t)g.sy, (cuuint64_t)g.sz, (cuuint64_t)NF};
-  cuuint64_t strides[3] = {(cuuint64_t)g.pitch * 4, (cuuint64_t)g.plane * 4, (cuuint64_t)g.fstride * 4};
-  cuuint32_t box[4] = {(cuuint32_t)TmaDefault::BX, (cuuint32_t)by, (cuuint32_t)bz, 1};
+  cuuint64_t strides[3] = {(cuuint64_t)g.pitch * elem, (cuuint64_t)g.plane * elem, (cuuint64_t)g.fstride * elem};
+  cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = g_encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (void*)base, dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  CUresult r = g_encode(out, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
+                        const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+cudaError_t make_stage_tensor_map(const Grid& g, const float* base, CUtensorMap* out, int variant) {
+  return encode_tensor_map(g, base, 4, TmaDefault::BX, variant >= 1 ? TmaShape<8>::BY : TmaShape<4>::BY,
+                           TmaShape<4>::BZ, out);
 }
 
 // dynamic shared memory above the default limit, once per kernel and device

@@ -12,12 +12,10 @@ __device__ __forceinline__ bool on_shell(const Grid& g, int ii, int jj, int kk) 
   return ii == 0 || jj == 0 || kk == 0 || ii == g.n0 - 1 || jj == g.n1 - 1 || kk == g.n2 - 1;
 }
 
-// Fused stage at interior point (ii, jj, kk) (interior indices), float64.
-__device__ __forceinline__ void stage_point_fp64(const Grid& g, const StageArgs& a, int ii, int jj, int kk) {
-  const int i = ii + GH, j = jj + GH, k = kk + GH;
-  const long long id = lin(g, i, j, k);
-  double r[NF];
-  rhs_fx(g, a.src, id, i, j, k, r);
+// Combine of a float64 stage at interior point (ii, jj, kk), linear index id,
+// with its right-hand side r.
+__device__ __forceinline__ void combine_fp64(const Grid& g, const StageArgs& a, long long id, int ii, int jj, int kk,
+                                             const double r[NF]) {
   const long long fs = g.fstride;
   const bool anchor = a.mode != MODE_RHS && a.kshell && on_shell(g, ii, jj, kk);
 #pragma unroll 4
@@ -35,6 +33,14 @@ __device__ __forceinline__ void stage_point_fp64(const Grid& g, const StageArgs&
       a.ksum[o] = a.mode == MODE_FIRST ? r[f] : fma(2.0, r[f], a.ksum[o]);
     }
   }
+}
+
+// Fused stage at interior point (ii, jj, kk) (interior indices), float64.
+__device__ __forceinline__ void stage_point_fp64(const Grid& g, const StageArgs& a, int ii, int jj, int kk) {
+  const long long id = lin(g, ii + GH, jj + GH, kk + GH);
+  double r[NF];
+  rhs_fx(g, a.src, id, ii + GH, jj + GH, kk + GH, r);
+  combine_fp64(g, a, id, ii, jj, kk, r);
 }
 
 // ---------------------------------------------------------------- mixed

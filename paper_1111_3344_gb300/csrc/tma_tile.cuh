@@ -1,7 +1,7 @@
 // Shared-memory tile of the TMA-staged mixed stage kernels (single grid:
 // k_stage_tma.cu; batched: k_batch_tma.cu): tile shape, the staged fields,
-// the accessor that reads them from shared memory, and the bounded mbarrier
-// wait.
+// the accessor that reads them from shared memory (bounded mbarrier wait:
+// tma.cuh).
 //
 // A block owns TTX x TTY x TTZ interior points.  One cp.async.bulk.tensor load
 // per staged field brings the field's box over the tile plus three ghost
@@ -13,11 +13,11 @@
 #include <cuda.h>
 
 #include "stage_point.cuh"
+#include "tma.cuh"
 
 namespace bssn {
 
 constexpr int NSTAGED = 8;
-constexpr long long WAIT_LIMIT = 1LL << 24;
 
 // Tile of 32 x TY x TZ interior points and its boxes: BX = 32 + 6 rounded up
 // to a multiple of 4 floats, BY = TY + 6, BZ = TZ + 6 (three ghost layers on
@@ -76,29 +76,6 @@ struct TileAccT {
 };
 using TileAcc = TileAccT<TmaDefault>;
 
-__device__ __forceinline__ unsigned smem_addr(const void* p) {
-  return (unsigned)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, long long limit) {
-  for (long long it = 0; it < limit; it++) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
-__device__ __forceinline__ void mbar_init(unsigned bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
 // Thread 0: arm the barrier for the staged bytes and issue one tensor load per
 // staged field, box origin (x0, y0, z0) in stored coordinates (the interior
 // start of the tile minus the ghost width; x0 a multiple of 32, so the
@@ -107,16 +84,11 @@ __device__ __forceinline__ void mbar_init(unsigned bar) {
 template <typename Sh = TmaDefault>
 __device__ __forceinline__ void issue_staged_loads(const void* tmap, unsigned bar, float* smem, int x0, int y0,
                                                    int z0) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(Sh::BYTES)
-               : "memory");
+  mbar_expect(bar, Sh::BYTES);
 #pragma unroll
   for (int s = 0; s < Sh::NST; s++) {
     const int f = staged_field(s);
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_addr(smem + s * Sh::SLOT)),
-        "l"(reinterpret_cast<unsigned long long>(tmap)), "r"(x0), "r"(y0), "r"(z0), "r"(f), "r"(bar)
-        : "memory");
+    tensor_load_4d(smem + s * Sh::SLOT, tmap, x0, y0, z0, f, bar);
   }
 }
 

@@ -105,3 +105,35 @@ def test_norms_at_block_edges(n, r_excise):
     got = evo.constraints()
     assert np.isnan(got[:8]).any() and (r_excise > 10 or np.isnan(got[8:]).any())
     evo.close()
+
+
+@pytest.mark.parametrize("n", [(8, 4, 4), (9, 5, 5), (7, 3 + 1, 8), (16, 8, 4), (57, 58, 59), (72, 20, 36)])
+@pytest.mark.parametrize("conformal", ["W", "phi"])
+def test_tile_form_equals_the_point_form(n, conformal):
+    """The stage in tiles (csrc/k_stage_fx.cu; whole tiles, one point past them,
+    one point short) against the oracle and against one point at a time, which
+    a register that no tensor load can describe (8-byte aligned) takes: also
+    with a field of zeros, fields that hold one tiny and one subnormal value
+    (those tiles by the float64 sums), a shift of zero, and not a number in the padding of the rows.  Bars as above; the two forms differ
+    by the roundings of both, twice the bar."""
+    import torch
+    from paper_1111_3344_gb300.bssn import Evolution
+    c, st = _case(n, 23, conformal=conformal)
+    if conformal == "phi":
+        st[0] = -0.5 * np.log(st[0])
+    st[21:24] = 0.0
+    st[22, 4, 5, 4], st[23, 4, 5, 4] = 1e-290, 5e-324
+    st[18:21, -6:] = 0.0
+    evo = Evolution(T.gpu_params(c))
+    reg = evo.numpy_to_register(st)
+    reg.view(24, st.shape[1], st.shape[2], -1)[..., st.shape[3]:] = float("nan")  # the padding of a row may hold anything
+    got = evo.register_to_numpy(evo.rhs(reg))
+    odd = torch.empty(reg.numel() + 1, dtype=reg.dtype, device=reg.device)[1:].view(reg.shape)
+    assert odd.data_ptr() % 16 == 8
+    odd.copy_(reg)
+    point = evo.register_to_numpy(evo.rhs(odd))
+    evo.close()
+    want, mag = O.rhs_mag(T.oracle_cfg(c), st)
+    assert T.rounding_aware_errors(got, want, mag).max() <= 1.0
+    assert T.rounding_aware_errors(point, want, mag).max() <= 1.0
+    assert T.rounding_aware_errors(got, point, mag).max() <= 2.0
