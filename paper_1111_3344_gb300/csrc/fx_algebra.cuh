@@ -221,11 +221,11 @@ __device__ __forceinline__ void fx_lapse(const Grid& g, const FxMetric& M, doubl
 // dissipation (zero for a frozen shift).  DB(a, d) = 12h d_d beta^a, LAPB(a) =
 // 144 h^2 gt^kl d_k d_l beta^a, ROW(a, k) = 144 h^2 d_k d_a beta^a (no sum), DK(d) =
 // 12h d_d K.  (i, j, k), id: the point's stored indices and linear index.
-template <typename B_, typename L_, typename R, typename K_>
+template <typename B_, typename L_, typename R, typename K_, typename Out>
 __device__ __forceinline__ void fx_assemble(const Grid& g, const double* __restrict__ c0, long long id, int i, int j,
                                             int k, const FxMetric& M, B_ DB, L_ LAPB, R ROW, K_ DK,
                                             const double G2[3][6], const double V2[3], const double vj[3],
-                                            const double X[6], double lap, double out[NF]) {
+                                            const double X[6], double lap, Out out) {
   const long long fs = g.fstride;
   const double u = g.i12h, chi = M.chi;
   const double(&gt)[6] = M.gt, (&gu)[6] = M.gu;

@@ -12,6 +12,21 @@ __device__ __forceinline__ bool on_shell(const Grid& g, int ii, int jj, int kk) 
   return ii == 0 || jj == 0 || kk == 0 || ii == g.n0 - 1 || jj == g.n1 - 1 || kk == g.n2 - 1;
 }
 
+// Combine of one field of a float64 stage at register offset o with its
+// right-hand side r; anchor: the point is next to the outer boundary.
+__device__ __forceinline__ void combine_field_fp64(const StageArgs& a, long long o, double r, bool anchor) {
+  if (a.mode == MODE_RHS) {
+    a.rhs[o] = r;
+    return;
+  }
+  if (anchor) a.kshell[o] = r;
+  if (a.mode == MODE_LAST) {
+    a.yn[o] = fma(a.b_dt, a.ksum[o] + r, a.yn[o]);
+  } else {
+    a.out0[o] = fma(a.a_dt, r, a.src0[o]);
+    a.ksum[o] = a.mode == MODE_FIRST ? r : fma(2.0, r, a.ksum[o]);
+  }
+}
 // Combine of a float64 stage at interior point (ii, jj, kk), linear index id,
 // with its right-hand side r.
 __device__ __forceinline__ void combine_fp64(const Grid& g, const StageArgs& a, long long id, int ii, int jj, int kk,
@@ -19,20 +34,7 @@ __device__ __forceinline__ void combine_fp64(const Grid& g, const StageArgs& a, 
   const long long fs = g.fstride;
   const bool anchor = a.mode != MODE_RHS && a.kshell && on_shell(g, ii, jj, kk);
 #pragma unroll 4
-  for (int f = 0; f < NF; f++) {
-    const long long o = f * fs + id;
-    if (a.mode == MODE_RHS) {
-      a.rhs[o] = r[f];
-      continue;
-    }
-    if (anchor) a.kshell[o] = r[f];
-    if (a.mode == MODE_LAST) {
-      a.yn[o] = fma(a.b_dt, a.ksum[o] + r[f], a.yn[o]);
-    } else {
-      a.out0[o] = fma(a.a_dt, r[f], a.src0[o]);
-      a.ksum[o] = a.mode == MODE_FIRST ? r[f] : fma(2.0, r[f], a.ksum[o]);
-    }
-  }
+  for (int f = 0; f < NF; f++) combine_field_fp64(a, f * fs + id, r[f], anchor);
 }
 
 // Fused stage at interior point (ii, jj, kk) (interior indices), float64.

@@ -107,11 +107,13 @@ def test_norms_at_block_edges(n, r_excise):
     evo.close()
 
 
-@pytest.mark.parametrize("n", [(8, 4, 4), (9, 5, 5), (7, 3 + 1, 8), (16, 8, 4), (57, 58, 59), (72, 20, 36)])
+@pytest.mark.parametrize("n", [(8, 4, 4), (9, 5, 5), (7, 4, 8), (16, 8, 4), (72, 20, 36),
+                               (74, 21, 36), (64, 32, 60), (57, 58, 59)])
 @pytest.mark.parametrize("conformal", ["W", "phi"])
 def test_tile_form_equals_the_point_form(n, conformal):
     """The stage in tiles (csrc/k_stage_fx.cu; whole tiles, one point past them,
-    one point short) against the oracle and against one point at a time, which
+    one point short; with groups of threads up to 456 tiles, (72, 20, 36) being
+    405 and (74, 21, 36) 540, without from there) against the oracle and against one point at a time, which
     a register that no tensor load can describe (8-byte aligned) takes: also
     with a field of zeros, fields that hold one tiny and one subnormal value
     (those tiles by the float64 sums), a shift of zero, and not a number in the padding of the rows.  Bars as above; the two forms differ
