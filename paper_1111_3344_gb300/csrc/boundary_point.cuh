@@ -4,6 +4,7 @@
 #pragma once
 #include "bssn_internal.cuh"
 #include "rhs_point.cuh"
+#include "stage_point.cuh"
 
 namespace bssn {
 
@@ -34,33 +35,89 @@ __device__ __forceinline__ ff cvt<ff, float2>(float2 v) {
   return ff(v);
 }
 
-// Radiative right-hand side of field f at stored point I in arithmetic C;
-// p points at the field's value there; ns = (x / r) / (2h), the normal scaled
-// by the difference weight (formed once per point for all fields), ir = 1 / r.
-template <typename C, typename S, bool DEV = false>
-__device__ __forceinline__ C rad_at(const Grid& g, const S* __restrict__ p, int f, const int I[3],
-                                    const C ns[3], C ir) {
+// Offsets of the two neighbours per axis that the first differences at stored
+// point I read: centred where both are stored, else the two inward ones.  Formed
+// once per point, so that the fields' loads are under no branch and in flight
+// together.
+struct RadTaps {
+  long long oa[3], ob[3];
+  int kind[3];  // 0 centred, 1 one-sided at the last point, -1 at the first
+  __device__ __forceinline__ bool edge() const { return (kind[0] | kind[1] | kind[2]) != 0; }
+};
+__device__ __forceinline__ RadTaps rad_taps(const Grid& g, const int I[3]) {
   const long long sd[3] = {1, g.pitch, g.plane};
   const int dims[3] = {g.sx, g.sy, g.sz};
-  const bool one = (f == F_ALP || (f == F_CHI && g.use_w) || f == F_GT + 0 || f == F_GT + 3 ||
-                   f == F_GT + 5);
-  const C X0 = (DEV || !one) ? C(0) : C(1);  // DEV: p holds X - X0 already
+  RadTaps T;
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    T.kind[d] = I[d] >= 1 && I[d] + 1 < dims[d] ? 0 : (I[d] + 1 >= dims[d] ? 1 : -1);
+    T.oa[d] = T.kind[d] == 1 ? -sd[d] : sd[d];
+    T.ob[d] = T.kind[d] == 0 ? -sd[d] : 2 * T.oa[d];
+  }
+  return T;
+}
+// at an interior point
+__device__ __forceinline__ RadTaps rad_taps_inside(const Grid& g) {
+  return {{1, g.pitch, g.plane}, {-1, -g.pitch, -g.plane}, {0, 0, 0}};
+}
+
+// Radiative right-hand side of field f in arithmetic C at the point whose value
+// p points at (its taps T); ns = (x / r) / (2h), the normal scaled by the
+// difference weight (formed once per point for all fields), ir = 1 / r.
+__device__ __forceinline__ bool rad_background(const Grid& g, int f) {
+  return f == F_ALP || (f == F_CHI && g.use_w) || f == F_GT + 0 || f == F_GT + 3 || f == F_GT + 5;
+}
+template <typename C, typename S, bool DEV = false>
+__device__ __forceinline__ C rad_at(const Grid& g, const S* __restrict__ p, int f, const RadTaps& T,
+                                    const C ns[3], C ir) {
+  const C X0 = (DEV || !rad_background(g, f)) ? C(0) : C(1);  // DEV: p holds X - X0 already
   const C v0 = (f == F_ALP || f == F_TRK) ? C(1.4142135623730951) : C(1);
   C s = (cvt<C>(p[0]) - X0) * ir;
 #pragma unroll
   for (int d = 0; d < 3; d++) {
-    const long long q = sd[d];
+    const C va = cvt<C>(p[T.oa[d]]), vb = cvt<C>(p[T.ob[d]]);
     C der;
-    if (I[d] >= 1 && I[d] + 1 < dims[d])
-      der = cvt<C>(p[q]) - cvt<C>(p[-q]);
-    else if (I[d] + 1 >= dims[d])
-      der = C(3) * cvt<C>(p[0]) - C(4) * cvt<C>(p[-q]) + cvt<C>(p[-2 * q]);
-    else
-      der = -(C(3) * cvt<C>(p[0]) - C(4) * cvt<C>(p[q]) + cvt<C>(p[2 * q]));
+    if (T.kind[d] == 0) {
+      der = va - vb;
+    } else {
+      der = C(3) * cvt<C>(p[0]) - C(4) * va + vb;
+      if (T.kind[d] < 0) der = -der;
+    }
     s = fmaT<C>(ns[d], der, s);
   }
   return -v0 * s;
 }
+
+// The same in float64 in two halves, for a group of fields: the values, then
+// the sum.  One-sided differences become a - b with a = 3 p0 - 4 a, b = -b,
+// negated at the first point with the normal's sign: one branch for the group
+// (edge), for the float64 pipe bounds that kernel and most points need none.
+struct RadVals {
+  double p0, a[3], b[3];
+  __device__ __forceinline__ void load(const double* __restrict__ p, const RadTaps& T) {
+    p0 = p[0];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+      a[d] = p[T.oa[d]];
+      b[d] = p[T.ob[d]];
+    }
+  }
+  __device__ __forceinline__ void edge(const RadTaps& T) {
+#pragma unroll
+    for (int d = 0; d < 3; d++)
+      if (T.kind[d] != 0) {
+        a[d] = 3.0 * p0 - 4.0 * a[d];
+        b[d] = -b[d];
+      }
+  }
+  __device__ __forceinline__ double sum(const Grid& g, int f, const RadTaps& T, const double ns[3], double ir) const {
+    const double v0 = (f == F_ALP || f == F_TRK) ? 1.4142135623730951 : 1.0;
+    double s = (p0 - (rad_background(g, f) ? 1.0 : 0.0)) * ir;
+#pragma unroll
+    for (int d = 0; d < 3; d++) s = fma(T.kind[d] < 0 ? -ns[d] : ns[d], a[d] - b[d], s);
+    return -v0 * s;
+  }
+};
 
 // Geometry of one ghost point: its anchor and the radial factors.
 struct GhostGeo {
@@ -142,21 +199,25 @@ __device__ __forceinline__ void sommerfeld_point_fp64_tab(const Grid& g, const S
   const long long ib = lin(g, I[0], I[1], I[2]), ia = lin(g, A[0], A[1], A[2]);
   const long long fs = g.fstride;
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
+  const RadTaps tb = rad_taps(g, I);
+  constexpr int N = F1 - F0;
+  long long o[N];
+  RadVals v[N];
+  double ka[N], rhs[N];
 #pragma unroll
-  for (int f = F0; f < F1; f++) {
-    double rhs = 0.0;
-    if (f < nf) {
-      const double radb = rad_at<double, double>(g, a.src + f * fs + ib, f, I, nbs, irb);
-      rhs = fma(fac, kanchor[f * fs + ia], radb);
-    }
-    const long long o = f * fs + ib;
-    if (a.mode == MODE_LAST) {
-      a.yn[o] = fma(a.b_dt, a.ksum[o] + rhs, a.yn[o]);
-    } else {
-      a.out0[o] = fma(a.a_dt, rhs, a.src0[o]);
-      a.ksum[o] = a.mode == MODE_FIRST ? rhs : fma(2.0, rhs, a.ksum[o]);
-    }
+  for (int n = 0; n < N; n++) {
+    o[n] = (F0 + n) * fs + ib;
+    v[n].load(a.src + o[n], tb);
+    ka[n] = kanchor[(F0 + n) * fs + ia];
   }
+  if (tb.edge()) {
+#pragma unroll
+    for (int n = 0; n < N; n++) v[n].edge(tb);
+  }
+#pragma unroll
+  for (int n = 0; n < N; n++)
+    rhs[n] = F0 + n < nf ? fma(fac, ka[n], v[n].sum(g, F0 + n, tb, nbs, irb)) : 0.0;
+  combine_fields_fp64(a, o, rhs);
 }
 
 // float64 path, anchor pass: interior point q of the boundary shell, fields
@@ -181,12 +242,14 @@ __device__ __forceinline__ void sommerfeld_anchor_fp64(const Grid& g, const Stag
   const long long ia = lin(g, A[0], A[1], A[2]);
   const long long fs = g.fstride;
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
+  const RadTaps ta = rad_taps_inside(g);
+  double k[F1 - F0];  // every load before the stores
 #pragma unroll
-  for (int f = F0; f < F1; f++) {
-    if (f >= nf) break;
-    const double rada = rad_at<double, double>(g, a.src + f * fs + ia, f, A, nas, ira);
-    kanchor[f * fs + ia] -= rada;
-  }
+  for (int f = F0; f < F1; f++)
+    if (f < nf) k[f - F0] = kanchor[f * fs + ia] - rad_at<double, double>(g, a.src + f * fs + ia, f, ta, nas, ira);
+#pragma unroll
+  for (int f = F0; f < F1; f++)
+    if (f < nf) kanchor[f * fs + ia] = k[f - F0];
 }
 
 // float64 path: ghost point q, all fields.  PRE: kanchor already holds
@@ -198,14 +261,15 @@ __device__ __forceinline__ void sommerfeld_point_fp64(const Grid& g, const Stage
   ghost_geo(g, q, G);
   const long long fs = g.fstride;
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
+  const RadTaps tb = rad_taps(g, G.I), ta = rad_taps_inside(g);
   for (int f = 0; f < NF; f++) {
     double rhs = 0.0;
     if (f < nf) {
-      const double radb = rad_at<double, double>(g, a.src + f * fs + G.ib, f, G.I, G.nbs, G.irb);
+      const double radb = rad_at<double, double>(g, a.src + f * fs + G.ib, f, tb, G.nbs, G.irb);
       if (PRE && a.mode != MODE_RHS) {
         rhs = fma(G.fac, kanchor[f * fs + G.ia], radb);
       } else {
-        const double rada = rad_at<double, double>(g, a.src + f * fs + G.ia, f, G.A, G.nas, G.ira);
+        const double rada = rad_at<double, double>(g, a.src + f * fs + G.ia, f, ta, G.nas, G.ira);
         const double ka = (a.mode == MODE_RHS) ? a.rhs[f * fs + G.ia] : kanchor[f * fs + G.ia];
         rhs = fma(G.fac, ka - rada, radb);
       }
@@ -237,11 +301,12 @@ __device__ __forceinline__ void sommerfeld_point_mixed(const Grid& g, const Stag
   const long long ib = lin(g, I[0], I[1], I[2]);
   const long long ia = lin(g, A[0], A[1], A[2]);
   const long long o = f * fs + ib;
+  const RadTaps tb = rad_taps(g, I), ta = rad_taps_inside(g);
   if (f == F_CHI) {
     GhostGeo G;
     ghost_geo(g, q, G);
-    const double radb = rad_at<double, double>(g, a.srcw + ib, f, I, G.nbs, G.irb);
-    const double rada = rad_at<double, double>(g, a.srcw + ia, f, A, G.nas, G.ira);
+    const double radb = rad_at<double, double>(g, a.srcw + ib, f, tb, G.nbs, G.irb);
+    const double rada = rad_at<double, double>(g, a.srcw + ia, f, ta, G.nas, G.ira);
     const double ka = (a.mode == MODE_RHS) ? a.rhs[ia] : (double)kanchor[ia];
     const double rhs = fma(G.fac, ka - rada, radb);
     if (a.mode == MODE_RHS) {
@@ -272,8 +337,8 @@ __device__ __forceinline__ void sommerfeld_point_mixed(const Grid& g, const Stag
     const float nbs[3] = {xb[0] * irb * g.i2hf, xb[1] * irb * g.i2hf, xb[2] * irb * g.i2hf};
     const float nas[3] = {xa[0] * ira * g.i2hf, xa[1] * ira * g.i2hf, xa[2] * ira * g.i2hf};
     const float fac = (irb / ira) * (irb / ira);
-    const float radb = rad_at<float, float, true>(g, a.src + o, f, I, nbs, irb);
-    const float rada = rad_at<float, float, true>(g, a.src + f * fs + ia, f, A, nas, ira);
+    const float radb = rad_at<float, float, true>(g, a.src + o, f, tb, nbs, irb);
+    const float rada = rad_at<float, float, true>(g, a.src + f * fs + ia, f, ta, nas, ira);
     const float ka = (a.mode == MODE_RHS) ? (float)a.rhs[f * fs + ia] : kanchor[f * fs + ia];
     rhs = fmaf(fac, ka - rada, radb);
   }
@@ -324,29 +389,58 @@ __device__ __forceinline__ void sommerfeld_point_mixed_fields(const Grid& g, con
   const float nbs[3] = {xb[0] * irb * g.i2hf, xb[1] * irb * g.i2hf, xb[2] * irb * g.i2hf};
   const float nas[3] = {xa[0] * ira * g.i2hf, xa[1] * ira * g.i2hf, xa[2] * ira * g.i2hf};
   const float fac = (irb / ira) * (irb / ira);
-#pragma unroll (UNROLL ? F1 - FB : 1)
-  for (int f = FB; f < F1; f++) {
-    const long long o = f * fs + ib;
-    float rhs = 0.0f;
-    if (f < nf) {
-      const float radb = rad_at<float, float, true>(g, a.src + o, f, I, nbs, irb);
-      const float rada = rad_at<float, float, true>(g, a.src + f * fs + ia, f, A, nas, ira);
-      const float ka = (a.mode == MODE_RHS) ? (float)a.rhs[f * fs + ia] : kanchor[f * fs + ia];
-      rhs = fmaf(fac, ka - rada, radb);
+  const RadTaps tb = rad_taps(g, I), ta = rad_taps_inside(g);
+  // groups of N fields, every load of a group before its stores
+  constexpr int N = UNROLL && F1 > FB ? F1 - FB : 1;
+#pragma unroll 1
+  for (int f0 = FB; f0 < F1; f0 += N) {
+    float rhs[N], b[N], ks[N];
+    double bd[N], kd[N];
+#pragma unroll
+    for (int m = 0; m < N; m++) {
+      const int f = f0 + m;
+      rhs[m] = 0.0f;
+      if (f < nf) {
+        const float radb = rad_at<float, float, true>(g, a.src + f * fs + ib, f, tb, nbs, irb);
+        const float rada = rad_at<float, float, true>(g, a.src + f * fs + ia, f, ta, nas, ira);
+        const float ka = (a.mode == MODE_RHS) ? (float)a.rhs[f * fs + ia] : kanchor[f * fs + ia];
+        rhs[m] = fmaf(fac, ka - rada, radb);
+      }
     }
     if (a.mode == MODE_RHS) {
-      a.rhs[o] = (double)rhs;
-    } else if (a.mode == MODE_LAST) {
-      const double ks = a.ksum64 ? a.ksum64[o] + (double)rhs : (double)(a.ksum[o] + rhs);
-      const double v = fma(a.b_dt, ks, a.yn[o]);
-      a.yn[o] = v;
-      a.out0[o] = (float)(v - background(g, f));
-    } else {
-      a.out0[o] = fmaf(a.a_dtf, rhs, a.src0[o]);
+#pragma unroll
+      for (int m = 0; m < N; m++) a.rhs[(f0 + m) * fs + ib] = (double)rhs[m];
+      continue;
+    }
+    if (a.mode != MODE_FIRST && a.ksum64) {
+#pragma unroll
+      for (int m = 0; m < N; m++) kd[m] = a.ksum64[(f0 + m) * fs + ib];
+    } else if (a.mode != MODE_FIRST) {
+#pragma unroll
+      for (int m = 0; m < N; m++) ks[m] = a.ksum[(f0 + m) * fs + ib];
+    }
+    if (a.mode == MODE_LAST) {
+#pragma unroll
+      for (int m = 0; m < N; m++) bd[m] = a.yn[(f0 + m) * fs + ib];
+#pragma unroll
+      for (int m = 0; m < N; m++) {
+        const long long o = (f0 + m) * fs + ib;
+        const double v = fma(a.b_dt, a.ksum64 ? kd[m] + (double)rhs[m] : (double)(ks[m] + rhs[m]), bd[m]);
+        a.yn[o] = v;
+        a.out0[o] = (float)(v - background(g, f0 + m));
+      }
+      continue;
+    }
+#pragma unroll
+    for (int m = 0; m < N; m++) b[m] = a.src0[(f0 + m) * fs + ib];
+#pragma unroll
+    for (int m = 0; m < N; m++) {
+      const long long o = (f0 + m) * fs + ib;
+      a.out0[o] = fmaf(a.a_dtf, rhs[m], b[m]);
       if (a.ksum64)
-        a.ksum64[o] = a.mode == MODE_FIRST ? (double)rhs : fma(2.0, (double)rhs, a.ksum64[o]);
+        a.ksum64[o] = a.mode == MODE_FIRST ? (double)rhs[m] : fma(2.0, (double)rhs[m], kd[m]);
       else
-        a.ksum[o] = a.mode == MODE_FIRST ? rhs : fmaf(2.0f, rhs, a.ksum[o]);
+        a.ksum[o] = a.mode == MODE_FIRST ? rhs[m] : fmaf(2.0f, rhs[m], ks[m]);
     }
   }
 }
@@ -368,7 +462,16 @@ __device__ __forceinline__ void periodic_point(const Grid& g, S* __restrict__ y,
   const int sj = GH + ((j - GH) % g.n1 + g.n1) % g.n1;
   const int sk = GH + ((k - GH) % g.n2 + g.n2) % g.n2;
   const long long d = lin(g, i, j, k), s = lin(g, si, sj, sk);
-  for (int f = 0; f < NF; f++) y[f * g.fstride + d] = y[f * g.fstride + s];
+  // every load of a group before its stores
+  constexpr int N = 8;
+#pragma unroll
+  for (int f0 = 0; f0 < NF; f0 += N) {
+    S v[N];
+#pragma unroll
+    for (int n = 0; n < N; n++) v[n] = y[(f0 + n) * g.fstride + s];
+#pragma unroll
+    for (int n = 0; n < N; n++) y[(f0 + n) * g.fstride + d] = v[n];
+  }
   if (w) w[d] = w[s];
 }
 
@@ -391,11 +494,12 @@ __device__ __forceinline__ void sommerfeld_point_ff(const Grid& g, const StageAr
   const ff adt(a.a_hi, a.a_lo);
   const long long fs = g.fstride;
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
+  const RadTaps tb = rad_taps(g, G.I), ta = rad_taps_inside(g);
   for (int f = 0; f < NF; f++) {
     ff rhs(0.0f, 0.0f);
     if (f < nf) {
-      const ff radb = rad_at<ff, float2>(g, a.src + f * fs + G.ib, f, G.I, nbs, irb);
-      const ff rada = rad_at<ff, float2>(g, a.src + f * fs + G.ia, f, G.A, nas, ira);
+      const ff radb = rad_at<ff, float2>(g, a.src + f * fs + G.ib, f, tb, nbs, irb);
+      const ff rada = rad_at<ff, float2>(g, a.src + f * fs + G.ia, f, ta, nas, ira);
       const ff ka = (a.mode == MODE_RHS) ? ff_from_double(a.rhs[f * fs + G.ia]) : ff(kanchor[f * fs + G.ia]);
       rhs = ff_fma(fac, ka - rada, radb);
     }

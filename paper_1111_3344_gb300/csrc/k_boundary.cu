@@ -38,6 +38,10 @@ __global__ void sommerfeld_anchor_fp64_kernel(Grid g, StageArgs a, double* __res
   }
 }
 
+// Loads first as well; the one-sided differences of the outermost points under
+// one branch for the group, for the float64 pipe bounds it (computed for every
+// point and selected: 328 us at 128^3 against 293; one field after another: 38 us
+// at 24^3, 74 at 48^3, 299 at 128^3; so 29, 61, 293).
 __global__ void sommerfeld_fp64_tab_kernel(Grid g, StageArgs a, const double* __restrict__ kanchor,
                                            const double* __restrict__ tab, const long long* __restrict__ itab) {
   const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -70,8 +74,11 @@ size_t ghost_table_size(const Grid& g) { return ghost_table_bytes(g); }
 // one thread per ghost point, every field (geometry formed once)
 // mixed: blockIdx.y picks one of four field groups (W and gt_ij; K and
 // At_ij but its last; the rest of At_ij, Gt^i, alpha; beta^i and B^i), each
-// a few unrolled fields per thread (their loads in flight together; the
-// kernel is bound by load latency)
+// a few unrolled fields per thread.  Bound by load latency: every load of a
+// group comes before its stores and under no branch (loads and stores of one
+// field after another, the neighbours of each under its own branches: 34 us
+// at 48^3, 175 at 128^3; so 25 and 139).  Interleaving the groups' blocks (31 at
+// 48^3) and fewer registers (40 with 80) are slower.
 __global__ void sommerfeld_mixed_kernel(Grid g, StageArgsMixed a, const float* __restrict__ kanchor) {
   const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= ghost_count(g)) return;

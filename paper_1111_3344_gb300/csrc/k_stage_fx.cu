@@ -201,8 +201,15 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
   __syncthreads();
   if (ii >= g.n0 || jj >= g.n1 || kk >= g.n2) return;
   const bool anchor = a.mode != MODE_RHS && a.kshell && on_shell(g, ii, jj, kk);
+  constexpr int N = NF / GROUPS;
+  long long o[N];
+  double r[N];
 #pragma unroll
-  for (int f = grp; f < NF; f += GROUPS) combine_field_fp64(a, f * fs + id, sm.out[f][tid], anchor);
+  for (int n = 0; n < N; n++) {
+    o[n] = (n * GROUPS + grp) * fs + id;
+    r[n] = sm.out[n * GROUPS + grp][tid];
+  }
+  combine_point_fp64(a, o, r, anchor);
 }
 
 // (and the shared-memory limit of the kernel that may read through the map, so

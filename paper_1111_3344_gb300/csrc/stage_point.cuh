@@ -12,20 +12,42 @@ __device__ __forceinline__ bool on_shell(const Grid& g, int ii, int jj, int kk) 
   return ii == 0 || jj == 0 || kk == 0 || ii == g.n0 - 1 || jj == g.n1 - 1 || kk == g.n2 - 1;
 }
 
-// Combine of one field of a float64 stage at register offset o with its
-// right-hand side r; anchor: the point is next to the outer boundary.
-__device__ __forceinline__ void combine_field_fp64(const StageArgs& a, long long o, double r, bool anchor) {
-  if (a.mode == MODE_RHS) {
-    a.rhs[o] = r;
-    return;
+// RK4 roles of N fields of a float64 stage, register offsets o[n], right-hand
+// sides r[n].  Every load comes before the first store, so that they are in
+// flight together (the compiler cannot move a load above a store to a register
+// it cannot tell apart).
+template <int N>
+__device__ __forceinline__ void combine_fields_fp64(const StageArgs& a, const long long (&o)[N], const double (&r)[N]) {
+  double b[N], ks[N];
+  const double* base = a.mode == MODE_LAST ? a.yn : a.src0;
+#pragma unroll
+  for (int n = 0; n < N; n++) b[n] = base[o[n]];
+  if (a.mode != MODE_FIRST) {
+#pragma unroll
+    for (int n = 0; n < N; n++) ks[n] = a.ksum[o[n]];
   }
-  if (anchor) a.kshell[o] = r;
   if (a.mode == MODE_LAST) {
-    a.yn[o] = fma(a.b_dt, a.ksum[o] + r, a.yn[o]);
+#pragma unroll
+    for (int n = 0; n < N; n++) a.yn[o[n]] = fma(a.b_dt, ks[n] + r[n], b[n]);
   } else {
-    a.out0[o] = fma(a.a_dt, r, a.src0[o]);
-    a.ksum[o] = a.mode == MODE_FIRST ? r : fma(2.0, r, a.ksum[o]);
+#pragma unroll
+    for (int n = 0; n < N; n++) {
+      a.out0[o[n]] = fma(a.a_dt, r[n], b[n]);
+      a.ksum[o[n]] = a.mode == MODE_FIRST ? r[n] : fma(2.0, r[n], ks[n]);
+    }
   }
+}
+// The same for an interior point, with the right-hand side written out
+// (MODE_RHS) or left at an anchor (next to the outer boundary).
+template <int N>
+__device__ __forceinline__ void combine_point_fp64(const StageArgs& a, const long long (&o)[N], const double (&r)[N],
+                                                   bool anchor) {
+  double* k = a.mode == MODE_RHS ? a.rhs : a.kshell;
+  if (a.mode == MODE_RHS || anchor) {
+#pragma unroll
+    for (int n = 0; n < N; n++) k[o[n]] = r[n];
+  }
+  if (a.mode != MODE_RHS) combine_fields_fp64(a, o, r);
 }
 // Combine of a float64 stage at interior point (ii, jj, kk), linear index id,
 // with its right-hand side r.
@@ -33,8 +55,18 @@ __device__ __forceinline__ void combine_fp64(const Grid& g, const StageArgs& a, 
                                              const double r[NF]) {
   const long long fs = g.fstride;
   const bool anchor = a.mode != MODE_RHS && a.kshell && on_shell(g, ii, jj, kk);
-#pragma unroll 4
-  for (int f = 0; f < NF; f++) combine_field_fp64(a, f * fs + id, r[f], anchor);
+  constexpr int N = 6;
+#pragma unroll 1
+  for (int f = 0; f < NF; f += N) {
+    long long o[N];
+    double x[N];
+#pragma unroll
+    for (int n = 0; n < N; n++) {
+      o[n] = (f + n) * fs + id;
+      x[n] = r[f + n];
+    }
+    combine_point_fp64(a, o, x, anchor);
+  }
 }
 
 // Fused stage at interior point (ii, jj, kk) (interior indices), float64.
@@ -147,6 +179,10 @@ __device__ __forceinline__ void stage_point_mixed_acc(const Grid& g, const Stage
     return;
   }
   const float af = a.a_dtf;
+  if (a.mode == MODE_FIRST) {  // every load before the stores
+#pragma unroll
+    for (int f = 1; f < NF; f++) ps[f] = a.src0[f * fs + id];
+  }
   {
     const double v = fma(a.a_dt, rchi, a.src0w[id]);
     a.out0w[id] = v;
@@ -156,7 +192,7 @@ __device__ __forceinline__ void stage_point_mixed_acc(const Grid& g, const Stage
 #pragma unroll
   for (int f = 1; f < NF; f++) {
     const long long o = f * fs + id;
-    a.out0[o] = fmaf(af, r[f], a.mode == MODE_FIRST ? a.src0[o] : ps[f]);
+    a.out0[o] = fmaf(af, r[f], ps[f]);
     if (ks64)
       a.ksum64[o] = a.mode == MODE_FIRST ? (double)r[f] : fma(2.0, (double)r[f], a.ksum64[o]);
     else
