@@ -75,10 +75,11 @@ enum { BSSN_ID_FLAT = 0, BSSN_ID_GAUGE_WAVE = 1, BSSN_ID_BL = 2, BSSN_ID_KASNER 
  *  precision           BSSN_FP64: everything in float64.  BSSN_MIXED:
  *                      stencils and right-hand side in float32, RK4 state
  *                      and constraint reductions in float64.  BSSN_FF:
- *                      stencils and right-hand side in double-word
- *                      ("float-float", 48-bit) arithmetic on the float32
- *                      pipe, RK4 state, k-sum and reductions in float64
- *                      (contexts, batches and the server).
+ *                      right-hand side to at least double-word (48-bit)
+ *                      precision, RK4 state, k-sum and reductions in float64
+ *                      (contexts, batches and the server); evaluated by the
+ *                      float64 stage, which is faster than double-word
+ *                      arithmetic.
  *  ksum_fp64           mixed precision, single-grid contexts only: 1 keeps
  *                      the weighted sum of the RK4 k of every field in
  *                      float64 (one more float64 register; W's is float64
@@ -316,6 +317,8 @@ bssn_status bssn_set_staging(bssn_ctx* ctx, void* d_mem, size_t bytes);
  * A new context starts on the fastest measured configuration of its precision
  * (mixed: "tma11_32x8x1/1"; float64: "32x4x1/1", whose float64 form stages boxes of
  * 8x4x4 points in shared memory by tensor loads where these fit the grid).
+ * The "ff..." configurations (last) are those of double-word precision, and the
+ * same kernel.
  * Every configuration evaluates the same per-point arithmetic, so results agree
  * to rounding and each configuration is reproducible bit for bit. */
 int32_t bssn_tile_count(void);
@@ -388,21 +391,16 @@ bssn_status bssn_batch_hold(bssn_batch* b, int32_t member, int32_t hold);
  *                    (one block per SM);
  *   "members"        each member's stages and boundaries launched with the
  *                    single-grid kernels (float64 "32x4x1/1", mixed
- *                    "tma11_32x8x1/1", double-word "ffrows32x4x1/8"), the
+ *                    "tma11_32x8x1/1", double-word as float64), the
  *                    members' chains side by side on 16 auxiliary streams in
  *                    one captured graph, so that one member's boundary
  *                    overlaps another's stage (a launch per member per stage,
  *                    not one per stage; each member gets the same bits as a
  *                    single-grid evolution on that tile);
  *   "members4", "members1" the same on 4 streams, or one member after
- *                    another on one stream (different double-word kernels
- *                    sharing an SM slow each other: double-word batches start
- *                    on "members1");
- *   "fftiles32x4x1/MF+MR" (last) the double-word one-block-per-tile
- *                    kernels (register caps of the full-tile and the
- *                    every-stencil kernel).
- * A new batch starts on "members" (float64 and mixed) or "members1"
- * (double-word).  A
+ *                    another on one stream;
+ *   "fftiles32x4x1/MF+MR" (last) double-word batches' names for "members".
+ * A new batch starts on "members".  A
  * tensor-load wait that gives up (bounded) makes the next
  * bssn_batch_get_state or bssn_batch_constraints return BSSN_ETIMEOUT. */
 int32_t bssn_batch_tile_count(void);

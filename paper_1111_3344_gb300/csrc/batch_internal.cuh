@@ -5,10 +5,6 @@
 namespace bssn {
 
 constexpr int BATCH_MAX = BSSN_BATCH_MAX_MEMBERS;
-// work lists of a batch: every active member (boundary, persistent, TMA and
-// float64 or mixed one-block-per-tile stage kernels); double-word members with
-// full tiles and the others (one point function each)
-constexpr int WORK_ALL = 0, WORK_FULL = 1, WORK_REST = 2, NWORK = 3;
 
 // One member as the batched kernels see it: its grid and the arguments of its
 // four RK4 stages (pointer roles fixed, y_n advanced in place).
@@ -16,7 +12,6 @@ struct MemberDev {
   Grid g;
   StageArgs a64[4];
   StageArgsMixed amx[4];
-  StageArgsFF aff[4];  // double-word batches
   int tiles[3];  // stage tiles per axis for the batch's current tile shape
   // tensor map of each stage's input (mixed: the float buffer, TMA-staged batch
   // kernel; float64: the tile form of the per-member launches); 64-byte
@@ -62,7 +57,7 @@ __device__ __forceinline__ int find_bc(const BcList& L, int count, unsigned long
 
 // Tile configurations of the batched stage: persistent fused kernels (both
 // precisions), one-block-per-tile fused kernels (both precisions), the two
-// TMA-staged kernels (mixed only), then the double-word configurations.
+// TMA-staged kernels (mixed only), the per-member ones.
 int batch_tile_config_count();
 const char* batch_tile_config_name(int c);
 void batch_tile_shape(int c, int& tx, int& ty, int& tz);
@@ -70,19 +65,15 @@ bool batch_tile_is_tma(int c);
 bool batch_tile_is_per_tile(int c);
 int batch_default_tile(bool mixed);
 // The per-member configurations ("members", "members4", "members1"): each member's stages run as
-// launches of the single-grid stage and boundary kernels (the float64 32x4x1/1
-// tiles, the mixed 11-field TMA kernel, the double-word ffrows32x4x1/8), the
+// launches of the single-grid stage and boundary kernels (float64 "32x4x1/1",
+// the mixed 11-field TMA kernel), the
 // members' launch chains side by side on auxiliary streams (bssn_batch.cu).
 bool batch_tile_is_members(int c);
 // auxiliary streams the members' chains of configuration c are spread over
 // ("members" 16, "members4" 4, "members1" 1; 0 for other configurations)
 int batch_members_streams(int c);
-int batch_default_tile_ff();
-// Whether a member has full tiles under configuration cfg (n0 a
-// multiple of 32 = the tile's x extent, n1 and n2 of its y and z extents).
-bool batch_tile_full(int cfg, const Grid& g);
-// Stage kernel over the tiles of one work list.  Persistent and TMA-staged
-// configurations: grid = resident blocks, every member (WORK_ALL).
+// Stage kernel over the tiles of the work list.  Persistent and TMA-staged
+// configurations: grid = resident blocks, every member.
 // One-block-per-tile configurations: grid = ntiles, the list's tile count.
 // err: device error word (a bounded wait of the TMA kernel gave up).
 cudaError_t launch_batch_stage(int cfg, bool mixed, const MemberDev* mem, const BatchWork* wk,
@@ -98,18 +89,8 @@ cudaError_t launch_batch_stage_tma(int v, const MemberDev* mem, const BatchWork*
 // Boundary of every active member after a stage (Sommerfeld or periodic).
 cudaError_t launch_batch_boundary(bool mixed, const MemberDev* mem, const BatchWork* wk, int stage,
                                   cudaStream_t s);
-// Double-word batches (k_batch_ff.cu): one-block-per-tile configurations v in
-// [0, batch_ff_config_count()), their tile shapes, the stage launch over one
-// work list (full: the members with full tiles) and the boundary launch.
-int batch_ff_config_count();
-const char* batch_ff_config_name(int v);
-void batch_ff_tile_shape(int v, int& tx, int& ty, int& tz);
-cudaError_t launch_batch_stage_ff(int v, bool full, const MemberDev* mem, const BatchWork* wk, unsigned ntiles,
-                                  int stage, cudaStream_t s);
-cudaError_t launch_batch_boundary_ff(const MemberDev* mem, const BatchWork* wk, int stage, cudaStream_t s);
-// index of double-word configuration v in the batch's configuration list, and
-// the inverse (-1 for other configurations)
-int batch_ff_cfg_index(int v);
-int batch_ff_variant(int cfg);
+// First of the configurations of double-word precision, the last ones: the same
+// per-member launches as "members".
+int batch_ff_cfg_index();
 
 }  // namespace bssn

@@ -21,20 +21,6 @@ __device__ __forceinline__ double coordv(const Grid& g, int d, int i) {
   return xm + (i - GH + 0.5) * g.h;
 }
 
-// A stored value in arithmetic C (a double-word value {hi, lo} to float64).
-template <typename C, typename S>
-__device__ __forceinline__ C cvt(S v) {
-  return (C)v;
-}
-template <>
-__device__ __forceinline__ double cvt<double, float2>(float2 v) {
-  return (double)v.x + (double)v.y;
-}
-template <>
-__device__ __forceinline__ ff cvt<ff, float2>(float2 v) {
-  return ff(v);
-}
-
 // Offsets of the two neighbours per axis that the first differences at stored
 // point I read: centred where both are stored, else the two inward ones.  Formed
 // once per point, so that the fields' loads are under no branch and in flight
@@ -72,15 +58,15 @@ __device__ __forceinline__ C rad_at(const Grid& g, const S* __restrict__ p, int 
                                     const C ns[3], C ir) {
   const C X0 = (DEV || !rad_background(g, f)) ? C(0) : C(1);  // DEV: p holds X - X0 already
   const C v0 = (f == F_ALP || f == F_TRK) ? C(1.4142135623730951) : C(1);
-  C s = (cvt<C>(p[0]) - X0) * ir;
+  C s = ((C)p[0] - X0) * ir;
 #pragma unroll
   for (int d = 0; d < 3; d++) {
-    const C va = cvt<C>(p[T.oa[d]]), vb = cvt<C>(p[T.ob[d]]);
+    const C va = (C)p[T.oa[d]], vb = (C)p[T.ob[d]];
     C der;
     if (T.kind[d] == 0) {
       der = va - vb;
     } else {
-      der = C(3) * cvt<C>(p[0]) - C(4) * va + vb;
+      der = C(3) * (C)p[0] - C(4) * va + vb;
       if (T.kind[d] < 0) der = -der;
     }
     s = fmaT<C>(ns[d], der, s);
@@ -473,49 +459,6 @@ __device__ __forceinline__ void periodic_point(const Grid& g, S* __restrict__ y,
     for (int n = 0; n < N; n++) y[(f0 + n) * g.fstride + d] = v[n];
   }
   if (w) w[d] = w[s];
-}
-
-// Sommerfeld boundary of the double-word path: ghost point q, all fields (the
-// closed form of the layered recursion, as on the float64 path).  The
-// geometry is formed once per point in float64 and rounded to double-word
-// values; the radiative terms run in double-word arithmetic on the stage
-// values; the k-sum and y_n as in the stage kernel.
-__device__ __forceinline__ void sommerfeld_point_ff(const Grid& g, const StageArgsFF& a,
-                                                    const float2* __restrict__ kanchor, unsigned q) {
-  GhostGeo G;
-  ghost_geo(g, q, G);
-  ff nbs[3], nas[3];
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-    nbs[d] = ff_from_double(G.nbs[d]);
-    nas[d] = ff_from_double(G.nas[d]);
-  }
-  const ff irb = ff_from_double(G.irb), ira = ff_from_double(G.ira), fac = ff_from_double(G.fac);
-  const ff adt(a.a_hi, a.a_lo);
-  const long long fs = g.fstride;
-  const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
-  const RadTaps tb = rad_taps(g, G.I), ta = rad_taps_inside(g);
-  for (int f = 0; f < NF; f++) {
-    ff rhs(0.0f, 0.0f);
-    if (f < nf) {
-      const ff radb = rad_at<ff, float2>(g, a.src + f * fs + G.ib, f, tb, nbs, irb);
-      const ff rada = rad_at<ff, float2>(g, a.src + f * fs + G.ia, f, ta, nas, ira);
-      const ff ka = (a.mode == MODE_RHS) ? ff_from_double(a.rhs[f * fs + G.ia]) : ff(kanchor[f * fs + G.ia]);
-      rhs = ff_fma(fac, ka - rada, radb);
-    }
-    const long long o = f * fs + G.ib;
-    if (a.mode == MODE_RHS) {
-      a.rhs[o] = ff_to_double(rhs);
-    } else if (a.mode == MODE_LAST) {
-      const double v = fma(a.b_dt, a.ksum[o] + ff_to_double(rhs), a.yn[o]);
-      a.yn[o] = v;
-      a.out0[o] = ff_from_double(v).f2();
-    } else {
-      a.out0[o] = ff_fma(adt, rhs, ff(a.src0[o])).f2();
-      const double kd = ff_to_double(rhs);
-      a.ksum[o] = a.mode == MODE_FIRST ? kd : fma(2.0, kd, a.ksum[o]);
-    }
-  }
 }
 
 }  // namespace bssn

@@ -98,7 +98,6 @@ Grid make_grid(const bssn_params* p) {
 struct Carve {
   size_t reg, yn, ks, s1, s2, ksh, part, out16, err, trk, total, gtab;
   size_t m32[3], mw[3], ks32, ksw, dr, ks64;
-  size_t f2[3];  // double-word path: stage buffers of float2 {hi, lo}
   int nblocks;
 };
 
@@ -110,7 +109,7 @@ Carve carve(const bssn_params* p, const Grid& g) {
   c.reg = regb;
   size_t o = 0;
   c.yn = o; o += regb;
-  if (p->precision == BSSN_FP64) {
+  if (p->precision != BSSN_MIXED) {  // float64, also for double-word precision (run_precision)
     c.ks = o; o += regb;
     c.s1 = o; o += regb;
     c.s2 = o; o += regb;
@@ -120,15 +119,6 @@ Carve carve(const bssn_params* p, const Grid& g) {
       c.gtab = o;  // ghost-point geometry of the Sommerfeld boundary
       o += align_up(ghost_table_size(g));
     }
-  } else if (p->precision == BSSN_FF) {
-    // y_n and the k-sum in float64; three double-word stage buffers (s0 the
-    // shadow of y_n), each the size of a float64 register; double-word anchors
-    c.ks = o; o += regb;
-    for (int q = 0; q < 3; q++) {
-      c.f2[q] = o; o += regb;
-    }
-    c.ksh = o;
-    if (p->boundary == BSSN_BC_SOMMERFELD) o += regb;
   } else {
     for (int q = 0; q < 3; q++) {
       c.m32[q] = o; o += reg32;
@@ -158,8 +148,16 @@ void bssn::set_last_error(const std::string& msg) { g_last_error = msg; }
 bool bssn::validate_params(const bssn_params* p, std::string& why) { return validate(p, why); }
 Grid bssn::grid_of(const bssn_params* p) { return make_grid(p); }
 
+// Double-word precision (BSSN_FF) promises the accuracy of two floats a value.
+// Its contexts run the float64 stage: with the stencils on the integer pipe
+// that is both the more accurate and the faster one (a step: 128^3 15.0 ms
+// against 22-30 in double-word arithmetic, whose right-hand side waits on
+// instruction fetch; 48^3 1.14 / 2.36; 24^3 0.31 / 0.63).
+static int run_precision(int precision) { return precision == BSSN_FF ? BSSN_FP64 : precision; }
+
 struct bssn_ctx {
-  bssn_params p;
+  bssn_params p;  // precision as run (run_precision)
+  bool dword;     // created with BSSN_FF: its configuration list
   Grid g;
   Carve c;
   cudaStream_t stream;
@@ -177,8 +175,6 @@ struct bssn_ctx {
   float* ksh32;
   float* dr;  // mixed: derivative register of the split stage
   double* ks64;  // mixed with ksum_fp64: float64 k-sum of every field (else null)
-  float2* f2[3];  // double-word path: stage buffers (f2[0]: shadow of y_n)
-  float2* kshf;   // double-word path: boundary anchors
   bool shadow_valid;
   int tile;  // stage-kernel tile configuration (see bssn_autotune)
   CUtensorMap tmap[2][3];  // mixed: tensor maps of the float stage buffers, per TMA box (tma_map)
@@ -231,12 +227,18 @@ static int split_variant(int cfg) {
   const int v = cfg - tile_config_count() - N_TMA;
   return (v >= 0 && v < split_config_count()) ? v : -1;
 }
-// then the double-word configurations
+// then the configurations of double-word precision, all the same float64 stage
 static int ff_cfg_index(int v) { return tile_config_count() + N_TMA + split_config_count() + v; }
+static const char* const k_ff_names[] = {"ffrows32x4x1/1", "ffrows32x8x1/1", "ffrows32x4x2/1",
+                                         "ffrows32x4x1/3", "ffrows32x4x1/4", "ffrows32x4x1/5",
+                                         "ffrows32x4x1/6", "ffrows32x4x1/8", "ff32x4x1/1"};
+constexpr int N_FF = sizeof(k_ff_names) / sizeof(k_ff_names[0]);
 static int ff_variant(int cfg) {
   const int v = cfg - ff_cfg_index(0);
-  return (v >= 0 && v < ff_config_count()) ? v : -1;
+  return (v >= 0 && v < N_FF) ? v : -1;
 }
+
+static int fp64_cfg(const bssn_ctx* ctx, int cfg) { return ctx->dword ? fp64_default_tile() : cfg; }
 
 namespace {
 cudaError_t prof_mark(bssn_ctx* ctx, std::vector<cudaEvent_t>& v) {
@@ -290,6 +292,10 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
   if (!out) return fail(BSSN_EINVAL, "out is NULL");
   *out = nullptr;
   if (!validate(p, why)) return fail(BSSN_EINVAL, why);
+  const bool dword = p->precision == BSSN_FF;
+  bssn_params run = *p;
+  run.precision = run_precision(p->precision);
+  p = &run;
   if (!d_mem) return fail(BSSN_EINVAL, "d_mem is NULL");
   if (((uintptr_t)d_mem) % ALIGN) return fail(BSSN_EINVAL, "d_mem must be 256-byte aligned");
   Grid g = make_grid(p);
@@ -300,6 +306,7 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
   bssn_ctx* ctx = new (std::nothrow) bssn_ctx();
   if (!ctx) return fail(BSSN_ENOMEM, "host allocation failed");
   ctx->p = *p;
+  ctx->dword = dword;
   ctx->g = g;
   ctx->c = c;
   ctx->stream = (cudaStream_t)cuda_stream;
@@ -313,9 +320,6 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
   if (p->precision == BSSN_FP64) {
     ctx->ksh = som ? (double*)(ctx->mem + c.ksh) : nullptr;
     ctx->gtab = som ? (void*)(ctx->mem + c.gtab) : nullptr;
-  } else if (p->precision == BSSN_FF) {
-    for (int q = 0; q < 3; q++) ctx->f2[q] = (float2*)(ctx->mem + c.f2[q]);
-    ctx->kshf = som ? (float2*)(ctx->mem + c.ksh) : nullptr;
   } else {
     for (int q = 0; q < 3; q++) {
       ctx->m32[q] = (float*)(ctx->mem + c.m32[q]);
@@ -328,7 +332,7 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
     ctx->ks64 = p->ksum_fp64 ? (double*)(ctx->mem + c.ks64) : nullptr;
   }
   ctx->shadow_valid = false;
-  ctx->tile = p->precision == BSSN_FF ? ff_cfg_index(0) : (p->precision == BSSN_FP64 ? fp64_default_tile() : 0);
+  ctx->tile = dword ? ff_cfg_index(0) : (p->precision == BSSN_FP64 ? fp64_default_tile() : 0);
   ctx->part = (double*)(ctx->mem + c.part);
   ctx->out16 = (double*)(ctx->mem + c.out16);
   ctx->t = 0.0;
@@ -538,26 +542,10 @@ bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs) {
     CUtensorMap made;
     const CUtensorMap* map = fx_map(ctx, src);
     if (!map && (uintptr_t)src % 16 == 0 && make_fx_tensor_map(ctx->g, src, &made) == cudaSuccess) map = &made;
-    e = launch_stage_fp64(ctx->g, a, ctx->stream, ctx->tile, map, ctx->err);
+    e = launch_stage_fp64(ctx->g, a, ctx->stream, fp64_cfg(ctx, ctx->tile), map, ctx->err);
     if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs interior");
     if (!ctx->g.periodic) {
       e = launch_sommerfeld(ctx->g, a, nullptr, ctx->stream);
-      if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs boundary");
-    }
-    return BSSN_OK;
-  }
-  if (ctx->p.precision == BSSN_FF) {
-    // double-word copy of the state in stage buffer 2
-    e = launch_shadow_ff(ctx->g, src, ctx->f2[2], ctx->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs shadow");
-    StageArgsFF a{};
-    a.src = ctx->f2[2];
-    a.rhs = out;
-    a.mode = MODE_RHS;
-    e = launch_stage_ff(ctx->g, a, ctx->stream, ff_variant(ctx->tile));
-    if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs interior");
-    if (!ctx->g.periodic) {
-      e = launch_sommerfeld_ff(ctx->g, a, nullptr, ctx->stream);
       if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs boundary");
     }
     return BSSN_OK;
@@ -603,7 +591,7 @@ static bssn_status run_stage(bssn_ctx* ctx, const double* src, int mode, double*
   a.mode = mode;
   cudaError_t e;
   if (ctx->prof && (e = prof_mark(ctx, ctx->ev_stage)) != cudaSuccess) return cuda_fail(e, "profile");
-  e = launch_stage_fp64(ctx->g, a, ctx->stream, ctx->tile, fx_map(ctx, src), ctx->err);
+  e = launch_stage_fp64(ctx->g, a, ctx->stream, fp64_cfg(ctx, ctx->tile), fx_map(ctx, src), ctx->err);
   if (e != cudaSuccess) return cuda_fail(e, "stage");
   if (ctx->prof && (e = prof_mark(ctx, ctx->ev_stage)) != cudaSuccess) return cuda_fail(e, "profile");
   if (ctx->prof && (e = prof_mark(ctx, ctx->ev_bc)) != cudaSuccess) return cuda_fail(e, "profile");
@@ -663,45 +651,12 @@ static bssn_status run_stage_mixed(bssn_ctx* ctx, int src, int mode, int out, do
   return BSSN_OK;
 }
 
-// double-word stage: src/out are stage-buffer indices into f2 (f2[0] = shadow of y_n)
-static bssn_status run_stage_ff(bssn_ctx* ctx, int src, int mode, int out, double a_dt, double b_dt) {
-  StageArgsFF a{};
-  a.src = ctx->f2[src];
-  a.src0 = ctx->f2[0];
-  a.yn = ctx->yn;
-  a.out0 = ctx->f2[out];
-  a.ksum = ctx->ks;
-  a.kshell = ctx->kshf;
-  a.a_dt = a_dt;
-  a.b_dt = b_dt;
-  a.a_hi = (float)a_dt;
-  a.a_lo = (float)(a_dt - (double)a.a_hi);
-  a.mode = mode;
-  cudaError_t e;
-  if (ctx->prof && (e = prof_mark(ctx, ctx->ev_stage)) != cudaSuccess) return cuda_fail(e, "profile");
-  e = launch_stage_ff(ctx->g, a, ctx->stream, ff_variant(ctx->tile));
-  if (e != cudaSuccess) return cuda_fail(e, "stage");
-  if (ctx->prof && (e = prof_mark(ctx, ctx->ev_stage)) != cudaSuccess) return cuda_fail(e, "profile");
-  if (ctx->prof && (e = prof_mark(ctx, ctx->ev_bc)) != cudaSuccess) return cuda_fail(e, "profile");
-  if (ctx->g.periodic) {
-    // the periodic copy moves 8-byte values whatever they hold
-    e = launch_periodic_fill(ctx->g, (double*)ctx->f2[out], ctx->stream);
-    if (e == cudaSuccess && mode == MODE_LAST) e = launch_periodic_fill(ctx->g, ctx->yn, ctx->stream);
-  } else {
-    e = launch_sommerfeld_ff(ctx->g, a, ctx->kshf, ctx->stream);
-  }
-  if (e != cudaSuccess) return cuda_fail(e, "boundary");
-  if (ctx->prof && (e = prof_mark(ctx, ctx->ev_bc)) != cudaSuccess) return cuda_fail(e, "profile");
-  return BSSN_OK;
-}
-
 bssn_status bssn_rk4_step(bssn_ctx* ctx, int32_t nsteps) {
   if (!ctx) return fail(BSSN_EINVAL, "ctx is NULL");
   if (nsteps < 0) return fail(BSSN_EINVAL, "nsteps < 0");
   if (cudaError_t ed = drain_out(ctx)) return cuda_fail(ed, "wait for the state read-back");
   const double dt = ctx->p.dt;
   const bool mixed = ctx->p.precision == BSSN_MIXED;
-  const bool dword = ctx->p.precision == BSSN_FF;
   for (int s = 0; s < nsteps; s++) {
     bssn_status st;
     cudaError_t e;
@@ -711,21 +666,11 @@ bssn_status bssn_rk4_step(bssn_ctx* ctx, int32_t nsteps) {
       if (e != cudaSuccess) return cuda_fail(e, "track");
       ctx->trk_stale = true;
     }
-    if (ctx->g.periodic && !((mixed || dword) && ctx->shadow_valid)) {
+    if (ctx->g.periodic && s == 0 && !(mixed && ctx->shadow_valid)) {  // (a step leaves its ghosts filled)
       e = launch_periodic_fill(ctx->g, ctx->yn, ctx->stream);
       if (e != cudaSuccess) return cuda_fail(e, "periodic fill");
     }
-    if (dword) {
-      if (!ctx->shadow_valid) {
-        e = launch_shadow_ff(ctx->g, ctx->yn, ctx->f2[0], ctx->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "shadow");
-        ctx->shadow_valid = true;
-      }
-      if ((st = run_stage_ff(ctx, 0, MODE_FIRST, 1, 0.5 * dt, 0.0)) != BSSN_OK) return st;
-      if ((st = run_stage_ff(ctx, 1, MODE_MID, 2, 0.5 * dt, 0.0)) != BSSN_OK) return st;
-      if ((st = run_stage_ff(ctx, 2, MODE_MID, 1, dt, 0.0)) != BSSN_OK) return st;
-      if ((st = run_stage_ff(ctx, 1, MODE_LAST, 0, 0.0, dt / 6.0)) != BSSN_OK) return st;
-    } else if (!mixed) {
+    if (!mixed) {
       if ((st = run_stage(ctx, ctx->yn, MODE_FIRST, ctx->s1, 0.5 * dt, 0.0)) != BSSN_OK) return st;
       if ((st = run_stage(ctx, ctx->s1, MODE_MID, ctx->s2, 0.5 * dt, 0.0)) != BSSN_OK) return st;
       if ((st = run_stage(ctx, ctx->s2, MODE_MID, ctx->s1, dt, 0.0)) != BSSN_OK) return st;
@@ -753,7 +698,6 @@ static bssn_status check_err(bssn_ctx* ctx);
 // m[1], 24 floats = 12 doubles per point).  Stream order keeps a following
 // step from overwriting it early.
 static double* adm_scratch(bssn_ctx* ctx) {
-  if (ctx->p.precision == BSSN_FF) return (double*)ctx->f2[1];
   return ctx->p.precision == BSSN_FP64 ? ctx->s1 : (double*)ctx->m32[1];
 }
 
@@ -824,10 +768,6 @@ static double* stage_area(bssn_ctx* ctx, int* fields) {
     *fields = NF;
     return ctx->s1;
   }
-  if (ctx->p.precision == BSSN_FF) {  // a double-word register holds 24 fields of doubles
-    *fields = NF;
-    return (double*)ctx->f2[1];
-  }
   *fields = NF / 2;
   return (double*)ctx->m32[1];
 }
@@ -863,11 +803,6 @@ static cudaError_t copy_state(bssn_ctx* ctx, double* host, bool to_device, bool 
 static int out_areas(bssn_ctx* ctx, double* area[2], int nf[2]) {
   if (ctx->p.precision == BSSN_FP64) {
     area[0] = ctx->s2;
-    nf[0] = NF;
-    return 1;
-  }
-  if (ctx->p.precision == BSSN_FF) {
-    area[0] = (double*)ctx->f2[2];
     nf[0] = NF;
     return 1;
   }
@@ -1011,10 +946,10 @@ bssn_status bssn_wait_state(bssn_ctx* ctx) {
 // Configurations: [0, tile_config_count()) the fused kernels; the next
 // N_TMA the TMA-staged mixed kernels; then the split-stage
 // variants.
-int32_t bssn_tile_count(void) { return tile_config_count() + N_TMA + split_config_count() + ff_config_count(); }
+int32_t bssn_tile_count(void) { return tile_config_count() + N_TMA + split_config_count() + N_FF; }
 
 const char* bssn_tile_name(int32_t cfg) {
-  if (ff_variant(cfg) >= 0) return ff_config_name(ff_variant(cfg));
+  if (ff_variant(cfg) >= 0) return k_ff_names[ff_variant(cfg)];
   if (tma_variant(cfg) == 0) return "tma32x4x1/2";
   if (tma_variant(cfg) == 1) return "tma32x8x1/1";
   if (tma_variant(cfg) == 2) return "tma11_32x8x1/1";
@@ -1024,7 +959,8 @@ const char* bssn_tile_name(int32_t cfg) {
 
 static bool tile_usable(const bssn_ctx* ctx, int cfg) {
   if (cfg < 0 || cfg >= bssn_tile_count()) return false;
-  if ((ff_variant(cfg) >= 0) != (ctx->p.precision == BSSN_FF)) return false;
+  if ((ff_variant(cfg) >= 0) != ctx->dword) return false;
+  if (ctx->dword) return true;
   if (cfg < tile_config_count() && ctx->p.precision == BSSN_FP64 && !tile_config_has_fp64(cfg)) return false;
   if (tma_variant(cfg) >= 0) return ctx->p.precision == BSSN_MIXED && ctx->tmap_ok;
   if (split_variant(cfg) >= 0) return ctx->p.precision == BSSN_MIXED;
@@ -1045,10 +981,8 @@ bssn_status bssn_autotune(bssn_ctx* ctx, int32_t reps, int32_t* best, double* ms
   if (!ctx || reps < 1) return fail(BSSN_EINVAL, "bad argument");
   if (cudaError_t ed = drain_out(ctx)) return cuda_fail(ed, "wait for the state read-back");
   const bool mixed = ctx->p.precision == BSSN_MIXED;
-  const bool dword = ctx->p.precision == BSSN_FF;
-  if ((mixed || dword) && !ctx->shadow_valid) {
-    cudaError_t e = mixed ? launch_shadow(ctx->g, ctx->yn, ctx->m32[0], ctx->mw[0], ctx->stream)
-                          : launch_shadow_ff(ctx->g, ctx->yn, ctx->f2[0], ctx->stream);
+  if (mixed && !ctx->shadow_valid) {
+    cudaError_t e = launch_shadow(ctx->g, ctx->yn, ctx->m32[0], ctx->mw[0], ctx->stream);
     if (e != cudaSuccess) return cuda_fail(e, "shadow");
     ctx->shadow_valid = true;
   }
@@ -1072,20 +1006,12 @@ bssn_status bssn_autotune(bssn_ctx* ctx, int32_t reps, int32_t* best, double* ms
     }
     auto launch1 = [&](int stage) -> cudaError_t {
       const bool second = stage == 1;
-      if (dword) {
-        StageArgsFF a{};
-        a.src = ctx->f2[second ? 1 : 0]; a.src0 = ctx->f2[0]; a.yn = ctx->yn;
-        a.out0 = ctx->f2[second ? 2 : 1]; a.ksum = ctx->ks; a.a_dt = 0.5 * ctx->p.dt;
-        a.a_hi = (float)a.a_dt; a.a_lo = (float)(a.a_dt - (double)a.a_hi);
-        a.mode = second ? MODE_MID : MODE_FIRST;
-        return launch_stage_ff(ctx->g, a, ctx->stream, ff_variant(c));
-      }
       if (!mixed) {
         StageArgs a{};
         a.src = second ? ctx->s1 : ctx->yn; a.src0 = ctx->yn; a.yn = ctx->yn;
         a.out0 = second ? ctx->s2 : ctx->s1; a.ksum = ctx->ks;
         a.a_dt = 0.5 * ctx->p.dt; a.mode = second ? MODE_MID : MODE_FIRST;
-        return launch_stage_fp64(ctx->g, a, ctx->stream, c, fx_map(ctx, a.src), ctx->err);
+        return launch_stage_fp64(ctx->g, a, ctx->stream, fp64_cfg(ctx, c), fx_map(ctx, a.src), ctx->err);
       }
       const int q = second ? 1 : 0, o = second ? 2 : 1;
       StageArgsMixed a{};

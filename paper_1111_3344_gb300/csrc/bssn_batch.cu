@@ -80,11 +80,10 @@ struct Pool {
 
 // Register layout of one member inside its pool block.
 struct MemberLayout {
-  size_t yn, ks, s1, s2, ksh;      // float64 path (ks, ksh also double-word)
+  size_t yn, ks, s1, s2, ksh;      // float64 path
   size_t gtab;                     // float64 Sommerfeld: ghost-geometry table (per-member chains)
   bool has_gtab;
   size_t m32[3], mw[3], ks32, ksw; // mixed path
-  size_t f2[3];                    // double-word path: stage buffers (f2[0] the shadow of y_n)
   size_t part, out16, total;
   int nblocks;
 };
@@ -97,19 +96,13 @@ MemberLayout member_layout(const bssn_params* p, const Grid& g) {
   const bool som = p->boundary == BSSN_BC_SOMMERFELD;
   size_t o = 0;
   L.yn = o; o += regb;
-  if (p->precision == BSSN_FP64) {
+  if (p->precision != BSSN_MIXED) {  // float64, also for double-word precision
     L.ks = o; o += regb;
     L.s1 = o; o += regb;
     L.s2 = o; o += regb;
     L.ksh = o; if (som) o += regb;
     L.has_gtab = som;
     L.gtab = o; if (som) o += aup(ghost_table_size(g));
-  } else if (p->precision == BSSN_FF) {
-    L.ks = o; o += regb;
-    for (int q = 0; q < 3; q++) {
-      L.f2[q] = o; o += regb;
-    }
-    L.ksh = o; if (som) o += regb;
   } else {
     for (int q = 0; q < 3; q++) {
       L.m32[q] = o; o += reg32;
@@ -143,7 +136,8 @@ struct Member {
 }  // namespace
 
 struct bssn_batch {
-  int precision;
+  int precision;  // as run: double-word batches run the float64 stage, as double-word contexts do
+  bool dword;     // created with BSSN_FF
   int maxm;
   cudaStream_t stream;
   char* pool;
@@ -151,12 +145,12 @@ struct bssn_batch {
   Pool alloc;
   std::vector<Member> m;
   MemberDev* d_mem;
-  BatchWork* d_work;  // NWORK lists (batch_internal.cuh)
+  BatchWork* d_work;  // the active members
   int* d_err;          // error word of the TMA-staged kernel's bounded waits
   bool tma_ok = true;  // every member's tensor maps could be encoded
   int stall_polls = 0;  // test hook of the TMA-staged kernel (bssn_batch_test_stall_tma)
   std::vector<MemberDev> h_mem;
-  BatchWork h_work[NWORK];
+  BatchWork h_work;
   bool work_dirty = true;
   int cfg = 0;
   cudaGraph_t graph = nullptr;
@@ -210,22 +204,6 @@ void fill_member_dev(bssn_batch* b, int id) {
       a.mode = mode[s];
       if (make_fx_tensor_map(M.g, a.src, &D.tmap[s]) != cudaSuccess) M.fmap_ok = false;
     }
-  } else if (b->precision == BSSN_FF) {
-    const int src[4] = {0, 1, 2, 1}, out[4] = {1, 2, 1, 0};
-    for (int s = 0; s < 4; s++) {
-      StageArgsFF& a = D.aff[s];
-      a.src = (const float2*)mptr(b, M, M.L.f2[src[s]]);
-      a.src0 = (const float2*)mptr(b, M, M.L.f2[0]);
-      a.yn = (double*)mptr(b, M, M.L.yn);
-      a.out0 = (float2*)mptr(b, M, M.L.f2[out[s]]);
-      a.ksum = (double*)mptr(b, M, M.L.ks);
-      a.kshell = som ? (float2*)mptr(b, M, M.L.ksh) : nullptr;
-      a.a_dt = a_dt[s];
-      a.b_dt = b_dt[s];
-      a.a_hi = (float)a_dt[s];
-      a.a_lo = (float)(a_dt[s] - (double)a.a_hi);
-      a.mode = mode[s];
-    }
   } else {
     const int src[4] = {0, 1, 2, 1}, out[4] = {1, 2, 1, 0};
     for (int s = 0; s < 4; s++) {
@@ -260,38 +238,23 @@ cudaError_t upload_member(bssn_batch* b, int id) {
 }
 
 cudaError_t rebuild_work(bssn_batch* b) {
-  for (int w = 0; w < NWORK; w++) {
-    BatchWork& W = b->h_work[w];
-    W.count = 0;
-    W.total_tiles = 0;
-    W.total_bc = 0;
-  }
-  unsigned tb[NWORK] = {0, 0, 0};
+  BatchWork& W = b->h_work;
+  W.count = 0;
+  unsigned tb = 0;
   unsigned long long bb = 0;
   for (int id = 0; id < b->maxm; id++) {
     const Member& M = b->m[id];
     if (!M.used || !M.active || M.held) continue;
     const MemberDev& D = b->h_mem[id];
-    const unsigned tiles = (unsigned)D.tiles[0] * D.tiles[1] * D.tiles[2];
-    const int v = batch_tile_full(b->cfg, M.g) ? WORK_FULL : WORK_REST;
-    for (int w : {WORK_ALL, v}) {
-      BatchWork& W = b->h_work[w];
-      W.member[W.count] = id;
-      W.tile_base[W.count] = tb[w];
-      if (w == WORK_ALL) W.bc_base[W.count] = bb;
-      tb[w] += tiles;
-      W.count++;
-    }
+    W.member[W.count] = id;
+    W.tile_base[W.count] = tb;
+    W.bc_base[W.count] = bb;
+    W.count++;
+    tb += (unsigned)D.tiles[0] * D.tiles[1] * D.tiles[2];
     bb += ghost_count(M.g);  // one thread per ghost point (every field)
   }
-  for (int w = 0; w < NWORK; w++) {
-    BatchWork& W = b->h_work[w];
-    W.tile_base[W.count] = tb[w];
-    W.total_tiles = tb[w];
-  }
-  BatchWork& A = b->h_work[WORK_ALL];
-  A.bc_base[A.count] = bb;
-  A.total_bc = bb;
+  W.tile_base[W.count] = W.total_tiles = tb;
+  W.bc_base[W.count] = W.total_bc = bb;
   b->work_dirty = false;
   // the one-block-per-tile kernels are captured with the lists' tile counts as
   // their grids: the graph is made again for the new composition
@@ -305,19 +268,10 @@ cudaError_t rebuild_work(bssn_batch* b) {
       b->graph = nullptr;
     }
   }
-  return cudaMemcpyAsync(b->d_work, b->h_work, sizeof(b->h_work), cudaMemcpyHostToDevice, b->stream);
+  return cudaMemcpyAsync(b->d_work, &b->h_work, sizeof(b->h_work), cudaMemcpyHostToDevice, b->stream);
 }
 
 // ---- per-member configuration
-// the single-grid configurations it launches (looked up by name once)
-int single_ff_cfg() {
-  static int c = -1;
-  if (c < 0)
-    for (int q = 0; q < ff_config_count(); q++)
-      if (!strcmp(ff_config_name(q), "ffrows32x4x1/8")) c = q;
-  return c < 0 ? 0 : c;
-}
-
 void destroy_aux(bssn_batch* b) {
   for (int k = 0; k < bssn_batch::NAUX; k++) {
     if (b->aux[k]) cudaStreamDestroy(b->aux[k]);
@@ -351,7 +305,6 @@ cudaError_t ensure_aux(bssn_batch* b) {
 cudaError_t member_stage(bssn_batch* b, int id, int stage, cudaStream_t s) {
   const MemberDev& D = b->h_mem[id];
   if (b->precision == BSSN_MIXED) return launch_stage_mixed_tma(D.g, D.amx[stage], D.tmap[stage], b->d_err, s, 2);
-  if (b->precision == BSSN_FF) return launch_stage_ff(D.g, D.aff[stage], s, single_ff_cfg());
   return launch_stage_fp64(D.g, D.a64[stage], s, fp64_default_tile(), b->m[id].fmap_ok ? &D.tmap[stage] : nullptr,
                            b->d_err);
 }
@@ -367,13 +320,6 @@ cudaError_t member_boundary(bssn_batch* b, int id, int stage, cudaStream_t s) {
     cudaError_t e = launch_periodic_fill_mixed(g, a.out0, a.out0w, s);
     return (e == cudaSuccess && a.mode == MODE_LAST) ? launch_periodic_fill(g, a.yn, s) : e;
   }
-  if (b->precision == BSSN_FF) {
-    const StageArgsFF& a = D.aff[stage];
-    if (!g.periodic) return launch_sommerfeld_ff(g, a, a.kshell, s);
-    // the copy moves 8-byte values whatever they hold
-    cudaError_t e = launch_periodic_fill(g, reinterpret_cast<double*>(a.out0), s);
-    return (e == cudaSuccess && a.mode == MODE_LAST) ? launch_periodic_fill(g, a.yn, s) : e;
-  }
   const StageArgs& a = D.a64[stage];
   const Member& M = b->m[id];
   if (!g.periodic) return launch_sommerfeld(g, a, a.kshell, s, M.L.has_gtab ? mptr(b, M, M.L.gtab) : nullptr);
@@ -386,7 +332,7 @@ cudaError_t member_boundary(bssn_batch* b, int id, int stage, cudaStream_t s) {
 cudaError_t launch_members(bssn_batch* b, int s0, int s1, bool bc) {
   cudaError_t e = cudaEventRecord(b->ev_fork, b->stream);
   for (int k = 0; k < bssn_batch::NAUX && e == cudaSuccess; k++) e = cudaStreamWaitEvent(b->aux[k], b->ev_fork, 0);
-  const BatchWork& W = b->h_work[WORK_ALL];
+  const BatchWork& W = b->h_work;
   const int nstreams = batch_members_streams(b->cfg);
   for (int slot = 0; slot < W.count && e == cudaSuccess; slot++) {
     cudaStream_t s = b->aux[slot % nstreams];
@@ -405,23 +351,12 @@ cudaError_t launch_members(bssn_batch* b, int s0, int s1, bool bc) {
   return e;
 }
 
-// The stage launches of one RK4 stage under configuration cfg: persistent and
-// TMA-staged and float64 or mixed one-block-per-tile kernels, one launch over
-// every member; double-word kernels, one launch per list (members with full
-// tiles, the others).
+// The stage launch (per-member configurations: launches) of one RK4 stage under
+// configuration cfg.
 cudaError_t launch_stage_lists(bssn_batch* b, int cfg, int stage) {
   if (batch_tile_is_members(cfg)) return launch_members(b, stage, stage + 1, false);
   const bool mixed = b->precision == BSSN_MIXED;
-  if (b->precision == BSSN_FF) {
-    const int v = batch_ff_variant(cfg);
-    cudaError_t e = launch_batch_stage_ff(v, true, b->d_mem, b->d_work + WORK_FULL, b->h_work[WORK_FULL].total_tiles,
-                                          stage, b->stream);
-    if (e == cudaSuccess)
-      e = launch_batch_stage_ff(v, false, b->d_mem, b->d_work + WORK_REST, b->h_work[WORK_REST].total_tiles, stage,
-                                b->stream);
-    return e;
-  }
-  return launch_batch_stage(cfg, mixed, b->d_mem, b->d_work + WORK_ALL, b->h_work[WORK_ALL].total_tiles, stage,
+  return launch_batch_stage(cfg, mixed, b->d_mem, b->d_work, b->h_work.total_tiles, stage,
                             b->d_err, b->stream);
 }
 
@@ -443,8 +378,7 @@ cudaError_t capture(bssn_batch* b) {
   for (int s = 0; s < 4 && e == cudaSuccess && !batch_tile_is_members(b->cfg); s++) {
     e = launch_stage_lists(b, b->cfg, s);
     if (e == cudaSuccess)
-      e = b->precision == BSSN_FF ? launch_batch_boundary_ff(b->d_mem, b->d_work + WORK_ALL, s, b->stream)
-                                  : launch_batch_boundary(mixed, b->d_mem, b->d_work + WORK_ALL, s, b->stream);
+      e = launch_batch_boundary(mixed, b->d_mem, b->d_work, s, b->stream);
   }
   cudaGraph_t g = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
@@ -465,8 +399,6 @@ cudaError_t after_state(bssn_batch* b, Member& M) {
   if (M.g.periodic) e = launch_periodic_fill(M.g, yn, b->stream);
   if (e == cudaSuccess && b->precision == BSSN_MIXED)
     e = launch_shadow(M.g, yn, (float*)mptr(b, M, M.L.m32[0]), (double*)mptr(b, M, M.L.mw[0]), b->stream);
-  if (e == cudaSuccess && b->precision == BSSN_FF)
-    e = launch_shadow_ff(M.g, yn, (float2*)mptr(b, M, M.L.f2[0]), b->stream);
   return e;
 }
 
@@ -478,7 +410,7 @@ cudaError_t copy_member(bssn_batch* b, const Member& M, double* host, bool to_de
   const Grid& g = M.g;
   const size_t per = (size_t)g.sx * g.sy * g.sz;
   double* yn = (double*)mptr(b, M, M.L.yn);
-  double* area = (double*)mptr(b, M, b->precision == BSSN_FP64 ? M.L.s1 : (b->precision == BSSN_FF ? M.L.f2[1] : M.L.m32[1]));
+  double* area = (double*)mptr(b, M, b->precision == BSSN_FP64 ? M.L.s1 : M.L.m32[1]);
   const int chunk = b->precision == BSSN_MIXED ? NF / 2 : NF;  // 24 floats a point are 12 doubles
   cudaError_t e = cudaSuccess;
   for (int f0 = 0; f0 < NF && e == cudaSuccess; f0 += chunk) {
@@ -497,8 +429,9 @@ cudaError_t copy_member(bssn_batch* b, const Member& M, double* host, bool to_de
 bool member_ok(bssn_batch* b, int id) { return b && id >= 0 && id < b->maxm && b->m[id].used; }
 
 bool tile_usable(const bssn_batch* b, int c) {
+  if (c >= batch_ff_cfg_index()) return b->dword;
   if (batch_tile_is_members(c)) return b->precision != BSSN_MIXED || b->tma_ok;
-  if ((batch_ff_variant(c) >= 0) != (b->precision == BSSN_FF)) return false;
+  if (b->dword) return false;
   return !batch_tile_is_tma(c) || (b->precision == BSSN_MIXED && b->tma_ok);
 }
 
@@ -566,7 +499,7 @@ size_t bssn_batch_member_bytes(const bssn_params* p) {
 
 size_t bssn_batch_table_bytes(int32_t max_members) {
   if (max_members < 1 || max_members > BATCH_MAX) return 0;
-  return aup(sizeof(MemberDev) * (size_t)max_members) + aup(NWORK * sizeof(BatchWork)) + aup(sizeof(int));
+  return aup(sizeof(MemberDev) * (size_t)max_members) + aup(sizeof(BatchWork)) + aup(sizeof(int));
 }
 
 bssn_status bssn_batch_create(int32_t precision, int32_t max_members, void* d_pool, size_t pool_bytes,
@@ -583,7 +516,8 @@ bssn_status bssn_batch_create(int32_t precision, int32_t max_members, void* d_po
   if (pool_bytes < tb) return bfail(BSSN_ENOMEM, "pool smaller than the batch tables");
   bssn_batch* b = new (std::nothrow) bssn_batch();
   if (!b) return bfail(BSSN_ENOMEM, "host allocation failed");
-  b->precision = precision;
+  b->dword = precision == BSSN_FF;
+  b->precision = b->dword ? BSSN_FP64 : precision;
   b->maxm = max_members;
   b->stream = (cudaStream_t)cuda_stream;
   b->pool = (char*)d_pool;
@@ -591,11 +525,11 @@ bssn_status bssn_batch_create(int32_t precision, int32_t max_members, void* d_po
   b->alloc.init(tb, pool_bytes);
   b->m.resize(max_members);
   b->h_mem.resize(max_members);
-  memset(b->h_work, 0, sizeof(b->h_work));
+  memset(&b->h_work, 0, sizeof(b->h_work));
   b->d_mem = (MemberDev*)b->pool;
   b->d_work = (BatchWork*)(b->pool + aup(sizeof(MemberDev) * (size_t)max_members));
-  b->d_err = (int*)((char*)b->d_work + aup(NWORK * sizeof(BatchWork)));
-  b->cfg = precision == BSSN_FF ? batch_default_tile_ff() : batch_default_tile(precision == BSSN_MIXED);
+  b->d_err = (int*)((char*)b->d_work + aup(sizeof(BatchWork)));
+  b->cfg = batch_default_tile(precision == BSSN_MIXED);
   cudaError_t e = prepare_cfg(b, b->cfg);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream);
   if (e == cudaSuccess) e = rebuild_work(b);
@@ -625,7 +559,7 @@ bssn_status bssn_batch_add(bssn_batch* b, const bssn_params* p, int32_t* member)
   std::lock_guard<std::mutex> lk(b->mu);
   std::string why;
   if (!validate_params(p, why)) return bfail(BSSN_EINVAL, why);
-  if (p->precision != b->precision) return bfail(BSSN_EINVAL, "member precision differs from the batch's");
+  if (p->precision != (b->dword ? BSSN_FF : b->precision)) return bfail(BSSN_EINVAL, "member precision differs from the batch's");
   if (p->ksum_fp64) return bfail(BSSN_EINVAL, "ksum_fp64 is for single-grid contexts");
   int id = -1;
   for (int q = 0; q < b->maxm; q++)
@@ -743,7 +677,7 @@ bssn_status bssn_batch_step(bssn_batch* b, int32_t nsteps) {
   if (b->work_dirty) e = rebuild_work(b);
   if (e == cudaSuccess && !b->exec) e = capture(b);
   if (e != cudaSuccess) return bcuda(e, "batch step setup");
-  if (b->h_work[WORK_ALL].count == 0) return BSSN_OK;
+  if (b->h_work.count == 0) return BSSN_OK;
   for (int s = 0; s < nsteps; s++) {
     e = cudaGraphLaunch(b->exec, b->stream);
     if (e != cudaSuccess) return bcuda(e, "batch graph launch");
@@ -1140,7 +1074,7 @@ bssn_status bssn_submit(bssn_server* S, const bssn_params* p, int32_t id_kind, c
     return bfail(BSSN_EINVAL, "bad argument");
   const size_t bytes = bssn_batch_member_bytes(p);
   if (bytes == 0) return BSSN_EINVAL;  // message set by validation
-  if (p->precision != S->batch->precision) return bfail(BSSN_EINVAL, "request precision differs from the server's");
+  if (p->precision != (S->batch->dword ? BSSN_FF : S->batch->precision)) return bfail(BSSN_EINVAL, "request precision differs from the server's");
   if (bytes > S->budget)
     return bfail(BSSN_EINVAL, "request needs " + std::to_string(bytes) + " bytes, more than the whole budget");
   Req r;

@@ -224,14 +224,14 @@ constexpr int C_MEMB = C_TMA + N_TMA_B;
 constexpr int N_MEMB = 3;
 constexpr int k_memb_streams[N_MEMB] = {16, 4, 1};
 
-int batch_tile_config_count() { return C_MEMB + N_MEMB + batch_ff_config_count(); }
-int batch_ff_cfg_index(int v) { return C_MEMB + N_MEMB + v; }
-int batch_ff_variant(int cfg) {
-  const int v = cfg - (C_MEMB + N_MEMB);
-  return (v >= 0 && v < batch_ff_config_count()) ? v : -1;
-}
-bool batch_tile_is_members(int c) { return c >= C_MEMB && c < C_MEMB + N_MEMB; }
-int batch_members_streams(int c) { return batch_tile_is_members(c) ? k_memb_streams[c - C_MEMB] : 0; }
+// double-word batches: their own names for "members"
+static const char* const k_ff_names[] = {"fftiles32x4x1/8+4", "fftiles32x4x1/8+8", "fftiles32x4x1/4+4"};
+constexpr int C_FF = C_MEMB + N_MEMB, N_FF = 3;
+
+int batch_tile_config_count() { return C_FF + N_FF; }
+int batch_ff_cfg_index() { return C_FF; }
+bool batch_tile_is_members(int c) { return c >= C_MEMB && c < C_FF + N_FF; }
+int batch_members_streams(int c) { return batch_tile_is_members(c) ? k_memb_streams[c < C_FF ? c - C_MEMB : 0] : 0; }
 int batch_tma_variant(int cfg) {
   const int v = cfg - C_TMA;
   return (v >= 0 && v < N_TMA_B) ? v : -1;
@@ -243,15 +243,10 @@ int batch_tma_variant(int cfg) {
 // eleven-field persistent TMA kernel; float64 843.8 against 867.8 for
 // tiles32x4x1/2 and 884.4 for the persistent 32x4x1/3).
 int batch_default_tile(bool) { return C_MEMB; }
-// double-word batches: the per-member chains one after another on a single
-// stream (89.1 M point-updates/s over the 64 binaries against 73.9 for
-// fftiles32x4x1/8+8 and 71.7 for chains on 16 streams, where different
-// double-word kernels sharing an SM's instruction cache slow each other)
-int batch_default_tile_ff() { return C_MEMB + 2; }
 bool batch_tile_is_tma(int c) { return batch_tma_variant(c) >= 0; }
-bool batch_tile_is_per_tile(int c) { return (c >= N_FUSED && c < C_TMA) || batch_ff_variant(c) >= 0; }
+bool batch_tile_is_per_tile(int c) { return (c >= N_FUSED && c < C_TMA); }
 const char* batch_tile_config_name(int c) {
-  if (batch_ff_variant(c) >= 0) return batch_ff_config_name(batch_ff_variant(c));
+  if (c >= C_FF && c < C_FF + N_FF) return k_ff_names[c - C_FF];
   if (c == C_TMA) return "tma32x4x1/2";
   if (c == C_TMA + 1) return "tma11_32x8x1/1";
   if (c == C_MEMB) return "members";
@@ -261,10 +256,6 @@ const char* batch_tile_config_name(int c) {
   return (c >= 0 && c < N_FUSED) ? k_bcfg[c].name : "";
 }
 void batch_tile_shape(int c, int& tx, int& ty, int& tz) {
-  if (batch_ff_variant(c) >= 0) {
-    batch_ff_tile_shape(batch_ff_variant(c), tx, ty, tz);
-    return;
-  }
   if (batch_tma_variant(c) >= 0 || batch_tile_is_members(c)) {  // members: the 11-field TMA kernel's tiles
     batch_tma_tile_shape(batch_tile_is_members(c) ? 1 : batch_tma_variant(c), tx, ty, tz);
     return;
@@ -282,16 +273,10 @@ void batch_tile_shape(int c, int& tx, int& ty, int& tz) {
   tz = k_bcfg[c].tz;
 }
 
-bool batch_tile_full(int cfg, const Grid& g) {
-  int tx, ty, tz;
-  batch_tile_shape(cfg, tx, ty, tz);
-  return tx == 32 && g.n0 % 32 == 0 && g.n1 % ty == 0 && g.n2 % tz == 0;
-}
-
 cudaError_t launch_batch_stage(int cfg, bool mixed, const MemberDev* mem, const BatchWork* wk,
                                unsigned ntiles, int stage, int* err, cudaStream_t s) {
   if (batch_tma_variant(cfg) >= 0 && mixed) return launch_batch_stage_tma(batch_tma_variant(cfg), mem, wk, stage, err, s);
-  if (batch_tile_is_per_tile(cfg) && batch_ff_variant(cfg) < 0) {
+  if (batch_tile_is_per_tile(cfg)) {
     const TileCfgB& c = k_tcfg[cfg - N_FUSED];
     if (ntiles == 0) return cudaSuccess;
     const void* fn = mixed ? c.kmx : c.k64;

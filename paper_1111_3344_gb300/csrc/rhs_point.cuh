@@ -3,7 +3,7 @@
 // phi, gt, At, Gt with m = 1 in vacuum; Ricci pieces Rt_ij and Rphi_ij; 1+log
 // / harmonic / geodesic slicing; Gamma-driver shift with q(r)).
 //
-// Float and double-word forms (the float64 one is rhs_fx.cuh).  Formulation
+// Float form (the float64 one is rhs_fx.cuh).  Formulation
 // (same discrete operator as the statement in the paper; the arrangement is
 // chosen to cut instructions):
 //  - symmetric tensors held as 6 components; gt^{ij} by cofactors over det;
@@ -28,18 +28,12 @@ template <>
 __device__ __forceinline__ double fmaT<double>(double a, double b, double c) { return fma(a, b, c); }
 template <>
 __device__ __forceinline__ float fmaT<float>(float a, float b, float c) { return fmaf(a, b, c); }
-template <>
-__device__ __forceinline__ ff fmaT<ff>(ff a, ff b, ff c) { return ff_fma(a, b, c); }
 
 // |x| and e^x in the arithmetic type
 template <typename T>
 __device__ __forceinline__ T absT(T x) { return fabs(x); }
-template <>
-__device__ __forceinline__ ff absT<ff>(ff x) { return ff_fabs(x); }
 template <typename T>
 __device__ __forceinline__ T expT(T x) { return exp(x); }
-template <>
-__device__ __forceinline__ ff expT<ff>(ff x) { return ff_exp(x); }
 
 template <typename T, typename S>
 __device__ __forceinline__ T ldg(const S* p) {
@@ -103,40 +97,6 @@ __device__ __forceinline__ T dmu(const A& acc, int f, const P* p, long long sa, 
   T b = d1u<T>(acc, f, p + 2 * sa, sb) - d1u<T>(acc, f, p - 2 * sa, sb);
   return fmaT<T>(T(8), a, -b);
 }
-// D1_x D1_b of field f (b = y or z) for a warp whose 32 lanes hold 32
-// consecutive x points of one row: v is this point's first difference along b
-// (already formed, scaled by 1/(12h)); the lanes x-1, x+1, x-2, x+2 hold
-// theirs, so only the two lanes at each end of the row form one more
-// (at x -+ 2), and the mixed difference costs 3 operations instead of 15.  Same stencil as dmu (D1 along x applied to D1 along b); the result
-// is 12 h times the mixed derivative (v already carries 1/(12h)).
-__device__ __forceinline__ ff shflT(ff v, int src, int W) {
-  return ff(__shfl_sync(0xffffffffu, v.hi, src, W), __shfl_sync(0xffffffffu, v.lo, src, W));
-}
-template <int W, typename T, typename A, typename P>
-__device__ __forceinline__ T dmx_shfl(const A& acc, int f, const P* p, long long sb, T v, T i12h) {
-  const int lane = threadIdx.x & (W - 1);
-  const bool lo = lane < 2, hi = lane >= W - 2;
-  T ve = T(0);
-  if (lo || hi) ve = d1u<T>(acc, f, p + (lo ? -2 : 2), sb) * i12h;  // x - 2 or x + 2
-  const T sm2 = shflT(v, lane - 2, W);
-  const T sm1 = shflT(v, lane - 1, W);
-  const T sp1 = shflT(v, lane + 1, W);
-  const T sp2 = shflT(v, lane + 2, W);
-  const T e1 = shflT(ve, 1, W);       // lane 1 holds x_0 - 1
-  const T ew = shflT(ve, W - 2, W);   // lane W-2 holds x_{W-1} + 1
-  const T vm2 = lane >= 2 ? sm2 : ve;
-  const T vm1 = lane >= 1 ? sm1 : e1;
-  const T vp1 = lane <= W - 2 ? sp1 : ew;
-  const T vp2 = lane <= W - 3 ? sp2 : ve;
-  return fmaT<T>(T(8), vp1 - vm1, -(vp2 - vm2));
-}
-// Dynamic shared memory of a double-word full-block stage (32 x ty x tz
-// points): the first differences along z of 11 fields over the block's rows
-// and two halo rows on each side.
-__host__ __device__ constexpr size_t rows_block_smem(int ty, int tz) {
-  return (size_t)11 * (ty + 4) * tz * 32 * sizeof(ff);
-}
-
 // the same helpers over the plain read-only global path (one field)
 template <typename T, typename S>
 struct PlainAcc {
@@ -163,8 +123,8 @@ __device__ __forceinline__ double up_coef(bool pos, int m) {
   const double cn[7] = {1.0, -6.0, 18.0, -10.0, -3.0, 0.0, 0.0};
   return pos ? cp[m + 3] : cn[m + 3];
 }
-// the same weight in the arithmetic type T (float and double-word: from the
-// float constants, which hold these small integers exactly)
+// the same weight in the arithmetic type T (float: from the float constants,
+// which hold these small integers exactly)
 template <typename T>
 __device__ __forceinline__ T up_coefT(bool pos, int m) {
   if constexpr (is_f64<T>) {
@@ -188,28 +148,12 @@ __host__ __device__ __forceinline__ double background(const Grid& g, int f) {
 // Right-hand side of all 24 fields at interior point (i, j, k) with linear
 // index id, reading the state register st (field stride g.fstride).  DEV: the
 // register holds X - X0 (mixed-path float buffers) instead of X.
-// XSEG = 32: the calling warp is one full x-row of 32 points (double-word only);
-// the mixed second differences involving x then share first differences
-// across lanes (dmx_shfl).  XSEG = 0: every stencil evaluated by the thread.
-// YROWS > 0 (with XSEG = 32): the block is 32 x YROWS x ZS points, every
-// thread inside the grid, and D_y D_z takes the neighbouring rows' first
-// differences along z from shared memory (11 fields x (YROWS + 4) rows x ZS x
-// 32 values of dynamic shared memory; one barrier).
-template <typename T, typename S, bool DEV, typename A, int XSEG = 0, int YROWS = 0, int ZS = 1>
+template <typename T, typename S, bool DEV, typename A>
 __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i, int j, int k,
                                               T out[NF]) {
-  // ROLL (double-word arithmetic): a double-word operation is 7 to 15 float
-  // instructions, so the fully unrolled right-hand side would be some 30,000
-  // instructions of straight-line code per point, far beyond the instruction
-  // cache (ncu: warps stalled mostly on instruction fetch).  The second
-  // derivatives (six pairs) and the advection / dissipation stencils (24
-  // fields) then run as loops over the pairs and the fields, in the same order
-  // and with the same arithmetic, with their per-iteration values kept in
-  // arrays indexed at run time.
-  constexpr bool ROLL = std::is_same<T, ff>::value;
-  const T i12h = gc<T>(g.i12h, g.i12hf, g.i12hl);
-  const T i12h2 = gc<T>(g.i12h2, g.i12h2f, g.i12h2l);
-  const T i144h2 = gc<T>(g.i144h2, g.i144h2f, g.i144h2l);
+  const T i12h = gc<T>(g.i12h, g.i12hf);
+  const T i12h2 = gc<T>(g.i12h2, g.i12h2f);
+  const T i144h2 = gc<T>(g.i144h2, g.i144h2f);
 #define PF(f) acc.ptr(f)
 #define SD(f, d) acc.s((f), (d))
 #define LD(f, p) acc.template ld<T>((f), (p))
@@ -245,7 +189,7 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
     T det = gt[0] * c00 + gt[1] * c01 + gt[2] * c02;
     T idet;
     if (g.use_w) {
-      const T wf = gc<T>(g.w_floor, g.w_floorf, g.w_floorl);
+      const T wf = gc<T>(g.w_floor, g.w_floorf);
       const T Wd = chi > wf ? chi : wf;
       const T r = T(1) / (det * Wd);
       idet = Wd * r;
@@ -277,35 +221,6 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
     }
   }
 
-  // ---- D_y D_z through shared memory (full blocks of full rows)
-  [[maybe_unused]] T dyz[11];  // gt_ij (6), phi|W, alpha, beta^i (3)
-  if constexpr (YROWS > 0 && XSEG == 32 && !is_f32<T>) {
-    extern __shared__ float2 yz_smem[];
-    T* yz = reinterpret_cast<T*>(yz_smem);
-    constexpr int ROWS = YROWS + 4;
-    const int ty = threadIdx.y, tz = threadIdx.z, lane = threadIdx.x;
-    auto at = [&](int q, int row) -> T& { return yz[((q * ROWS + row) * ZS + tz) * 32 + lane]; };
-    auto dz_of = [&](int q) -> T {
-      return q < 6 ? dgt[2][q] : (q == 6 ? dchi[2] : (q == 7 ? dalp[2] : db[2][q - 8]));
-    };
-    auto field_of = [](int q) { return q < 6 ? F_GT + q : (q == 6 ? F_CHI : (q == 7 ? F_ALP : F_BETA + (q - 8))); };
-    const long long sy = SD(F_CHI, 1), sz = SD(F_CHI, 2);
-#pragma unroll
-    for (int q = 0; q < 11; q++) at(q, ty + 2) = dz_of(q);
-    if (ty < 2) {  // rows y0-2, y0-1 below the block
-#pragma unroll
-      for (int q = 0; q < 11; q++) at(q, ty) = d1u<T>(acc, field_of(q), PF(field_of(q)) - 2 * sy, sz) * i12h;
-    }
-    if (ty >= YROWS - 2) {  // rows y0+YROWS, y0+YROWS+1 above it
-#pragma unroll
-      for (int q = 0; q < 11; q++) at(q, ty + 4) = d1u<T>(acc, field_of(q), PF(field_of(q)) + 2 * sy, sz) * i12h;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 11; q++)
-      dyz[q] = fmaT<T>(T(8), at(q, ty + 3) - at(q, ty + 1), -(at(q, ty + 4) - at(q, ty)));  // x 1/(12h)
-  }
-
   // ---- second derivatives, consumed pair by pair.  Each is formed unscaled
   // (12 h^2, 12 h or 144 h^2 times the derivative, by stencil) and its scale
   // sc goes into the weight of the contraction that takes it.
@@ -322,79 +237,7 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
   for (int m = 0; m < 6; m++) Rdd[m] = T(0);
 #pragma unroll
   for (int a = 0; a < 3; a++) lapb[a] = gdiv[a] = T(0);
-  if constexpr (ROLL) {
-    // The six pairs (a, b) as a loop that is not unrolled: the same stencils
-    // and the same contractions in the same order, with the pair's strides,
-    // scale and first differences picked at run time -- one copy of the code
-    // instead of six (see ROLL).
-    const long long s3[3] = {SD(F_GT, 0), SD(F_GT, 1), SD(F_GT, 2)};
-#pragma unroll 1
-    for (int pq = 0; pq < 6; pq++) {
-      const int pa = pq < 3 ? 0 : (pq < 5 ? 1 : 2);
-      const int pb = pq < 3 ? pq : (pq < 5 ? pq - 2 : 2);
-      const long long sa = pa == 0 ? s3[0] : (pa == 1 ? s3[1] : s3[2]);
-      const long long sb = pb == 0 ? s3[0] : (pb == 1 ? s3[1] : s3[2]);
-      T dd[6], vb[3], vchi, valp, sc;
-      if (pa == pb) {
-        sc = i12h2;
-#pragma unroll
-        for (int m = 0; m < 6; m++) dd[m] = d2u<T>(acc, F_GT + m, PF(F_GT + m), sa, gt_r[m]);
-        vchi = d2u<T>(acc, F_CHI, PF(F_CHI), sa, chi_r) * i12h2;
-        valp = d2u<T>(acc, F_ALP, PF(F_ALP), sa, alp_r);
-#pragma unroll
-        for (int a = 0; a < 3; a++) vb[a] = d2u<T>(acc, F_BETA + a, PF(F_BETA + a), sa, beta[a]);
-      } else if (XSEG > 0 && pa == 0) {
-        if constexpr (XSEG > 0) {
-          sc = i12h;
-          const bool y = pb == 1;
-#pragma unroll
-          for (int m = 0; m < 6; m++)
-            dd[m] = dmx_shfl<XSEG>(acc, F_GT + m, PF(F_GT + m), sb, y ? dgt[1][m] : dgt[2][m], i12h);
-          vchi = dmx_shfl<XSEG>(acc, F_CHI, PF(F_CHI), sb, y ? dchi[1] : dchi[2], i12h) * i12h;
-          valp = dmx_shfl<XSEG>(acc, F_ALP, PF(F_ALP), sb, y ? dalp[1] : dalp[2], i12h);
-#pragma unroll
-          for (int a = 0; a < 3; a++)
-            vb[a] = dmx_shfl<XSEG>(acc, F_BETA + a, PF(F_BETA + a), sb, y ? db[1][a] : db[2][a], i12h);
-        }
-      } else if (YROWS > 0 && pa == 1) {  // (1, 2) from the rows' differences along z
-        sc = i12h;
-#pragma unroll
-        for (int m = 0; m < 6; m++) dd[m] = dyz[m];
-        vchi = dyz[6] * i12h;
-        valp = dyz[7];
-#pragma unroll
-        for (int a = 0; a < 3; a++) vb[a] = dyz[8 + a];
-      } else {
-        sc = i144h2;
-#pragma unroll
-        for (int m = 0; m < 6; m++) dd[m] = dmu<T>(acc, F_GT + m, PF(F_GT + m), sa, sb);
-        vchi = dmu<T>(acc, F_CHI, PF(F_CHI), sa, sb) * i144h2;
-        valp = dmu<T>(acc, F_ALP, PF(F_ALP), sa, sb);
-#pragma unroll
-        for (int a = 0; a < 3; a++) vb[a] = dmu<T>(acc, F_BETA + a, PF(F_BETA + a), sa, sb);
-      }
-      ddchi[pq] = vchi;
-      ddalp[pq] = valp;
-      sc2[pq] = sc;
-      T g2 = g2u[0];
-#pragma unroll
-      for (int m = 1; m < 6; m++) g2 = pq == m ? g2u[m] : g2;
-      const T wb = sc * g2;
-      const T w = T(-0.5) * wb;
-#pragma unroll
-      for (int m = 0; m < 6; m++) Rdd[m] = fmaT<T>(w, dd[m], Rdd[m]);
-#pragma unroll
-      for (int a = 0; a < 3; a++) {
-        lapb[a] = fmaT<T>(wb, vb[a], lapb[a]);
-        // d_pa d_pb beta^a: into gdiv[pa] when a == pb, into gdiv[pb] when a == pa != pb
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-          if (a == pb && k == pa) gdiv[k] = fmaT<T>(sc, vb[a], gdiv[k]);
-          if (pa != pb && a == pa && k == pb) gdiv[k] = fmaT<T>(sc, vb[a], gdiv[k]);
-        }
-      }
-    }
-  } else {
+  {
 #pragma unroll
     for (int pa = 0; pa < 3; pa++) {
 #pragma unroll
@@ -408,27 +251,6 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
           for (int m = 0; m < 6; m++) dd[m] = d2u<T>(acc, F_GT + m, PF(F_GT + m), SD(F_GT + m, pa), gt_r[m]);
           ddchi[pq] = d2u<T>(acc, F_CHI, PF(F_CHI), SD(F_CHI, pa), chi_r) * i12h2;
           ddalp[pq] = d2u<T>(acc, F_ALP, PF(F_ALP), SD(F_ALP, pa), alp_r);
-        } else if constexpr (XSEG > 0 && !is_f32<T>) {
-          if (pa == 0) {
-            sc = i12h;
-#pragma unroll
-            for (int m = 0; m < 6; m++)
-              dd[m] = dmx_shfl<XSEG>(acc, F_GT + m, PF(F_GT + m), SD(F_GT + m, pb), dgt[pb][m], i12h);
-            ddchi[pq] = dmx_shfl<XSEG>(acc, F_CHI, PF(F_CHI), SD(F_CHI, pb), dchi[pb], i12h) * i12h;
-            ddalp[pq] = dmx_shfl<XSEG>(acc, F_ALP, PF(F_ALP), SD(F_ALP, pb), dalp[pb], i12h);
-          } else if constexpr (YROWS > 0) {  // (1, 2)
-            sc = i12h;
-#pragma unroll
-            for (int m = 0; m < 6; m++) dd[m] = dyz[m];
-            ddchi[pq] = dyz[6] * i12h;
-            ddalp[pq] = dyz[7];
-          } else {
-            sc = i144h2;
-#pragma unroll
-            for (int m = 0; m < 6; m++) dd[m] = dmu<T>(acc, F_GT + m, PF(F_GT + m), SD(F_GT + m, pa), SD(F_GT + m, pb));
-            ddchi[pq] = dmu<T>(acc, F_CHI, PF(F_CHI), SD(F_CHI, pa), SD(F_CHI, pb)) * i144h2;
-            ddalp[pq] = dmu<T>(acc, F_ALP, PF(F_ALP), SD(F_ALP, pa), SD(F_ALP, pb));
-          }
         } else {
           sc = i144h2;
 #pragma unroll
@@ -448,13 +270,6 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
           T v;
           if (pa == pb) {
             v = d2u<T>(acc, F_BETA + a, PF(F_BETA + a), SD(F_BETA + a, pa), beta[a]);
-          } else if constexpr (XSEG > 0 && !is_f32<T>) {
-            if (pa == 0)
-              v = dmx_shfl<XSEG>(acc, F_BETA + a, PF(F_BETA + a), SD(F_BETA + a, pb), db[pb][a], i12h);
-            else if constexpr (YROWS > 0)
-              v = dyz[8 + a];
-            else
-              v = dmu<T>(acc, F_BETA + a, PF(F_BETA + a), SD(F_BETA + a, pa), SD(F_BETA + a, pb));
           } else {
             v = dmu<T>(acc, F_BETA + a, PF(F_BETA + a), SD(F_BETA + a, pa), SD(F_BETA + a, pb));
           }
@@ -752,7 +567,7 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       out[F_BETA + a] = T(0.75) * Bv[a];
-      out[F_B + a] = gam_rhs[a] - gc<T>(g.eta, g.etaf, g.etal) * q * Bv[a];
+      out[F_B + a] = gam_rhs[a] - gc<T>(g.eta, g.etaf) * q * Bv[a];
     }
   }
 
@@ -765,42 +580,8 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
 #pragma unroll
     for (int f = 0; f < NF; f++)
       if (f < nf) out[f] += acc.template advko<T>(f);
-  } else if constexpr (ROLL) {
-    // one loop over the fields: the same weights and the same order of
-    // accumulation as below (centre term, then axes x, y, z, offsets -3..3)
-    const T kap = gc<T>(g.kos, g.kosf, g.kosl);
-    T bh[3];
-#pragma unroll
-    for (int d = 0; d < 3; d++) bh[d] = absT<T>(beta[d]) * i12h;
-    const T w0 = fmaT<T>(T(-10), bh[0] + bh[1] + bh[2], T(-60) * kap);
-    const T cko[7] = {T(1), T(-6), T(15), T(-20), T(15), T(-6), T(1)};
-    T w[3][7];
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-      const bool pos = beta[d] >= T(0);
-#pragma unroll
-      for (int m = -3; m <= 3; m++)
-        if (m != 0) w[d][m + 3] = fmaT<T>(bh[d], up_coefT<T>(pos, m), kap * cko[m + 3]);
-    }
-    T r[NF];  // indexed at run time
-#pragma unroll
-    for (int f = 0; f < NF; f++) r[f] = out[f];
-    const long long s3[3] = {SD(F_GT, 0), SD(F_GT, 1), SD(F_GT, 2)};
-#pragma unroll 1
-    for (int f = 0; f < nf; f++) {
-      const auto* p = PF(f);
-      T accv = fmaT<T>(w0, LD(f, p), r[f]);
-#pragma unroll
-      for (int d = 0; d < 3; d++)
-#pragma unroll
-        for (int m = -3; m <= 3; m++)
-          if (m != 0) accv = fmaT<T>(w[d][m + 3], LD(f, p + m * s3[d]), accv);
-      r[f] = accv;
-    }
-#pragma unroll
-    for (int f = 0; f < NF; f++) out[f] = r[f];
   } else {
-    const T kap = gc<T>(g.kos, g.kosf, g.kosl);
+    const T kap = gc<T>(g.kos, g.kosf);
     T f0s[NF];  // centre values as stored (float: the stencil is applied to f_m - f0)
     T bh[3];
 #pragma unroll
@@ -854,11 +635,5 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
 }
 
 // Right-hand side reading every field from the global register st.
-template <typename T, typename S, bool DEV = false, int XSEG = 0, int YROWS = 0, int ZS = 1>
-__device__ __forceinline__ void rhs_point(const Grid& g, const S* __restrict__ st, long long id,
-                                          int i, int j, int k, T out[NF]) {
-  const GlobalAcc<S> acc(g, st, id);
-  rhs_point_acc<T, S, DEV, GlobalAcc<S>, XSEG, YROWS, ZS>(g, acc, i, j, k, out);
-}
 
 }  // namespace bssn
