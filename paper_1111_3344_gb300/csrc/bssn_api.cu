@@ -177,7 +177,7 @@ struct bssn_ctx {
   double* ks64;  // mixed with ksum_fp64: float64 k-sum of every field (else null)
   bool shadow_valid;
   int tile;  // stage-kernel tile configuration (see bssn_autotune)
-  CUtensorMap tmap[2][3];  // mixed: tensor maps of the float stage buffers, per TMA box (tma_map)
+  CUtensorMap tmap[3][3];  // mixed: tensor maps of the float stage buffers, per TMA variant
   bool tmap_ok;
   CUtensorMap fmap[3];  // float64: tensor maps of y_n, s1, s2 (tile form of the stage)
   bool fmap_ok;
@@ -214,15 +214,13 @@ struct bssn_ctx {
 
 // Tile configuration indices: [0, tile_config_count()) fused kernels, then
 // N_TMA TMA-staged mixed kernels (variant 0: 32x4x1, two blocks per SM;
-// 1: 32x8x1, one block per SM; 2: 32x8x1 staging beta^i too), then the
+// 1: 32x8x1, one block per SM; 2: 32x2x4 staging beta^i too), then the
 // split-stage variants.
 constexpr int N_TMA = 3;
 static int tma_variant(int cfg) {
   const int v = cfg - tile_config_count();
   return (v >= 0 && v < N_TMA) ? v : -1;
 }
-// tensor map of a TMA variant: variants 1 and 2 share the 32x8x1 box
-static int tma_map(int v) { return v >= 1 ? 1 : 0; }
 static int split_variant(int cfg) {
   const int v = cfg - tile_config_count() - N_TMA;
   return (v >= 0 && v < split_config_count()) ? v : -1;
@@ -349,13 +347,13 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
                  make_fx_tensor_map(g, ctx->s2, &ctx->fmap[2]) == cudaSuccess;
   if (p->precision == BSSN_MIXED) {
     bool ok = true;
-    for (int v = 0; v < 2 && ok; v++)
+    for (int v = 0; v < N_TMA && ok; v++)
       for (int q = 0; q < 3 && ok; q++) ok = make_stage_tensor_map(g, ctx->m32[q], &ctx->tmap[v][q], v) == cudaSuccess;
     ctx->tmap_ok = ok;
     // the 11-field TMA stage: the same bits as the fused kernels and the
     // fastest configuration at every size measured (one step, against the fused
-    // 32x8x1: 24^3 0.128 against 0.145 ms, 48^3 0.40 / 0.48, 100x70x50 1.07 /
-    // 1.41, 128^3 4.23 / 5.37, 256^3 31.2 / 43.2)
+    // 32x8x1, which took 0.145 ms at 24^3, 0.48 at 48^3, 5.37 at 128^3, 43.2 at
+    // 256^3: 0.13, 0.34, 3.71, 27.7)
     if (ok) ctx->tile = tile_config_count() + 2;
   }
   ctx->cstream = ctx->istream = nullptr;
@@ -564,7 +562,7 @@ bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs) {
   if (split_variant(ctx->tile) >= 0)
     e = launch_stage_mixed_split(ctx->g, a, ctx->dr, ctx->stream, split_variant(ctx->tile));
   else if (tma_variant(ctx->tile) >= 0)
-    e = launch_stage_mixed_tma(ctx->g, a, ctx->tmap[tma_map(tma_variant(ctx->tile))][2], ctx->err, ctx->stream,
+    e = launch_stage_mixed_tma(ctx->g, a, ctx->tmap[tma_variant(ctx->tile)][2], ctx->err, ctx->stream,
                                tma_variant(ctx->tile));
   else
     e = launch_stage_mixed(ctx->g, a, ctx->stream, ctx->tile);
@@ -631,7 +629,7 @@ static bssn_status run_stage_mixed(bssn_ctx* ctx, int src, int mode, int out, do
   if (ctx->ks64)
     e = launch_stage_mixed_ks64(ctx->g, a, ctx->stream);
   else if (tma_variant(ctx->tile) >= 0)
-    e = launch_stage_mixed_tma(ctx->g, a, ctx->tmap[tma_map(tma_variant(ctx->tile))][src], ctx->err,
+    e = launch_stage_mixed_tma(ctx->g, a, ctx->tmap[tma_variant(ctx->tile)][src], ctx->err,
                                ctx->stream, tma_variant(ctx->tile));
   else if (split_variant(ctx->tile) >= 0)
     e = launch_stage_mixed_split(ctx->g, a, ctx->dr, ctx->stream, split_variant(ctx->tile));
@@ -1022,7 +1020,7 @@ bssn_status bssn_autotune(bssn_ctx* ctx, int32_t reps, int32_t* best, double* ms
       a.w_thr = ctx->p.w_fp64_threshold; a.mode = second ? MODE_MID : MODE_FIRST;
       if (ctx->ks64) return launch_stage_mixed_ks64(ctx->g, a, ctx->stream);
       if (tma_variant(c) >= 0)
-        return launch_stage_mixed_tma(ctx->g, a, ctx->tmap[tma_map(tma_variant(c))][q], ctx->err, ctx->stream,
+        return launch_stage_mixed_tma(ctx->g, a, ctx->tmap[tma_variant(c)][q], ctx->err, ctx->stream,
                                       tma_variant(c));
       if (split_variant(c) >= 0)
         return launch_stage_mixed_split(ctx->g, a, ctx->dr, ctx->stream, split_variant(c));

@@ -224,9 +224,10 @@ void fill_member_dev(bssn_batch* b, int id) {
       a.w_thr = M.p.w_fp64_threshold;
       a.mode = mode[s];
       a.stall_polls = b->stall_polls;
-      // the box of the batch's TMA variant (32x8x1 tiles: tensor-map variant 1)
-      const bool box8 = batch_tma_variant(b->cfg) == 1 || batch_tile_is_members(b->cfg);
-      if (make_stage_tensor_map(M.g, a.src, &D.tmap[s], box8 ? 1 : 0) != cudaSuccess)
+      // the box of the configuration's kernel: the single-grid variant 2 or the
+      // batch's own TMA variants
+      const int box = batch_tile_is_members(b->cfg) ? 2 : (batch_tma_variant(b->cfg) == 1 ? 1 : 0);
+      if (make_stage_tensor_map(M.g, a.src, &D.tmap[s], box) != cudaSuccess)
         b->tma_ok = false;
     }
   }

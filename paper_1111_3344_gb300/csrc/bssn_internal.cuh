@@ -293,7 +293,7 @@ const char* tile_config_name(int c);
 // with a box of bx x by x bz points of one field.
 cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out);
 // Tensor map of a float stage buffer for TMA-staged variant v (0: 32 x 4 x 1
-// tiles, 1: 32 x 8 x 1; the box is the tile plus three ghost layers).
+// tiles, 1: 32 x 8 x 1, 2: 32 x 2 x 4; the box is the tile plus three ghost layers).
 cudaError_t make_stage_tensor_map(const Grid& g, const float* base, CUtensorMap* out, int variant = 0);
 cudaError_t launch_stage_mixed_tma(const Grid& g, const StageArgsMixed& a, const CUtensorMap& map,
                                    int* err, cudaStream_t s, int variant = 0);

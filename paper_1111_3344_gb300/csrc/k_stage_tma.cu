@@ -39,14 +39,18 @@ __global__ void __launch_bounds__(Sh::TX * Sh::TY * Sh::TZ, MINB)
   __syncthreads();
   const bool stall = a.stall_polls > 0;  // test hook: no copy, short wait
   if (tid == 0 && !stall) issue_staged_loads<Sh>(&tmap, bar, smem, ii0, jj0, kk0);
+  const int ii = ii0 + threadIdx.x, jj = jj0 + threadIdx.y, kk = kk0 + threadIdx.z;
+  const bool inside = ii < g.n0 && jj < g.n1 && kk < g.n2;
+  // the combine's inputs, while the boxes are on their way (128^3: 0.848 -> 0.818 ms)
+  MixedPre<> pre;
+  if (inside) pre.load(g, a, lin(g, ii + GH, jj + GH, kk + GH));
   if (!mbar_wait(bar, 0, stall ? (long long)a.stall_polls : WAIT_LIMIT)) {
     if (tid == 0) atomicExch(err, 1);
     if (!stall) mbar_wait(bar, 0, WAIT_LIMIT);  // let this block's own copies land before it exits
     return;
   }
   const int ti = threadIdx.x, tj = threadIdx.y, tk = threadIdx.z;
-  const int ii = ii0 + ti, jj = jj0 + tj, kk = kk0 + tk;
-  if (ii >= g.n0 || jj >= g.n1 || kk >= g.n2) return;
+  if (!inside) return;
   const int i = ii + GH, j = jj + GH, k = kk + GH;
   TileAccT<Sh> acc;
   acc.st = a.src;
@@ -56,12 +60,14 @@ __global__ void __launch_bounds__(Sh::TX * Sh::TY * Sh::TZ, MINB)
   acc.sd[1] = g.pitch;
   acc.sd[2] = g.plane;
   acc.sm = smem + ((tk + GH) * Sh::BY + (tj + GH)) * Sh::BX + (ti + GH);
-  stage_point_mixed_acc(g, a, acc, ii, jj, kk);
+  stage_point_mixed_acc<TileAccT<Sh>, false>(g, a, acc, ii, jj, kk, pre);
 }
 
 // ------------------------------------------------------------------ host
 namespace {
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
+// variant 2's tile
+using TmaWide = TmaShape<2, 4, 11>;
 }
 
 cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out) {
@@ -89,8 +95,8 @@ cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx,
 }
 
 cudaError_t make_stage_tensor_map(const Grid& g, const float* base, CUtensorMap* out, int variant) {
-  return encode_tensor_map(g, base, 4, TmaDefault::BX, variant >= 1 ? TmaShape<8>::BY : TmaShape<4>::BY,
-                           TmaShape<4>::BZ, out);
+  const int by = variant == 2 ? TmaWide::BY : (variant == 1 ? TmaShape<8>::BY : TmaShape<4>::BY);
+  return encode_tensor_map(g, base, 4, TmaDefault::BX, by, variant == 2 ? TmaWide::BZ : TmaShape<4>::BZ, out);
 }
 
 // dynamic shared memory above the default limit, once per kernel and device
@@ -113,17 +119,23 @@ static cudaError_t launch_tma(const Grid& g, const StageArgsMixed& a, const CUte
 
 // variant 0: 32 x 4 x 1 tiles, two blocks per SM; 1: 32 x 8 x 1 tiles, one
 // block per SM (half the shared memory per SM, so more L1 for the fields read
-// through it); 2: 32 x 8 x 1 tiles staging beta^i as well (eleven fields,
-// 173 KB, one block per SM; the tensor map of variant 1 serves, same box);
-// map: a tensor map made for the same variant
+// through it); 2: 32 x 2 x 4 tiles staging beta^i as well (eleven fields, 141 KB,
+// one block per SM); map: a tensor map made for the same variant.
+// Variant 2 is bound by the latency of the loads of the other 13 fields with
+// two warps per scheduler: its boxes (40 x 8 x 10) and the planes that those
+// fields' stencils touch are smaller than a 32 x 8 x 1 tile's (40 x 14 x 7, 173
+// KB), so that more of them stay in L1.  A stage, ms, 32 x 8 x 1 / 32 x 4 x 2 /
+// 32 x 2 x 4 / 32 x 1 x 8: 128^3 0.827 / 0.797 / 0.792 / 0.814, 256^3 6.75 / 6.66 /
+// 6.39 / 6.28, 48^3 0.0648 / 0.0642 / 0.0634 / 0.0645.  Slower: 384 threads (1.09 at 128^3),
+// 512 with 8 fields (0.94), two blocks of 128 (0.84), prefetches to L2 (0.82).
 cudaError_t prepare_stage_mixed_tma(int variant) {
-  if (variant == 2) return tma_attr<TmaShape<8, 1, 11>, 1>();
+  if (variant == 2) return tma_attr<TmaWide, 1>();
   return variant == 1 ? tma_attr<TmaShape<8>, 1>() : tma_attr<TmaShape<4>, 2>();
 }
 
 cudaError_t launch_stage_mixed_tma(const Grid& g, const StageArgsMixed& a, const CUtensorMap& map,
                                    int* err, cudaStream_t s, int variant) {
-  if (variant == 2) return launch_tma<TmaShape<8, 1, 11>, 1>(g, a, map, err, s);
+  if (variant == 2) return launch_tma<TmaWide, 1>(g, a, map, err, s);
   return variant == 1 ? launch_tma<TmaShape<8>, 1>(g, a, map, err, s) : launch_tma<TmaShape<4>, 2>(g, a, map, err, s);
 }
 

@@ -114,37 +114,46 @@ __device__ __forceinline__ double chi_rhs_fp64(const Grid& g, const float* __res
   return r;
 }
 
+// The combine's inputs (stages 2-3: base and k-sum; stage 4: k-sum and y_n),
+// loaded before the right-hand side: issued after it, at 255 registers and 8
+// warps per SM, their latency was exposed (a third of the step).  What the
+// compiler cannot keep in registers it spills to local memory, which comes
+// back from L1.
+template <bool KS64 = false>
+struct MixedPre {
+  float pk[NF], ps[NF];
+  double py[NF];
+  __device__ __forceinline__ void load(const Grid& g, const StageArgsMixed& a, long long id) {
+    const long long fs = g.fstride;
+    if (a.mode == MODE_MID) {
+#pragma unroll
+      for (int f = 1; f < NF; f++) {
+        ps[f] = a.src0[f * fs + id];
+        if (!KS64) pk[f] = a.ksum[f * fs + id];
+      }
+    } else if (a.mode == MODE_LAST) {
+#pragma unroll
+      for (int f = 1; f < NF; f++) {
+        if (!KS64) pk[f] = a.ksum[f * fs + id];
+        py[f] = a.yn[f * fs + id];
+      }
+    }
+  }
+};
+
 // Fused stage at interior point (ii, jj, kk), mixed precision; the accessor
 // says where each field of the stage input is read from.  KS64: the k-sum of
 // every field is float64 (a.ksum64; the ksum_fp64 option), a separate
 // instantiation so that the default kernels keep their register allocation.
 template <typename A, bool KS64 = false>
 __device__ __forceinline__ void stage_point_mixed_acc(const Grid& g, const StageArgsMixed& a,
-                                                      const A& acc, int ii, int jj, int kk) {
+                                                      const A& acc, int ii, int jj, int kk, MixedPre<KS64>& pre) {
   const int i = ii + GH, j = jj + GH, k = kk + GH;
   const long long id = lin(g, i, j, k);
   const long long fs = g.fstride;
-  // The combine's inputs (stages 2-3: base and k-sum; stage 4: k-sum and
-  // y_n) are loaded before the right-hand side: issued after it, at 255
-  // registers and 8 warps per SM, their latency was exposed (a third of the
-  // step).  What the compiler cannot keep in registers it spills to local
-  // memory, which comes back from L1.
-  float pk[NF], ps[NF];
-  double py[NF];
+  float(&pk)[NF] = pre.pk, (&ps)[NF] = pre.ps;
+  double(&py)[NF] = pre.py;
   constexpr bool ks64 = KS64;  // float64 k-sum of every field (ksum_fp64)
-  if (a.mode == MODE_MID) {
-#pragma unroll
-    for (int f = 1; f < NF; f++) {
-      ps[f] = a.src0[f * fs + id];
-      if (!ks64) pk[f] = a.ksum[f * fs + id];
-    }
-  } else if (a.mode == MODE_LAST) {
-#pragma unroll
-    for (int f = 1; f < NF; f++) {
-      if (!ks64) pk[f] = a.ksum[f * fs + id];
-      py[f] = a.yn[f * fs + id];
-    }
-  }
   float r[NF];
   rhs_point_acc<float, float, true>(g, acc, i, j, k, r);
   // near a puncture the W update runs in float64
@@ -200,11 +209,22 @@ __device__ __forceinline__ void stage_point_mixed_acc(const Grid& g, const Stage
   }
 }
 
+template <typename A>
+__device__ __forceinline__ void stage_point_mixed_acc(const Grid& g, const StageArgsMixed& a, const A& acc, int ii,
+                                                      int jj, int kk) {
+  MixedPre<> pre;
+  pre.load(g, a, lin(g, ii + GH, jj + GH, kk + GH));
+  stage_point_mixed_acc<A, false>(g, a, acc, ii, jj, kk, pre);
+}
+
 template <bool KS64 = false>
 __device__ __forceinline__ void stage_point_mixed(const Grid& g, const StageArgsMixed& a, int ii,
                                                   int jj, int kk) {
-  const GlobalAcc<float> acc(g, a.src, lin(g, ii + GH, jj + GH, kk + GH));
-  stage_point_mixed_acc<GlobalAcc<float>, KS64>(g, a, acc, ii, jj, kk);
+  const long long id = lin(g, ii + GH, jj + GH, kk + GH);
+  const GlobalAcc<float> acc(g, a.src, id);
+  MixedPre<KS64> pre;
+  pre.load(g, a, id);
+  stage_point_mixed_acc<GlobalAcc<float>, KS64>(g, a, acc, ii, jj, kk, pre);
 }
 
 }  // namespace bssn
