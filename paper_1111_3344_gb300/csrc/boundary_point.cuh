@@ -203,12 +203,12 @@ __device__ __forceinline__ void sommerfeld_point_fp64_tab(const Grid& g, const S
 #pragma unroll
   for (int n = 0; n < N; n++)
     rhs[n] = F0 + n < nf ? fma(fac, ka[n], v[n].sum(g, F0 + n, tb, nbs, irb)) : 0.0;
-  combine_fields_fp64(a, o, rhs);
+  combine_point_fp64(a, o, rhs, false);
 }
 
 // float64 path, anchor pass: interior point q of the boundary shell, fields
 // [F0, F1): k - rad at the anchor, in place of the k the stage kernel left in
-// kanchor (the same operations the ghost points of that anchor would repeat,
+// kanchor (MODE_RHS: in rhs) (the same operations the ghost points of that anchor would repeat,
 // one to three layers and up to eight neighbours over; see sommerfeld_point_fp64).
 template <int F0 = 0, int F1 = NF>
 __device__ __forceinline__ void sommerfeld_anchor_fp64(const Grid& g, const StageArgs& a,
@@ -229,18 +229,18 @@ __device__ __forceinline__ void sommerfeld_anchor_fp64(const Grid& g, const Stag
   const long long fs = g.fstride;
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
   const RadTaps ta = rad_taps_inside(g);
+  const double* ks = a.mode == MODE_RHS ? a.rhs : kanchor;
   double k[F1 - F0];  // every load before the stores
 #pragma unroll
   for (int f = F0; f < F1; f++)
-    if (f < nf) k[f - F0] = kanchor[f * fs + ia] - rad_at<double, double>(g, a.src + f * fs + ia, f, ta, nas, ira);
+    if (f < nf) k[f - F0] = ks[f * fs + ia] - rad_at<double, double>(g, a.src + f * fs + ia, f, ta, nas, ira);
 #pragma unroll
   for (int f = F0; f < F1; f++)
     if (f < nf) kanchor[f * fs + ia] = k[f - F0];
 }
 
-// float64 path: ghost point q, all fields.  PRE: kanchor already holds
-// k - rad at the anchor (the anchor pass ran), else k itself.
-template <bool PRE = false>
+// float64 path: ghost point q, all fields, from the k at the anchors (the batched
+// kernel, whose members' anchors no pass of their own has treated).
 __device__ __forceinline__ void sommerfeld_point_fp64(const Grid& g, const StageArgs& a,
                                                       const double* __restrict__ kanchor, unsigned q) {
   GhostGeo G;
@@ -249,26 +249,14 @@ __device__ __forceinline__ void sommerfeld_point_fp64(const Grid& g, const Stage
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
   const RadTaps tb = rad_taps(g, G.I), ta = rad_taps_inside(g);
   for (int f = 0; f < NF; f++) {
-    double rhs = 0.0;
+    double rhs[1] = {0.0};
+    const long long o[1] = {f * fs + G.ib};
     if (f < nf) {
       const double radb = rad_at<double, double>(g, a.src + f * fs + G.ib, f, tb, G.nbs, G.irb);
-      if (PRE && a.mode != MODE_RHS) {
-        rhs = fma(G.fac, kanchor[f * fs + G.ia], radb);
-      } else {
-        const double rada = rad_at<double, double>(g, a.src + f * fs + G.ia, f, ta, G.nas, G.ira);
-        const double ka = (a.mode == MODE_RHS) ? a.rhs[f * fs + G.ia] : kanchor[f * fs + G.ia];
-        rhs = fma(G.fac, ka - rada, radb);
-      }
+      const double rada = rad_at<double, double>(g, a.src + f * fs + G.ia, f, ta, G.nas, G.ira);
+      rhs[0] = fma(G.fac, kanchor[f * fs + G.ia] - rada, radb);
     }
-    const long long o = f * fs + G.ib;
-    if (a.mode == MODE_RHS) {
-      a.rhs[o] = rhs;
-    } else if (a.mode == MODE_LAST) {
-      a.yn[o] = fma(a.b_dt, a.ksum[o] + rhs, a.yn[o]);
-    } else {
-      a.out0[o] = fma(a.a_dt, rhs, a.src0[o]);
-      a.ksum[o] = a.mode == MODE_FIRST ? rhs : fma(2.0, rhs, a.ksum[o]);
-    }
+    combine_fields_fp64(a, o, rhs);
   }
 }
 

@@ -323,7 +323,7 @@ cudaError_t member_boundary(bssn_batch* b, int id, int stage, cudaStream_t s) {
   }
   const StageArgs& a = D.a64[stage];
   const Member& M = b->m[id];
-  if (!g.periodic) return launch_sommerfeld(g, a, a.kshell, s, M.L.has_gtab ? mptr(b, M, M.L.gtab) : nullptr);
+  if (!g.periodic) return launch_sommerfeld(g, a, a.kshell, s, mptr(b, M, M.L.gtab));
   return launch_periodic_fill(g, a.mode == MODE_LAST ? a.yn : a.out0, s);
 }
 

@@ -307,9 +307,10 @@ int split_config_count();
 const char* split_config_name(int v);
 cudaError_t launch_stage_mixed_split(const Grid& g, const StageArgsMixed& a, float* dr, cudaStream_t s,
                                      int variant);
-// table (may be null): the context's ghost-geometry table (launch_ghost_table)
-cudaError_t launch_sommerfeld(const Grid& g, const StageArgs& a, const double* kanchor,
-                              cudaStream_t s, const void* table = nullptr);
+// kanchor: scratch register (the anchors' k of a stage; MODE_RHS: overwritten);
+// table: the ghost-geometry table (launch_ghost_table)
+cudaError_t launch_sommerfeld(const Grid& g, const StageArgs& a, double* kanchor, cudaStream_t s,
+                              const void* table);
 size_t ghost_table_size(const Grid& g);
 cudaError_t launch_ghost_table(const Grid& g, void* table, cudaStream_t s);
 cudaError_t launch_sommerfeld_mixed(const Grid& g, const StageArgsMixed& a, const float* kanchor,

@@ -18,13 +18,6 @@
 
 namespace bssn {
 
-template <bool PRE>
-__global__ void sommerfeld_fp64_kernel(Grid g, StageArgs a, const double* __restrict__ kanchor) {
-  const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= ghost_count(g)) return;
-  sommerfeld_point_fp64<PRE>(g, a, kanchor, q);
-}
-
 // blockIdx.y: one of four field groups (W and gt_ij; K and At_ij but its last;
 // the rest of At_ij, Gt^i, alpha; beta^i and B^i)
 __global__ void sommerfeld_anchor_fp64_kernel(Grid g, StageArgs a, double* __restrict__ kanchor) {
@@ -97,26 +90,18 @@ __global__ void periodic_fill_kernel(Grid g, S* __restrict__ y, double* __restri
   periodic_point<S>(g, y, w, q);
 }
 
-// Stage modes: the anchor pass (one thread per shell point) turns the k left at
-// the anchors into k - rad once, then the ghost points each form only their
-// own radiative term.  MODE_RHS (no anchors): every ghost point forms both.
-cudaError_t launch_sommerfeld(const Grid& g, const StageArgs& a, const double* kanchor,
-                              cudaStream_t s, const void* table) {
-  const unsigned total = ghost_count(g);
+// The anchor pass (one thread per shell point) forms k - rad at the anchors once
+// into kanchor, then the ghost points each form only their own radiative term
+// (a right-hand side of 80^3: 1.13 ms with both terms and the geometry at every
+// ghost point, 1.03 so).
+cudaError_t launch_sommerfeld(const Grid& g, const StageArgs& a, double* kanchor, cudaStream_t s,
+                              const void* table) {
+  const unsigned total = ghost_count(g), ns = shell_count(g);
   const int bs = 128;
-  if (a.mode != MODE_RHS && kanchor) {
-    const unsigned ns = shell_count(g);
-    sommerfeld_anchor_fp64_kernel<<<dim3((ns + bs - 1) / bs, 4), bs, 0, s>>>(g, a, const_cast<double*>(kanchor));
-    if (table) {
-      const double* tab = (const double*)table;
-      const long long* itab = (const long long*)(tab + (size_t)GEO_DOUBLES * total);
-      sommerfeld_fp64_tab_kernel<<<dim3((total + bs - 1) / bs, 6), bs, 0, s>>>(g, a, kanchor, tab, itab);
-    } else {
-      sommerfeld_fp64_kernel<true><<<(total + bs - 1) / bs, bs, 0, s>>>(g, a, kanchor);
-    }
-  } else {
-    sommerfeld_fp64_kernel<false><<<(total + bs - 1) / bs, bs, 0, s>>>(g, a, kanchor);
-  }
+  sommerfeld_anchor_fp64_kernel<<<dim3((ns + bs - 1) / bs, 4), bs, 0, s>>>(g, a, kanchor);
+  const double* tab = (const double*)table;
+  const long long* itab = (const long long*)(tab + (size_t)GEO_DOUBLES * total);
+  sommerfeld_fp64_tab_kernel<<<dim3((total + bs - 1) / bs, 6), bs, 0, s>>>(g, a, kanchor, tab, itab);
   return cudaGetLastError();
 }
 cudaError_t launch_sommerfeld_mixed(const Grid& g, const StageArgsMixed& a, const float* kanchor,
