@@ -99,6 +99,42 @@ inline cudaError_t smem_optin(K kernel, int bytes, std::atomic<unsigned>& done) 
   return e;
 }
 
+// Launch of a kernel that may start while the kernel before it on the stream
+// still runs (programmatic dependent launch): its blocks take free places and
+// wait, in hardware, in after_previous() until that kernel is complete and its
+// writes are visible.  Every thread of such a kernel calls after_previous()
+// before its first access to memory that earlier work writes or reads.  early
+// false, and under stream capture: an ordinary launch.  For the kernels of small
+// float64 grids, a few tens of microseconds each (up to two tiles per SM): a step
+// with periodic boundaries at 24^3 222 -> 204 us, Sommerfeld 8^3 263 -> 232, 24^3
+// 307 -> 294, 32^3 526 -> 515; but 36^3 733 -> 739, and the mixed kernels 48^3 349 ->
+// 434 (their blocks want different splits of shared memory and L1).
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool early,
+                                const A&... args) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (early) {
+    cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = early && cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+// wait for the kernel before this one, and let the one after it start
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename T>
 constexpr bool is_f32 = std::is_same<T, float>::value;
 template <typename T>
@@ -279,6 +315,7 @@ struct Punct {
 cudaError_t launch_stage_fp64(const Grid& g, const StageArgs& a, cudaStream_t s, int cfg = 0,
                               const CUtensorMap* map = nullptr, int* err = nullptr);
 bool fx_tile_fits(const Grid& g);
+bool fx_launch_early(const Grid& g);  // the kernels of a step are short: their launches overlap (launch_after)
 cudaError_t make_fx_tensor_map(const Grid& g, const double* base, CUtensorMap* out);
 cudaError_t launch_stage_fx(const Grid& g, const StageArgs& a, const CUtensorMap& map, int* err, cudaStream_t s);
 cudaError_t launch_stage_mixed(const Grid& g, const StageArgsMixed& a, cudaStream_t s, int cfg = 0);

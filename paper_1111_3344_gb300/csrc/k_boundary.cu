@@ -21,6 +21,7 @@ namespace bssn {
 // blockIdx.y: one of four field groups (W and gt_ij; K and At_ij but its last;
 // the rest of At_ij, Gt^i, alpha; beta^i and B^i)
 __global__ void sommerfeld_anchor_fp64_kernel(Grid g, StageArgs a, double* __restrict__ kanchor) {
+  after_previous();
   const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= shell_count(g)) return;
   switch (blockIdx.y) {
@@ -37,6 +38,7 @@ __global__ void sommerfeld_anchor_fp64_kernel(Grid g, StageArgs a, double* __res
 // at 24^3, 74 at 48^3, 299 at 128^3; so 29, 61, 293).
 __global__ void sommerfeld_fp64_tab_kernel(Grid g, StageArgs a, const double* __restrict__ kanchor,
                                            const double* __restrict__ tab, const long long* __restrict__ itab) {
+  after_previous();
   const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= ghost_count(g)) return;
   switch (blockIdx.y) {  // six groups of four fields
@@ -85,6 +87,7 @@ __global__ void sommerfeld_mixed_kernel(Grid g, StageArgsMixed a, const float* _
 
 template <typename S>
 __global__ void periodic_fill_kernel(Grid g, S* __restrict__ y, double* __restrict__ w) {
+  after_previous();
   const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= ghost_count(g)) return;
   periodic_point<S>(g, y, w, q);
@@ -98,11 +101,13 @@ cudaError_t launch_sommerfeld(const Grid& g, const StageArgs& a, double* kanchor
                               const void* table) {
   const unsigned total = ghost_count(g), ns = shell_count(g);
   const int bs = 128;
-  sommerfeld_anchor_fp64_kernel<<<dim3((ns + bs - 1) / bs, 4), bs, 0, s>>>(g, a, kanchor);
+  cudaError_t e = launch_after(sommerfeld_anchor_fp64_kernel, dim3((ns + bs - 1) / bs, 4), bs, 0, s, fx_launch_early(g), g, a,
+                               kanchor);
+  if (e != cudaSuccess) return e;
   const double* tab = (const double*)table;
   const long long* itab = (const long long*)(tab + (size_t)GEO_DOUBLES * total);
-  sommerfeld_fp64_tab_kernel<<<dim3((total + bs - 1) / bs, 6), bs, 0, s>>>(g, a, kanchor, tab, itab);
-  return cudaGetLastError();
+  return launch_after(sommerfeld_fp64_tab_kernel, dim3((total + bs - 1) / bs, 6), bs, 0, s, fx_launch_early(g), g, a,
+                      kanchor, tab, itab);
 }
 cudaError_t launch_sommerfeld_mixed(const Grid& g, const StageArgsMixed& a, const float* kanchor,
                                     cudaStream_t s) {
@@ -114,8 +119,7 @@ cudaError_t launch_sommerfeld_mixed(const Grid& g, const StageArgsMixed& a, cons
 
 cudaError_t launch_periodic_fill(const Grid& g, double* y, cudaStream_t s) {
   const unsigned total = ghost_count(g);
-  periodic_fill_kernel<double><<<(total + 255) / 256, 256, 0, s>>>(g, y, nullptr);
-  return cudaGetLastError();
+  return launch_after(periodic_fill_kernel<double>, (total + 255) / 256, 256, 0, s, fx_launch_early(g), g, y, nullptr);
 }
 
 cudaError_t launch_periodic_fill_mixed(const Grid& g, float* y, double* w, cudaStream_t s) {

@@ -86,10 +86,13 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
   if (tid == 0) {
     mbar_init(bar0);
     mbar_init(bar1);
-    fx_issue<Sh>(&map, sm.box[grp][0], bar0, ii0, jj0, kk0, fx_field(grp));
     if (grp == 0) sm.fail = 0;
   }
   const int cen = fx_center<Sh>(ii0, jj0, kk0, i, j, k);
+  int* sc = reinterpret_cast<int*>(sm.box[grp][1]) + tid;
+  fx_points<Sh>(g, tid, ii0, jj0, kk0, cen, sc);
+  after_previous();
+  if (tid == 0) fx_issue<Sh>(&map, sm.box[grp][0], bar0, ii0, jj0, kk0, fx_field(grp));
   FxMetric M;  // the first group's
   bool wok = true;
   if (grp == 0) {
@@ -106,8 +109,6 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
     sm.neg[tid] = (neg[0] & 1) | (neg[1] & 2) | (neg[2] & 4);
     wok = aw.ok && gw.ok;
   }
-  int* sc = reinterpret_cast<int*>(sm.box[grp][1]) + tid;
-  fx_points<Sh>(g, tid, ii0, jj0, kk0, cen, sc);
   int at[Sh::PER];
 #pragma unroll
   for (int e = 0; e < Sh::PER; e++) at[e] = sc[e * T];
@@ -225,6 +226,12 @@ cudaError_t make_fx_tensor_map(const Grid& g, const double* base, CUtensorMap* o
 // 24^3 (108 tiles) 0.053 / 0.100, 32^3 (256) 0.099 / 0.133, 36^3 (405) 0.148 / 0.162,
 // 40^3 (500) 0.196 / 0.187.
 constexpr long long FX_WIDE_BLOCKS = 3 * 152;
+static long long fx_tiles(const Grid& g) {
+  return (long long)((g.n0 + FxT::TX - 1) / FxT::TX) * ((g.n1 + FxT::TY - 1) / FxT::TY) *
+         ((g.n2 + FxT::TZ - 1) / FxT::TZ);
+}
+bool fx_launch_early(const Grid& g) { return fx_tiles(g) <= 2 * 152; }
+
 // A tile takes as long with points past the grid as without, 0.73 of the time
 // of the same points one at a time (k_stage.cu: blocks of consecutive points, no
 // padding).  Measured, ms a stage, tile against point form, with the share of
@@ -233,18 +240,16 @@ constexpr long long FX_WIDE_BLOCKS = 3 * 152;
 // With few tiles one block's latency counts, whatever the padding (129 x 5 x 5
 // 0.052 / 0.144, 33^3 with groups 0.144 / 0.147).
 bool fx_tile_fits(const Grid& g) {
-  const long long blocks = (long long)((g.n0 + FxT::TX - 1) / FxT::TX) * ((g.n1 + FxT::TY - 1) / FxT::TY) *
-                           ((g.n2 + FxT::TZ - 1) / FxT::TZ);
-  return blocks <= FX_WIDE_BLOCKS || 100LL * g.n0 * g.n1 * g.n2 >= 72LL * blocks * FxT::THREADS;
+  return fx_tiles(g) <= FX_WIDE_BLOCKS || 100LL * g.n0 * g.n1 * g.n2 >= 72LL * fx_tiles(g) * FxT::THREADS;
 }
 
 cudaError_t launch_stage_fx(const Grid& g, const StageArgs& a, const CUtensorMap& map, int* err, cudaStream_t s) {
   const dim3 grid((g.n0 + FxT::TX - 1) / FxT::TX, (g.n1 + FxT::TY - 1) / FxT::TY, (g.n2 + FxT::TZ - 1) / FxT::TZ);
-  if ((long long)grid.x * grid.y * grid.z <= FX_WIDE_BLOCKS) {
-    stage_fx_wide_kernel<<<grid, GROUPS * FxT::THREADS, sizeof(FxWideShared<FxT>), s>>>(map, g, a, err);
-  } else {
-    stage_fx_kernel<<<grid, FxT::THREADS, 0, s>>>(map, g, a, err);
+  if (fx_tiles(g) <= FX_WIDE_BLOCKS) {
+    return launch_after(stage_fx_wide_kernel, grid, GROUPS * FxT::THREADS, sizeof(FxWideShared<FxT>), s,
+                        fx_launch_early(g), map, g, a, err);
   }
+  stage_fx_kernel<<<grid, FxT::THREADS, 0, s>>>(map, g, a, err);
   return cudaGetLastError();
 }
 
