@@ -50,20 +50,16 @@ DOMAIN = 8.0
 # k-sum (960 each), stage 4 reads the stage value and the k-sum and writes
 # y_n (576); mixed 2496 B, the stage values in float (480 + 768 + 768 + 480).
 # The dominant kernel's roofline uses the mean per stage launch (a quarter).
-# The double-word path moves 8-byte values like float64 but also reads y_n and
-# writes its double-word shadow in stage 4 (576 + 960 + 960 + 960 = 3456 B).
-ALG_BYTES_PER_POINT_STEP = {"fp64": 3072.0, "mixed": 2496.0, "ff": 3456.0}
+# Double-word precision runs the float64 stage.
+ALG_BYTES_PER_POINT_STEP = {"fp64": 3072.0, "mixed": 2496.0, "ff": 3072.0}
 # Float64 work the stage kernels execute per interior point per launch
-# (right-hand side plus RK4 combine), from ncu instruction counts at 64^3
-# (DADD + DMUL + 2 DFMA): the every-stencil kernel 535 DADD + 239 DMUL + 1485
-# DFMA; the full-block kernel (32-wide rows, D_y D_z through shared memory)
-# 299.5 DADD + 246.8 DMUL + 1359.8 DFMA (per warp of 32 points, 1934 warp
-# instructions issued to the float64 pipe).
-FLOP_PER_POINT_RHS = 3744.0
-DPINST_PER_POINT_RHS = 2259.0
-ROWS_TILES = ("32x8x1/1", "32x4x1/1", "32x4x2/1", "32x2x2/2")
-FLOP_PER_POINT_RHS_ROWS = 3265.8
-DPINST_PER_POINT_RHS_ROWS = 1906.0
+# (right-hand side plus RK4 combine), from ncu instruction counts at 96^3
+# (DADD + DMUL + 2 DFMA): the tile form (configuration 32x4x1/1) 62 DADD + 119
+# DMUL + 631 DFMA; the point form 114 DADD + 156 DMUL + 796 DFMA.
+FLOP_PER_POINT_RHS = 1443.0
+DPINST_PER_POINT_RHS = 812.0
+FLOP_PER_POINT_RHS_POINT = 1862.0
+DPINST_PER_POINT_RHS_POINT = 1066.0
 # Operations of one right-hand side at an interior point in the oracle's
 # printed arrangement (its instrumented build, W variant, Gamma-driver shift:
 # 5395 additions, 7874 multiplications, 299 divisions).  The arrangement
@@ -79,9 +75,9 @@ ORACLE_FLOP_PER_POINT_RHS = 5395 + 7874 + 299
 # (where the share of ghosts, padding and L2 hits differs), reports null.
 TRAFFIC_N = 128
 STAGE_TRAFFIC_PER_POINT = {
-    ("fp64", "32x4x1/1"): 937.2,       # stage_fp64_blocks_kernel: 7861.6 MB per step
+    ("fp64", "32x4x1/1"): 4195.0,       # stage_fx_kernel: 35190.8 MB per step, most of it local memory
     ("mixed", "tma32x4x1/2"): 565.3,   # stage_mixed_tma_kernel, 8 staged fields: 4741.9 MB per step
-    ("mixed", "tma11_32x8x1/1"): 565.4,  # stage_mixed_tma_kernel, 11 staged fields: 4742.4 MB per step
+    ("mixed", "tma11_32x8x1/1"): 569.3,  # stage_mixed_tma_kernel, 11 staged fields: 4775.7 MB per step
 }
 # Float64 work per interior point of the analysis kernels (DADD + DMUL + 2 DFMA
 # from ncu instruction counts at 96^3).  psi4 and constraints include the
@@ -108,7 +104,7 @@ FP64_NOMINAL_GFLOPS = 1250.0        # nominal GB300 float64 rate (context only)
 def workload_params(precision="fp64"):
     """The benchmark puncture's parameters in one precision form: fp64, mixed,
     mixed_ks64 (mixed with the k-sum of every field in float64) or ff
-    (double-word right-hand side)."""
+    (double-word precision)."""
     from paper_1111_3344_gb300.bssn import Params
     h = 2 * DOMAIN / N_SIDE
     ks64 = precision == "mixed_ks64"
@@ -434,18 +430,17 @@ def run_ours(args):
     run = puncture_run(args, args.precision, world, local, args.steps)
     pts = N_SIDE ** 3
     mixed = args.precision == "mixed"
-    rows = run["tile"] in ROWS_TILES and N_SIDE % 32 == 0
+    tiled = args.precision == "ff" or run["tile"] == "32x4x1/1"
     if mixed:
         kernel = "stage_mixed_tma_kernel" if run["tile"].startswith("tma") else "stage_mixed_kernel"
         roofline = hbm_roofline(run, "mixed", kernel, STAGE_TRAFFIC_PER_POINT.get(("mixed", run["tile"])))
-    elif args.precision == "ff":
-        roofline = hbm_roofline(run, "ff", "stage_ff_kernel", None)
     else:
-        kernel = "stage_fp64_blocks_kernel" if rows else "stage_fp64_kernel"
-        roofline = hbm_roofline(run, "fp64", kernel, STAGE_TRAFFIC_PER_POINT.get(("fp64", run["tile"])))
+        kernel = "stage_fx_kernel" if tiled else "stage_fp64_kernel"
+        roofline = hbm_roofline(run, args.precision, kernel,
+                                STAGE_TRAFFIC_PER_POINT[("fp64", "32x4x1/1")] if tiled else None)
         peaks = measured_peaks(B, torch, torch.cuda.Stream())
-        flop_pt = FLOP_PER_POINT_RHS_ROWS if rows else FLOP_PER_POINT_RHS
-        dpinst_pt = DPINST_PER_POINT_RHS_ROWS if rows else DPINST_PER_POINT_RHS
+        flop_pt = FLOP_PER_POINT_RHS if tiled else FLOP_PER_POINT_RHS_POINT
+        dpinst_pt = DPINST_PER_POINT_RHS if tiled else DPINST_PER_POINT_RHS_POINT
         sec = run["stage_launch_ms"] * 1e-3
         # the pipe that binds the float64 stage: executed float64 work of a
         # launch over the float64 FMA rate measured in this run
@@ -461,13 +456,12 @@ def run_ours(args):
         roofline["measured_peaks"] = peaks
     line = {
         "metric": {"mixed": "BSSN RK4 point-updates/s (mixed FP32 RHS / FP64 state, Brill-Lindquist puncture 128^3)",
-                   "ff": "BSSN RK4 point-updates/s (double-word FP32 RHS / FP64 state, Brill-Lindquist puncture "
-                         "128^3)"}.get(args.precision,
+                   "ff": "BSSN RK4 point-updates/s (double-word precision, Brill-Lindquist puncture 128^3)"}.get(args.precision,
                                        "BSSN RK4 point-updates/s (FP64, Brill-Lindquist puncture 128^3)"),
         "value": run["value"], "unit": "Mpoint-updates/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": run["ms"] / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None,
-        "dtype": {"mixed": "f32+f64", "ff": "f32x2+f64"}.get(args.precision, "f64"),
+        "dtype": {"mixed": "f32+f64", "ff": "f64"}.get(args.precision, "f64"),
         "data": "synthetic",
         "config": {"workload": "single Brill-Lindquist puncture M=1, 128^3 on [-8,8]^3, W, 1+log, "
                                "Gamma-driver eta=2, Sommerfeld, RK4 dt=0.25h",
@@ -480,7 +474,7 @@ def run_ours(args):
         # the split mixed stage is two kernels per stage (stencils, algebra);
         # a float64 boundary pass is two (anchor pass, ghost points)
         "gpu_launches": run["stage_launches"] * (2 if run["tile"].startswith("split") else 1)
-                        + run["boundary_launches"] * (2 if args.precision == "fp64" else 1),
+                        + run["boundary_launches"] * (2 if args.precision != "mixed" else 1),
         "clocks": run["clocks"],
     }
     if world == 1 and not args.no_extras and args.precision == "fp64":
@@ -568,26 +562,20 @@ def batched_run(args, precision, steps=None, members=None):
     clk = clocks.stop()
     ms = start.elapsed_time(stop)
     pts = sum(p.n[0] * p.n[1] * p.n[2] for p in params)
-    # launches per step: a stage and a boundary launch per RK4 stage; the
-    # one-block-per-tile float64 configurations launch the members with full
-    # tiles and the others separately
+    # launches per step: a stage and a boundary launch per RK4 stage
     tname = list(tile_ms)[best]
     stage_launches, bc_launches = 1, 1
-    if tname.startswith(("tiles", "fftiles")) and precision in ("fp64", "ff"):
-        tx, ty, tz = (int(v) for v in tname.split("tiles")[1].split("/")[0].split("x"))
-        full = [tx == 32 and p.n[0] % 32 == 0 and p.n[1] % ty == 0 and p.n[2] % tz == 0 for p in params]
-        stage_launches = int(any(full)) + int(not all(full))
-    elif tname.startswith("members"):
+    if tname.startswith(("members", "fftiles")):
         # per member and stage: its stage kernel and its Sommerfeld boundary
         # (float64: the anchor pass and the ghost-point pass)
         stage_launches = len(params)
-        bc_launches = len(params) * (2 if precision == "fp64" else 1)
+        bc_launches = len(params) * (2 if precision != "mixed" else 1)
     batch.close()
     del batch
     torch.cuda.empty_cache()
     return {"metric": f"batched BSSN RK4 point-updates/s ({precision})",
             "value": pts * steps / (ms * 1e-3) / 1e6, "unit": "Mpoint-updates/s", "steps": steps,
-            "ms_per_step": ms / steps, "dtype": {"fp64": "f64", "mixed": "f32+f64", "ff": "f32x2+f64"}[precision],
+            "ms_per_step": ms / steps, "dtype": {"fp64": "f64", "mixed": "f32+f64", "ff": "f64"}[precision],
             "workload": f"{len(params)} Brill-Lindquist binaries, grids {{48,64,96,128}}^3, seed 1111, "
                         f"{steps} of the configuration's 100 steps",
             "interior_points": pts, "tile": tname,
@@ -694,7 +682,7 @@ def served_run(args, precision, requests, keep_norms=False):
             "p50_s": float(np.percentile(lats, 50)), "p99_s": p99,
             "p99_queued_s": float(queued[i99]), "mean_queued_s": float(queued.mean()),
             "failed": int(fails), "wall_s": wall, "busy_s": stats["busy_s"],
-            "dtype": {"fp64": "f64", "mixed": "f32+f64", "ff": "f32x2+f64"}[precision],
+            "dtype": {"fp64": "f64", "mixed": "f32+f64", "ff": "f64"}[precision],
             "workload": f"first {len(reqs)} requests of the served stream (seed 3344): Poisson arrivals of "
                         f"Brill-Lindquist binaries, grids 32^3..192^3, 50..400 steps",
             "policy": args.serve_policy,
