@@ -536,10 +536,14 @@ bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs) {
     a.src = src;
     a.rhs = out;
     a.mode = MODE_RHS;
-    // a caller's register is described here, where its address allows it
+    // a caller's register is described here, where its address allows it (also
+    // while the stream is captured; the query binds the thread's context)
     CUtensorMap made;
     const CUtensorMap* map = fx_map(ctx, src);
-    if (!map && (uintptr_t)src % 16 == 0 && make_fx_tensor_map(ctx->g, src, &made) == cudaSuccess) map = &made;
+    cudaStreamCaptureStatus cap;
+    if (!map && ctx->fmap_ok && (uintptr_t)src % 16 == 0 && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess &&
+        make_fx_tensor_map(ctx->g, src, &made, true) == cudaSuccess)
+      map = &made;
     e = launch_stage_fp64(ctx->g, a, ctx->stream, fp64_cfg(ctx, ctx->tile), map, ctx->err);
     if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs interior");
     if (!ctx->g.periodic) {

@@ -70,11 +70,13 @@ PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 using TmaWide = TmaShape<2, 4, 11>;
 }
 
-cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out) {
+cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out,
+                              bool bound) {
   // the encoding is a driver call and needs a current context: a thread whose
   // first CUDA call this is has none until a runtime call binds the primary
-  // context of its device (cudaFree(nullptr) does, and frees nothing)
-  cudaError_t ce = cudaFree(nullptr);
+  // context of its device (cudaFree(nullptr) does, and frees nothing; it is no
+  // call for a stream capture: bound says that one has been made)
+  cudaError_t ce = bound ? cudaSuccess : cudaFree(nullptr);
   if (ce != cudaSuccess) return ce;
   if (!g_encode) {
     cudaDriverEntryPointQueryResult q;

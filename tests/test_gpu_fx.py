@@ -139,3 +139,37 @@ def test_tile_form_equals_the_point_form(n, conformal):
     assert T.rounding_aware_errors(got, want, mag).max() <= 1.0
     assert T.rounding_aware_errors(point, want, mag).max() <= 1.0
     assert T.rounding_aware_errors(got, point, mag).max() <= 2.0
+
+
+@pytest.mark.parametrize("n", [(16, 12, 8), (64, 40, 33)])
+@pytest.mark.parametrize("precision", ["fp64", "ff"])
+def test_captured_calls_equal_direct_ones(n, precision):
+    """Steps and the right-hand side of a caller's register recorded into a graph
+    (ordinary launches, the tensor map made during the capture) give the bits
+    of the direct calls, whose launches overlap on the smaller grid; so does
+    the context's own stream being the default one."""
+    import torch
+    from paper_1111_3344_gb300 import bssn as B
+    c, st = _case(n, 29, precision=precision)
+    evo = B.Evolution(T.gpu_params(c), stream=torch.cuda.Stream())
+    evo.set_state(st)
+    evo.rk4_step(3)
+    want = evo.get_state()[0]
+    reg = evo.numpy_to_register(st)
+    torch.cuda.synchronize()
+    out = torch.zeros_like(reg)
+    B.bssn_rhs(evo.ctx, reg.data_ptr(), out.data_ptr())
+    torch.cuda.synchronize()
+    out2 = torch.zeros_like(reg)
+    evo.set_state(st)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=evo.stream):
+        B.bssn_rhs(evo.ctx, reg.data_ptr(), out2.data_ptr())
+        B.bssn_rk4_step(evo.ctx, 3)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, out2)
+    assert np.array_equal(evo.get_state()[0], want)
+    del graph
+    evo.close()
