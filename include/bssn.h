@@ -311,8 +311,8 @@ bssn_status bssn_set_staging(bssn_ctx* ctx, void* d_mem, size_t bytes);
  * second-differenced fields W, gt_ij and alpha of each tile in shared memory by
  * TMA (two blocks of 32x4 points per SM, or one block of 32x8 points per SM,
  * which leaves more L1 for the other fields); "tma11_32x8x1/1" stages beta^i
- * as well (eleven fields, 141 KB of shared memory, one block of 256 points,
- * 32x2x4, per SM); "split32x4x1/B" (B = 2, 3, 4) run the stencils as one
+ * as well (eleven fields, up to 141 KB of shared memory, one block of 256 points,
+ * 32x2x4 or 16x4x4, per SM); "split32x4x1/B" (B = 2, 3, 4) run the stencils as one
  * pass per field into a derivative register and the algebra as a second pass.
  * A new context starts on the fastest measured configuration of its precision
  * (mixed: "tma11_32x8x1/1"; float64: "32x4x1/1", whose float64 form stages boxes of

@@ -39,7 +39,10 @@ __global__ void __launch_bounds__(Sh::TX * Sh::TY * Sh::TZ, MINB)
   __syncthreads();
   const bool stall = a.stall_polls > 0;  // test hook: no copy, short wait
   if (tid == 0 && !stall) issue_staged_loads<Sh>(&tmap, bar, smem, ii0, jj0, kk0);
-  const int ii = ii0 + threadIdx.x, jj = jj0 + threadIdx.y, kk = kk0 + threadIdx.z;
+  // a warp of a 16-wide tile holds two rows, one above the other in z: their
+  // boxes' rows are 240 floats apart, on different banks (24 apart along y)
+  const int ti = threadIdx.x, tj = Sh::TX == 32 ? threadIdx.y : threadIdx.z, tk = Sh::TX == 32 ? threadIdx.z : threadIdx.y;
+  const int ii = ii0 + ti, jj = jj0 + tj, kk = kk0 + tk;
   const bool inside = ii < g.n0 && jj < g.n1 && kk < g.n2;
   // the combine's inputs, while the boxes are on their way (128^3: 0.848 -> 0.818 ms)
   MixedPre<> pre;
@@ -49,7 +52,6 @@ __global__ void __launch_bounds__(Sh::TX * Sh::TY * Sh::TZ, MINB)
     if (!stall) mbar_wait(bar, 0, WAIT_LIMIT);  // let this block's own copies land before it exits
     return;
   }
-  const int ti = threadIdx.x, tj = threadIdx.y, tk = threadIdx.z;
   if (!inside) return;
   const int i = ii + GH, j = jj + GH, k = kk + GH;
   TileAccT<Sh> acc;
@@ -66,8 +68,23 @@ __global__ void __launch_bounds__(Sh::TX * Sh::TY * Sh::TZ, MINB)
 // ------------------------------------------------------------------ host
 namespace {
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-// variant 2's tile
+// variant 2's tiles
 using TmaWide = TmaShape<2, 4, 11>;
+using TmaHalf = TmaShape<4, 4, 11, 16>;
+template <typename Sh>
+long long tile_count(const Grid& g) {
+  return (long long)((g.n0 + Sh::TX - 1) / Sh::TX) * ((g.n1 + Sh::TY - 1) / Sh::TY) * ((g.n2 + Sh::TZ - 1) / Sh::TZ);
+}
+// Whether variant 2 takes 16-wide tiles.  A block of them takes up to 1.05 of the
+// other's time (128^3 0.822 / 0.792 ms a stage) and leaves fewer threads without a
+// point where n0 is little above a multiple of 32: where both the tiles and the
+// rounds of one tile per SM are fewer by that.  A stage, ms, 16-wide / 32-wide:
+// 40^3 0.035 / 0.046, 48^3 0.052 / 0.064, 80^3 0.219 / 0.243, 112^3 0.565 / 0.605,
+// 66x57x50 0.109 / 0.119; 24^3 (72 tiles either way) 0.0203 / 0.0197.
+bool half_tiles(const Grid& g) {
+  const long long h = tile_count<TmaHalf>(g), w = tile_count<TmaWide>(g);
+  return 21 * h <= 20 * w && 21 * ((h + 151) / 152) <= 20 * ((w + 151) / 152);
+}
 }
 
 cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out,
@@ -97,8 +114,10 @@ cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx,
 }
 
 cudaError_t make_stage_tensor_map(const Grid& g, const float* base, CUtensorMap* out, int variant) {
-  const int by = variant == 2 ? TmaWide::BY : (variant == 1 ? TmaShape<8>::BY : TmaShape<4>::BY);
-  return encode_tensor_map(g, base, 4, TmaDefault::BX, by, variant == 2 ? TmaWide::BZ : TmaShape<4>::BZ, out);
+  if (variant == 2 && half_tiles(g)) return encode_tensor_map(g, base, 4, TmaHalf::BX, TmaHalf::BY, TmaHalf::BZ, out);
+  if (variant == 2) return encode_tensor_map(g, base, 4, TmaWide::BX, TmaWide::BY, TmaWide::BZ, out);
+  return encode_tensor_map(g, base, 4, TmaDefault::BX, variant == 1 ? TmaShape<8>::BY : TmaShape<4>::BY,
+                           TmaShape<4>::BZ, out);
 }
 
 // dynamic shared memory above the default limit, once per kernel and device
@@ -113,7 +132,7 @@ static cudaError_t launch_tma(const Grid& g, const StageArgsMixed& a, const CUte
                               cudaStream_t s) {
   cudaError_t e = tma_attr<Sh, MINB>();
   if (e != cudaSuccess) return e;
-  dim3 block(Sh::TX, Sh::TY, Sh::TZ);
+  dim3 block(Sh::TX, Sh::TX == 32 ? Sh::TY : Sh::TZ, Sh::TX == 32 ? Sh::TZ : Sh::TY);
   dim3 grid((g.n0 + Sh::TX - 1) / Sh::TX, (g.n1 + Sh::TY - 1) / Sh::TY, (g.n2 + Sh::TZ - 1) / Sh::TZ);
   stage_mixed_tma_kernel<Sh, MINB><<<grid, block, Sh::SMEM, s>>>(map, g, a, err);
   return cudaGetLastError();
@@ -122,7 +141,8 @@ static cudaError_t launch_tma(const Grid& g, const StageArgsMixed& a, const CUte
 // variant 0: 32 x 4 x 1 tiles, two blocks per SM; 1: 32 x 8 x 1 tiles, one
 // block per SM (half the shared memory per SM, so more L1 for the fields read
 // through it); 2: 32 x 2 x 4 tiles staging beta^i as well (eleven fields, 141 KB,
-// one block per SM); map: a tensor map made for the same variant.
+// one block per SM; 16 x 4 x 4 where these fit the grid better, half_tiles); map: a
+// tensor map made for the same variant and grid.
 // Variant 2 is bound by the latency of the loads of the other 13 fields with
 // two warps per scheduler: its boxes (40 x 8 x 10) and the planes that those
 // fields' stencils touch are smaller than a 32 x 8 x 1 tile's (40 x 14 x 7, 173
@@ -131,13 +151,16 @@ static cudaError_t launch_tma(const Grid& g, const StageArgsMixed& a, const CUte
 // 6.39 / 6.28, 48^3 0.0648 / 0.0642 / 0.0634 / 0.0645.  Slower: 384 threads (1.09 at 128^3),
 // 512 with 8 fields (0.94), two blocks of 128 (0.84), prefetches to L2 (0.82).
 cudaError_t prepare_stage_mixed_tma(int variant) {
-  if (variant == 2) return tma_attr<TmaWide, 1>();
+  if (variant == 2) {
+    cudaError_t e = tma_attr<TmaHalf, 1>();
+    return e == cudaSuccess ? tma_attr<TmaWide, 1>() : e;
+  }
   return variant == 1 ? tma_attr<TmaShape<8>, 1>() : tma_attr<TmaShape<4>, 2>();
 }
 
 cudaError_t launch_stage_mixed_tma(const Grid& g, const StageArgsMixed& a, const CUtensorMap& map,
                                    int* err, cudaStream_t s, int variant) {
-  if (variant == 2) return launch_tma<TmaWide, 1>(g, a, map, err, s);
+  if (variant == 2) return half_tiles(g) ? launch_tma<TmaHalf, 1>(g, a, map, err, s) : launch_tma<TmaWide, 1>(g, a, map, err, s);
   return variant == 1 ? launch_tma<TmaShape<8>, 1>(g, a, map, err, s) : launch_tma<TmaShape<4>, 2>(g, a, map, err, s);
 }
 

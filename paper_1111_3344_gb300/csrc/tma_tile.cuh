@@ -19,14 +19,14 @@ namespace bssn {
 
 constexpr int NSTAGED = 8;
 
-// Tile of 32 x TY x TZ interior points and its boxes: BX = 32 + 6 rounded up
+// Tile of TX x TY x TZ interior points and its boxes: BX = TX + 6 rounded up
 // to a multiple of 4 floats, BY = TY + 6, BZ = TZ + 6 (three ghost layers on
 // every side); slots of the staged fields 128-byte aligned.  NST: staged
 // fields, 8 (W, gt_ij, alpha) or 11 (and beta^i).
-template <int TY_, int TZ_ = 1, int NST_ = NSTAGED>
+template <int TY_, int TZ_ = 1, int NST_ = NSTAGED, int TX_ = 32>
 struct TmaShape {
-  static constexpr int TX = 32, TY = TY_, TZ = TZ_, NST = NST_;
-  static constexpr int BX = 40, BY = TY + 2 * GH, BZ = TZ + 2 * GH;
+  static constexpr int TX = TX_, TY = TY_, TZ = TZ_, NST = NST_;
+  static constexpr int BX = (TX + 2 * GH + 3) / 4 * 4, BY = TY + 2 * GH, BZ = TZ + 2 * GH;
   static constexpr int BOX = BX * BY * BZ;                              // floats of one field's box
   static constexpr int SLOT = (BOX + 31) / 32 * 32;                     // slot stride
   static constexpr unsigned BYTES = NST * BOX * sizeof(float);         // bytes the copies deliver

@@ -173,3 +173,24 @@ def test_captured_calls_equal_direct_ones(n, precision):
     assert np.array_equal(evo.get_state()[0], want)
     del graph
     evo.close()
+
+
+@pytest.mark.parametrize("n", [(40, 40, 40), (33, 50, 61), (48, 45, 47), (24, 24, 24)])
+@pytest.mark.parametrize("boundary", ["sommerfeld", "periodic"])
+def test_mixed_tile_widths_give_the_same_bits(n, boundary):
+    """The eleven-field mixed stage on 16-wide tiles (the first three grids, whole
+    and partial ones) and 32-wide ones against the fused kernel: the same
+    per-point operations, so the same bits (csrc/k_stage_tma.cu)."""
+    from paper_1111_3344_gb300 import bssn as B
+    c, st = _case(n, 31, precision="mixed", w_fp64_threshold=0.9)
+    c["boundary"] = boundary
+    names = [B.bssn_tile_name(q) for q in range(B.bssn_tile_count())]
+    out = []
+    for tile in ("tma11_32x8x1/1", "32x8x1/1"):
+        evo = B.Evolution(T.gpu_params(c))
+        B.bssn_set_tile(evo.ctx, names.index(tile))
+        evo.set_state(st)
+        evo.rk4_step(2)
+        out.append(evo.get_state()[0])
+        evo.close()
+    assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
