@@ -74,11 +74,20 @@ size_t ghost_table_size(const Grid& g) { return ghost_table_bytes(g); }
 // field after another, the neighbours of each under its own branches: 34 us
 // at 48^3, 175 at 128^3; so 25 and 139).  Interleaving the groups' blocks (31 at
 // 48^3) and fewer registers (40 with 80) are slower.
+// APART: W, with its float64 geometry, in a group of its own (five groups), so
+// that no thread does both one after the other.  Small grids, where the longest
+// thread counts: 24^3 17.1 -> 12.8 us, 32^3 20.0 -> 15.9, 48^3 24.8 -> 22.2; 64^3 39.7 / 39.8,
+// 128^3 139.6 / 149.2 (its neighbours' loads no longer shared).
+template <bool APART>
 __global__ void sommerfeld_mixed_kernel(Grid g, StageArgsMixed a, const float* __restrict__ kanchor) {
   const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= ghost_count(g)) return;
-  switch (blockIdx.y) {
-    case 0: sommerfeld_point_mixed_fields<0, 7, true>(g, a, kanchor, q); break;
+  if (APART && blockIdx.y == 0) {
+    sommerfeld_point_mixed(g, a, kanchor, q, F_CHI);
+    return;
+  }
+  switch (blockIdx.y - (APART ? 1 : 0)) {
+    case 0: sommerfeld_point_mixed_fields<APART ? 1 : 0, 7, true>(g, a, kanchor, q); break;
     case 1: sommerfeld_point_mixed_fields<7, 13, true>(g, a, kanchor, q); break;
     case 2: sommerfeld_point_mixed_fields<13, 18, true>(g, a, kanchor, q); break;
     default: sommerfeld_point_mixed_fields<18, NF, true>(g, a, kanchor, q); break;
@@ -113,7 +122,11 @@ cudaError_t launch_sommerfeld_mixed(const Grid& g, const StageArgsMixed& a, cons
                                     cudaStream_t s) {
   const unsigned total = ghost_count(g);
   const int bs = 128;
-  sommerfeld_mixed_kernel<<<dim3((total + bs - 1) / bs, 4), bs, 0, s>>>(g, a, kanchor);
+  const unsigned blocks = (total + bs - 1) / bs;
+  if (total <= 65536)
+    sommerfeld_mixed_kernel<true><<<dim3(blocks, 5), bs, 0, s>>>(g, a, kanchor);
+  else
+    sommerfeld_mixed_kernel<false><<<dim3(blocks, 4), bs, 0, s>>>(g, a, kanchor);
   return cudaGetLastError();
 }
 
