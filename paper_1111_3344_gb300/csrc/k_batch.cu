@@ -5,7 +5,9 @@
 // search in the work-list prefix sums, its grid and stage arguments are staged
 // in shared memory, and each thread runs the same per-point stage function as
 // the single-grid kernels (stage_point.cuh) -- so a member's result does not
-// depend on which other members share the launch, or on the tile shape.
+// depend on which other members share the launch, or on the tile shape.  (The
+// per-member configurations launch the single-grid kernels; in float64 these
+// run in tiles, equal to the work-list kernels to rounding.)
 #include <cuda_runtime.h>
 
 #include "batch_internal.cuh"
@@ -239,9 +241,9 @@ int batch_tma_variant(int cfg) {
 // Default tile of a new batch (the serving loop keeps it): the fastest
 // configuration of the 64-binary batched workload on GB300, for mixed and
 // float64 batches alike the per-member launches of the single-grid kernels
-// (whole steps over the 64 members: mixed 114.4 ms against 146.5 for the
-// eleven-field persistent TMA kernel; float64 843.8 against 867.8 for
-// tiles32x4x1/2 and 884.4 for the persistent 32x4x1/3).
+// (a stage over the 64 members: mixed 18.4 ms against 22.2 for the eleven-field
+// persistent TMA kernel; float64 87.6 against 96.3 for tiles32x4x1/2 and 108 for
+// the persistent 32x2x2/2).
 int batch_default_tile(bool) { return C_MEMB; }
 bool batch_tile_is_tma(int c) { return batch_tma_variant(c) >= 0; }
 bool batch_tile_is_per_tile(int c) { return (c >= N_FUSED && c < C_TMA); }

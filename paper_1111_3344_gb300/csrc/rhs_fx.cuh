@@ -9,10 +9,10 @@
 // derivatives, the algebra about 830.  The integer work, some 25,000
 // instructions a point, runs beside the float64 pipe.
 //
-// Advection: the lopsided stencil is the mean of the KO sum K and the odd
-//    sum O = 21 (f1 - f-1) - 6 (f2 - f-2) + (f3 - f-3), K + O on the side of
-//    positive beta and K - O on the other; the KO sums of the three axes are
-//    added as integers and scaled once.
+// Advection: the lopsided stencil is the mean of the KO sum K and the odd sum O =
+// 21 (f1 - f-1) - 6 (f2 - f-2) + (f3 - f-3), K + O on the side of positive beta and
+// K - O on the other; the KO sums of the three axes are added as integers and
+// scaled once.
 #pragma once
 #include "bssn_internal.cuh"
 #include "fx.cuh"
