@@ -6,17 +6,21 @@
 // neighbouring values with small whole coefficients, more than half of the
 // float64 instructions of a right-hand side -- are therefore summed as 64-bit
 // integers, and only their results become float64 again:
-//  - the values of one stencil are aligned to the largest exponent E among
-//    them: a value becomes its 53-bit significand times 2^FX_BITS (sign
-//    applied), shifted right by E minus its own exponent;
+//  - the values of a derivative along one axis (of a mixed derivative: all
+//    sixteen) are aligned to the largest exponent E among them: a value becomes
+//    its 53-bit significand times 2^FX_BITS (sign applied), shifted right by E
+//    minus its own exponent;
 //  - the sums of these integers are exact; FX_BITS = 2 leaves the headroom for
 //    the largest coefficient sum, 192 (|sum| < 192 2^55 < 2^63);
 //  - the result is rounded to float64 once.
 // The only other error is the bits shifted out of the values whose magnitude
-// is below a quarter of the stencil's largest: at most 2^-54 of that largest
-// value each, a quarter of the rounding that one float64 addition at its
-// magnitude makes.  Nothing is remembered between stencils or points, so the
-// result depends on the stencil's values alone.
+// is below a quarter of the largest: at most 2^-54 of that largest value each, a
+// quarter of the rounding that one float64 addition at its magnitude makes.
+// (Aligned to the largest value along all three axes, three points away as well,
+// a derivative lost the bits by which values that it does not use are larger; a
+// right-hand side one point at a time took 1 to 2 % less.)  Nothing is remembered
+// between stencils or points, so the result depends on the stencil's values
+// alone.  (The stage in tiles, rhs_fx_tile.cuh, aligns a box of a field at once.)
 //
 // Stencils that hold an infinity, a NaN, or only values so small or so large
 // that the result's exponent would leave the normal range take the same sums
@@ -27,6 +31,36 @@
 namespace bssn {
 
 constexpr int FX_BITS = 2;
+
+// Shifts by any count: 64 and more leave 0, or the sign.  (The C++ forms are for
+// tests of this header on the host.)
+__device__ __forceinline__ unsigned long long fx_shl(unsigned long long v, int n) {
+#ifdef __CUDA_ARCH__
+  unsigned long long r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+#else
+  return (unsigned)n > 63u ? 0 : v << n;
+#endif
+}
+__device__ __forceinline__ unsigned long long fx_shr(unsigned long long v, int n) {
+#ifdef __CUDA_ARCH__
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+#else
+  return (unsigned)n > 63u ? 0 : v >> n;
+#endif
+}
+__device__ __forceinline__ long long fx_sar(long long v, int n) {
+#ifdef __CUDA_ARCH__
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+#else
+  return v >> ((unsigned)n > 63u ? 63 : n);
+#endif
+}
 
 // largest high word (sign cleared) of the values: its top 11 bits are the
 // largest biased exponent
@@ -57,8 +91,7 @@ __device__ __forceinline__ long long fx_from(double v, int E) {
   const int sh = E - ((hi >> 20) & 0x7ff);
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
   const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)lo) << BITS;
-  unsigned long long r;
-  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(sh));  // shifts of 64 and more give 0
+  const unsigned long long r = fx_shr(m, sh);
   const long long s = hi >> 31;
   return (long long)((r ^ (unsigned long long)s) - (unsigned long long)s);
 }
@@ -70,9 +103,7 @@ __device__ __forceinline__ long long fx_near(double v, int E) {
   const int sh = E - ((hi >> 20) & 0x7ff);
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
   const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)lo) << (BITS + 1);
-  unsigned long long r;
-  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(sh));
-  r = (r + 1) >> 1;
+  const unsigned long long r = (fx_shr(m, sh) + 1) >> 1;
   const long long s = hi >> 31;
   return (long long)((r ^ (unsigned long long)s) - (unsigned long long)s);
 }
@@ -82,8 +113,7 @@ __device__ __forceinline__ double fx_to(long long s, int E) {
   const int neg = (int)(s >> 63);
   const unsigned long long a = (unsigned long long)((s ^ (long long)neg) - (long long)neg);
   const int n = __clzll((long long)a);
-  unsigned long long b;
-  asm("shl.b64 %0, %1, %2;" : "=l"(b) : "l"(a), "r"(n));  // leading bit to bit 63 (0 stays 0)
+  const unsigned long long b = fx_shl(a, n);  // leading bit to bit 63 (0 stays 0)
   const unsigned long long r = (b >> 11) + ((b >> 10) & 1ull);
   // exponent of the leading bit: E + 11 - FX_BITS - n; r's own leading bit adds one
   const unsigned ex = (unsigned)(E + 10 - FX_BITS - n) << 20;
@@ -187,14 +217,13 @@ __device__ __forceinline__ void fx_axes(const double* p, long long sy, long long
   }
   const unsigned top = fx_top(v);
   if (fx_ok(top)) {
-    const int E = (int)(top >> 20);
-    const long long f0 = SECOND ? fx_from(v[0], E) : 0;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-      const long long a = fx_from(v[1 + 4 * d], E), b = fx_from(v[2 + 4 * d], E), c = fx_from(v[3 + 4 * d], E),
-                      e = fx_from(v[4 + 4 * d], E);
+      const double ax[5] = {v[0], v[1 + 4 * d], v[2 + 4 * d], v[3 + 4 * d], v[4 + 4 * d]};
+      const int E = max((int)(fx_top(ax) >> 20), 256);
+      const long long a = fx_from(ax[1], E), b = fx_from(ax[2], E), c = fx_from(ax[3], E), e = fx_from(ax[4], E);
       d1[d] = fx_to(8 * (c - b) - (e - a), E + up);
-      if (SECOND) d2[d] = fx_to(3 * (16 * (c + b) - (e + a) - 30 * f0), E + 2 + up);
+      if (SECOND) d2[d] = fx_to(3 * (16 * (c + b) - (e + a) - 30 * fx_from(ax[0], E)), E + 2 + up);
     }
     return;
   }

@@ -5,14 +5,13 @@
 //
 // Bound: the float64 pipe, 64 cycles of an SM sub-partition for a warp
 // instruction.  With the stencils in float64 a point took 1906 of them; here
-// the stencils leave 4 per field (advection and dissipation) and none for the
+// the stencils leave 6 per field (advection and dissipation) and none for the
 // derivatives, the algebra about 830.  The integer work, some 25,000
 // instructions a point, runs beside the float64 pipe.
 //
 // Advection: the lopsided stencil is the mean of the KO sum K and the odd sum O =
 // 21 (f1 - f-1) - 6 (f2 - f-2) + (f3 - f-3), K + O on the side of positive beta and
-// K - O on the other; the KO sums of the three axes are added as integers and
-// scaled once.
+// K - O on the other.
 #pragma once
 #include "bssn_internal.cuh"
 #include "fx.cuh"
@@ -26,6 +25,18 @@ struct FxAdv {
   double bh[3], kap;
   int neg[3];
 };
+// of the point c0 of field 0; i12h = 1/(12h), kap = eps / (64h)
+__device__ __forceinline__ FxAdv fx_adv(const double* __restrict__ c0, long long fs, double i12h, double kap) {
+  FxAdv w;
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    const double b = __ldg(c0 + (F_BETA + d) * fs);
+    w.bh[d] = fabs(b) * (0.5 * i12h);
+    w.neg[d] = __double2hiint(b) >> 31;
+  }
+  w.kap = kap;
+  return w;
+}
 
 // The sums along the three axes of the field at p (strides 1, sy, sz): returns
 // sum_d bh[d] (K_d + sign_d O_d) + kap sum_d K_d, upwinded advection plus KO
@@ -49,26 +60,30 @@ __device__ __forceinline__ double fx_axes(const double* p, long long sy, long lo
 #pragma unroll
   for (int d = 0; d < 3; d++) d1[d] = d2[d] = 0.0;
   if (fx_ok(top)) {
-    const int E = (int)(top >> 20);
-    const long long f0 = fx_from(v[0], E);
-    long long K = 0;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
+      // the derivatives' five values in units of their own largest, the sums
+      // with the third neighbours in units of all seven's
+      const double* x = v + 6 * d;
+      const double in[5] = {v[0], x[1], x[2], x[3], x[4]}, far[2] = {x[5], x[6]};
+      const int Ei = max((int)(fx_top(in) >> 20), 256), E = max((int)(fx_top(far) >> 20), Ei);
+      const long long f0 = fx_from(v[0], Ei);
       long long sm[3], df[3];
 #pragma unroll
       for (int m = 0; m < 3; m++) {
-        const long long a = fx_from(v[6 * d + 2 * m + 1], E), b = fx_from(v[6 * d + 2 * m + 2], E);
+        const long long a = fx_from(x[2 * m + 1], m < 2 ? Ei : E), b = fx_from(x[2 * m + 2], m < 2 ? Ei : E);
         sm[m] = b + a;
         df[m] = b - a;
       }
-      if (order >= 1) d1[d] = fx_to(8 * df[0] - df[1], E + up);
-      if (order == 2) d2[d] = fx_to(3 * (16 * sm[0] - sm[1] - 30 * f0), E + 2 + up);
-      const long long k = 15 * sm[0] - 6 * sm[1] + sm[2] - 20 * f0, o = 21 * df[0] - 6 * df[1] + df[2];
+      if (order >= 1) d1[d] = fx_to(8 * df[0] - df[1], Ei + up);
+      if (order == 2) d2[d] = fx_to(3 * (16 * sm[0] - sm[1] - 30 * f0), Ei + 2 + up);
+      const long long k = fx_sar(15 * sm[0] - 6 * sm[1] - 20 * f0, E - Ei) + sm[2];
+      const long long o = fx_sar(21 * df[0] - 6 * df[1], E - Ei) + df[2];
       const long long s = w.neg[d];
-      K += k;
       r = fma(w.bh[d], fx_to(k + ((o ^ s) - s), E), r);
+      r = fma(w.kap, fx_to(k, E), r);
     }
-    return fma(w.kap, fx_to(K, E), r);
+    return r;
   }
   if (fx_zero(v)) return 0.0;
   const double sc = up ? 0.5 : 1.0;
@@ -157,14 +172,7 @@ __device__ __forceinline__ void rhs_fx(const Grid& g, const double* __restrict__
   const double u = g.i12h;
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
 
-  FxAdv w;
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-    const double b = __ldg(c0 + (F_BETA + d) * fs);
-    w.bh[d] = fabs(b) * (0.5 * u);
-    w.neg[d] = __double2hiint(b) >> 31;
-  }
-  w.kap = g.kos;
+  const FxAdv w = fx_adv(c0, fs, u, g.kos);
 
   FxMetric M;
   fx_metric(g, c0, M);

@@ -1,0 +1,58 @@
+"""The float64 right-hand side is as exact beside large values as without them:
+aligning a stencil's values to the largest among several (csrc/fx.cuh) must not
+cost a derivative the bits by which values that it does not use exceed its own.
+
+Bars.  A stencil's values are held to 2^-54 of their largest or better and its sums
+to a few 2^-53, so a point's right-hand side is off by some hundred times 2^-53 M,
+M the oracle's magnitude of the same expression at the same point: 1e-12 M has
+a factor of 30 to spare.  The grids run both forms of the stage in tiles (up to
+456 tiles with groups of threads, from there without)."""
+import numpy as np
+import pytest
+
+import cases as T
+import oracle as O
+from paper_1111_3344_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+GRIDS = [(24, 20, 16), (74, 21, 36), (64, 32, 32)]  # 60, 540 and 512 tiles
+
+
+def _rhs(c, st, point_form=False):
+    """One right-hand side; point_form: of a register that no tensor load can
+    describe (8-byte aligned), which is taken one point at a time."""
+    import torch
+    from paper_1111_3344_gb300.bssn import Evolution
+    evo = Evolution(T.gpu_params(c))
+    reg = evo.numpy_to_register(st)
+    if point_form:
+        odd = torch.empty(reg.numel() + 1, dtype=reg.dtype, device=reg.device)[1:].view(reg.shape)
+        odd.copy_(reg)
+        reg = odd
+    out = evo.register_to_numpy(evo.rhs(reg))
+    evo.close()
+    return out
+
+
+def _interior(n):
+    return np.array([(i, j, k) for k in range(3, 3 + n[2]) for j in range(3, 3 + n[1]) for i in range(3, 3 + n[0])],
+                    dtype=np.int32)
+
+
+@pytest.mark.parametrize("form", ["point"])
+@pytest.mark.parametrize("n", GRIDS[:2])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_large_values_three_points_away(n, axis, form):
+    """A lapse that is 1e6 larger from some index of an axis on: three points
+    before it only the advection and dissipation of the lapse itself read the
+    large values; every other field's right-hand side does not."""
+    c = dict(n=n, xmin=(-0.9, -1.1, -0.7), h=0.11, boundary="sommerfeld")
+    st = inputs.random_state(43, n, c["xmin"], c["h"], amp=0.05)
+    at = 3 + n[axis] // 2 + 1
+    st[(17,) + tuple(slice(at, None) if 2 - d == axis else slice(None) for d in range(3))] += 1e6
+    ijk = np.array([q for q in _interior(n) if q[axis] == at - 3], dtype=np.int32)
+    cfg = T.oracle_cfg(c)
+    want, mag = O.rhs_points_ext(cfg, st, ijk).T, O.rhs_points_mag(cfg, st, ijk)[1].T
+    got = _rhs(c, st, form == "point")[:, ijk[:, 2], ijk[:, 1], ijk[:, 0]]
+    assert (np.abs(got - want) <= 1e-12 * mag).all(), (np.abs(got - want) / mag).max(axis=1)
