@@ -81,7 +81,7 @@ __device__ __forceinline__ bool fx_zero(const double (&v)[N]) {
 }
 // biased exponents 256 .. 1900: every value below 2^-64 of the largest shifts
 // out whole (so a subnormal's missing leading bit never shows), and no result
-// overflows or underflows, products with weights (FxWeights) included
+// overflows or underflows, products with weights (fx_weight) included
 __device__ __forceinline__ bool fx_ok(unsigned top) { return (top >> 20) - 256u <= 1900u - 256u; }
 
 // v in units of 2^(E - 1075 - BITS), E the biased exponent of top
@@ -121,38 +121,42 @@ __device__ __forceinline__ double fx_to(long long s, int E) {
   return __hiloint2double((int)hi, (int)(unsigned)r);
 }
 
-// Weights of a point (float64) for sums over stencil results: fixed point in
-// units of 2^(E - 1083), the largest in [2^60, 2^61).
-template <int N>
-struct FxWeights {
-  long long w[N];
-  int E;
-  bool ok;  // exponent within 2^-50 .. 2^60 (or all zero)
-};
-template <int N>
-__device__ __forceinline__ FxWeights<N> fx_weights(const double (&v)[N]) {
-  FxWeights<N> r;
-  const unsigned top = fx_top(v);
-  r.E = top ? (int)(top >> 20) : 1023;
-  r.ok = (unsigned)(r.E - 973) <= 110u;
-#pragma unroll
-  for (int q = 0; q < N; q++) r.w[q] = top ? fx_from<8>(v[q], r.E) : 0;
-  return r;
+// Weights of a point for sums of products with stencil results: the significand
+// times 2^9 (below 2^62) plus, in the low nine bits, the biased exponent less 831;
+// 0 for a weight of zero.  False for exponents outside 895 .. 1123 (2^-128 ..
+// 2^100), with which a result could leave the normal range.
+__device__ __forceinline__ bool fx_weight(double v, long long& w) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)lo) << 9;
+  const long long s = hi >> 31;
+  const bool zero = ((hi & 0x7fffffff) | lo) == 0;
+  w = zero ? 0 : (long long)((m ^ (unsigned long long)s) - (unsigned long long)s) + (e - 831);
+  return zero || (unsigned)(e - 895) <= 228u;
 }
-
-// sum_q a[q] w[q], a in units of 2^(Ea - 1075 - FX_BITS): the a are shifted up
-// together to their full width, so each truncated product is off by at most
-// 2^-60 of the largest a times the largest weight.
+// sum_q a[q] w[q], a in units of 2^(E - 1075 - FX_BITS): each a is shifted up to
+// its full width, each product aligned to the largest one, and the sum rounded
+// once more: off by at most 2^-56 of the largest product, as good as four
+// float64 multiply-adds, which would hold the float64 pipe.  (Aligned to the
+// largest weight and the largest a instead, a small weight beside a large one
+// loses its last bits where only its a is large.)
 template <int N>
-__device__ __forceinline__ double fx_dot(const long long (&a)[N], int Ea, const FxWeights<N>& w) {
-  unsigned long long m = 0;
+__device__ __forceinline__ double fx_dot(const long long (&a)[N], int E, const long long (&w)[N]) {
+  static_assert(N <= 4, "the sum of |products| stays below 2^63");
+  long long p[N];
+  int t[N], T = -2048;
 #pragma unroll
-  for (int q = 0; q < N; q++) m |= (unsigned long long)(a[q] ^ (a[q] >> 63));
-  const int n = __clzll((long long)m) - 1;  // |a| < 2^63: n >= 0
+  for (int q = 0; q < N; q++) {
+    const int n = __clzll(a[q] ^ (a[q] >> 63));  // 1 .. 64, 64: a is 0 or -1
+    p[q] = __mul64hi((long long)fx_shl((unsigned long long)a[q], n - 1), w[q] & ~511ll);
+    t[q] = ((int)w[q] & 511) - n - (a[q] == 0 ? 1024 : 0);  // a zero has no exponent
+    T = max(T, t[q]);
+  }
   long long s = 0;
 #pragma unroll
-  for (int q = 0; q < N; q++) s += __mul64hi(a[q] << n, w.w[q]);
-  return fx_to(s, Ea - n + w.E - 1019);
+  for (int q = 0; q < N; q++) s += fx_sar(p[q], T - t[q]);
+  return fx_to(s, E + T - 188);
 }
 
 // 144 h^2 d_a d_b of the field at p (strides sa, sb; a != b) times 2^up, up 0 or -1.

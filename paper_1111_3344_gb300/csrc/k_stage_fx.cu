@@ -1,14 +1,14 @@
 // Float64 fused stage in tiles (rhs_fx_tile.cuh): one block per tile of 8 x 4 x 4
 // interior points, one thread per point.
 //
-// Bound: the float64 pipe (860 instructions of 64 cycles for a warp's points:
-// 55 thousand of the 68 thousand cycles a sub-partition takes), the integer
-// stencils beside it.  Shape and occupancy: six blocks of 128 threads per SM (80
-// registers, 33 KB of shared memory each).  A stage at 128^3: 3.51-3.65 ms (a
-// step 15.1; one point at a time 19.7, before that with float64 stencils 33.1);
-// with 4, 5, 7, 8 blocks 4.1, 3.8, 3.6, 3.7; tiles of 16 x 4 x 2 3.65, 16 x 2 x 4
-// 3.68, 8 x 8 x 2 3.60, 8 x 8 x 4 3.95, 32 x 2 x 2 4.4 (a flatter tile converts
-// more box points per tile point); one point at a time (k_stage.cu) 4.6.
+// Bound: the float64 pipe (some 870 instructions of 64 cycles for a warp's
+// points), the integer stencils beside it.  Shape and occupancy: six blocks of 128
+// threads per SM (80 registers, 33 KB of shared memory each).  A step at 128^3
+// 15.7 ms; one point at a time 19.7, before that with float64 stencils 33.1.
+// Found with slightly cheaper sums (a stage then 3.51-3.65 ms): with 4, 5, 7, 8
+// blocks 4.1, 3.8, 3.6, 3.7; tiles of 16 x 4 x 2 3.65, 16 x 2 x 4 3.68, 8 x 8 x 2
+// 3.60, 8 x 8 x 4 3.95, 32 x 2 x 2 4.4 (a flatter tile converts more box points per
+// tile point); one point at a time (k_stage.cu) 4.6.
 //
 // The waits for the tensor loads are bounded: a block whose wait runs out sets
 // the error word (read back by the host as BSSN_ETIMEOUT), waits once more,
@@ -50,10 +50,10 @@ template <typename Sh>
 struct FxWideShared {
   alignas(128) long long box[GROUPS][2][(Sh::BOX + 15) / 16 * 16];
   unsigned long long bar[GROUPS][2];
-  long long wt[10][Sh::THREADS];
+  double wt[10][Sh::THREADS];
   double slot[77][Sh::THREADS];  // of fx_stencils: gt_ij 0 (4 each), Gt^i 24 (3), phi|W, alpha 33 (10), beta^i 53 (7), K 74
   double out[NF][Sh::THREADS];
-  int we[Sh::THREADS], ge[Sh::THREADS], neg[Sh::THREADS];  // exponents of the weights, signs of beta
+  int neg[Sh::THREADS];  // signs of beta
   unsigned top[GROUPS][Sh::WARPS];
   int fail;
 };
@@ -94,28 +94,21 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
   after_previous();
   if (tid == 0) fx_issue<Sh>(&map, sm.box[grp][0], bar0, ii0, jj0, kk0, fx_field(grp));
   FxMetric M;  // the first group's
-  bool wok = true;
   if (grp == 0) {
     int neg[3];
-    const FxWeights<4> aw = fx_tile_adv(g, c0, neg);
     fx_metric(g, c0, M);
-    const FxWeights<6> gw = fx_tile_gu(M);
-#pragma unroll
-    for (int m = 0; m < 4; m++) sm.wt[m][tid] = aw.w[m];
-#pragma unroll
-    for (int m = 0; m < 6; m++) sm.wt[4 + m][tid] = gw.w[m];
-    sm.we[tid] = aw.E;
-    sm.ge[tid] = gw.E;
-    sm.neg[tid] = (neg[0] & 1) | (neg[1] & 2) | (neg[2] & 4);
-    wok = aw.ok && gw.ok;
+    const bool ok = fx_tile_weights<Sh>(g, c0, M, &sm.wt[0][tid], neg);
+    sm.neg[tid] = (neg[0] & 1) | (neg[1] & 2) | (neg[2] & 4) | (ok ? 8 : 0);
   }
   int at[Sh::PER];
 #pragma unroll
   for (int e = 0; e < Sh::PER; e++) at[e] = sc[e * T];
-  wok = __syncthreads_and(wok);  // (and the weights and barriers are there)
-  const int wE = sm.we[tid], gwE = sm.ge[tid], sg = sm.neg[tid];
+  __syncthreads();  // the weights and barriers are there
+  const int sg = sm.neg[tid];
+  const bool wok = sg & 8;
   const int neg[3] = {-(sg & 1), -(sg >> 1 & 1), -(sg >> 2 & 1)};
   auto S = [&](int n) -> double& { return sm.slot[n][tid]; };
+  const double* wt = &sm.wt[0][tid];
 
   double X[6], G2[3][6], V2[3], vj[3], lap = 0.0;
   // rounds 0-2: fields 0 .. 11, one per group; then the first group does the
@@ -150,12 +143,12 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
     unsigned top = sm.top[grp][0];
 #pragma unroll
     for (int n = 1; n < Sh::WARPS; n++) top = max(top, sm.top[grp][n]);
-    bool ok = fx_ok(top) && wok;
+    bool ok = fx_ok(top);
     if (top == 0) {
       unsigned lo = 0;
 #pragma unroll
       for (int e = 0; e < Sh::PER; e++) lo |= (unsigned)__double2loint(x[e]);
-      ok = group_and(1 + grp, T, lo == 0) && wok;
+      ok = group_and(1 + grp, T, lo == 0);
     }
     const int E = max((int)(top >> 20), 256) + FX_BITS - FX_TILE_BITS;
     if (ok) {
@@ -163,15 +156,12 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
       for (int e = 0; e < Sh::PER; e++) box[at[e]] = fx_near<FX_TILE_BITS>(x[e], E + FX_TILE_BITS - FX_BITS);
     }
     group_and(1 + grp, T, true);
-    double r;
-    if (ok) {
-      r = fx_stencils<Sh>(c, q, order, up, E, &sm.wt[0][tid], wE, gwE, neg, S, s0);
-    } else {
-      FxMetric Mc;
-      fx_metric(g, c0, Mc);
-      r = fx_stencils_f64<Sh>(g, c0, Mc, reinterpret_cast<const double*>(c), q, order, up, S, s0);
-    }
     const int f = fx_field(q);
+    double r = 0.0;
+    if (ok && wok)
+      r = fx_stencils<Sh>(c, q, order, up, E, wt, neg, S, s0);
+    else
+      r = fx_stencils_own<Sh>(c0, fs, g.pitch, g.plane, g.i12h, g.kos, q, order, up, wt, S, s0);
     sm.out[f][tid] = f < nf ? r : 0.0;
   }
   if (grp == 0) {

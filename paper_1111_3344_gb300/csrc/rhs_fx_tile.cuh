@@ -11,14 +11,14 @@
 //  - Each thread finds the exponents of its share of the points that stencils
 //    read, the block their maximum, and each thread turns its share into
 //    integers in place, rounded to FX_TILE_BITS bits below the last of the box's
-//    largest value: off by at most 2^-57 of it.  (Sums: |value| <= 2^56, the
-//    largest coefficient sum 120 -- the pure second derivatives without their
-//    factor 3, the mixed ones quartered, half the three axes' KO sum.)
+//    largest value.  (Sums: |value| < 2^57; the largest sum of coefficients is
+//    64 -- the pure second derivatives without their factor 3, the mixed ones an
+//    eighth, half the upwind sum of an axis, a quarter of the axes' KO sum.)
 //  - A thread then reads its taps (67 for a twice-differenced field) with fixed
-//    offsets and no conversion.  Advection, dissipation and the contraction
-//    gt^kl d_k d_l are sums of four and six products with weights of the point,
-//    kept as 64-bit integers too (FxWeights: off by at most 2^-60 of the largest
-//    product): 860 float64 instructions a point.
+//    offsets and no conversion.  Advection and dissipation are one sum of four
+//    products with weights of the point, kept as integers too (fx_weight,
+//    fx_dot); the contraction gt^kl d_k d_l is float64: some 870 float64
+//    instructions a point.
 //  - The algebra runs inside the loop as soon as its fields are there, so that
 //    few results wait at a time (33 local slots).
 // The stencil code exists once: the instruction cache holds 128 KB, and a
@@ -28,11 +28,12 @@
 #pragma once
 #include "fx.cuh"
 #include "fx_algebra.cuh"
+#include "rhs_fx.cuh"
 #include "tma.cuh"
 
 namespace bssn {
 
-constexpr int FX_TILE_BITS = 3;
+constexpr int FX_TILE_BITS = 4;
 
 // Tile of TX x TY x TZ interior points, one per thread, and its box: the tile
 // plus three points on every side.  TX and the box's x extent are even (tensor
@@ -89,13 +90,13 @@ struct FxTile {
   }
 };
 // Shared memory of a block: two boxes (one field's values, then integers; the
-// next field's on their way) and their barriers, each thread's advection (4)
+// next field's on their way) and their barriers, each thread's advection (3)
 // and contraction (6) weights, each warp's largest high word.
 template <typename Sh>
 struct FxShared {
   alignas(128) long long box[2][(Sh::BOX + 15) / 16 * 16];
   unsigned long long bar[2];
-  long long wt[10][Sh::THREADS];
+  double wt[10][Sh::THREADS];
   unsigned top[Sh::WARPS];
 };
 
@@ -106,50 +107,6 @@ __device__ __forceinline__ void fx_issue(const void* map, void* box, unsigned ba
   fence_async_proxy();
   mbar_expect(bar, Sh::BOX * 8);
   tensor_load_4d(box, map, x, y, z, f, bar);
-}
-
-// advection and dissipation weights of the point c0: |beta^d| / (24h), eps /
-// (64h), and the signs of beta as masks
-__device__ __forceinline__ void fx_adv_weights(const Grid& g, const double* __restrict__ c0, double wd[4], int neg[3]) {
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-    const double b = __ldg(c0 + (F_BETA + d) * g.fstride);
-    wd[d] = fabs(b) * (0.5 * g.i12h);
-    neg[d] = __double2hiint(b) >> 31;
-  }
-  wd[3] = g.kos;
-}
-
-// The float64 forms of a field's stencils at c, for boxes outside the integer
-// range (fx_ok): a call of its own, cold code kept out of the loop's
-// instructions.  up: the metric's and Gt's derivatives are halved.
-static __device__ __noinline__ double fx_field_f64(const double* c, int sy, int sz, const double wd[4], const int neg[3],
-                                                   int up, double d1[3], double dd[6]) {
-  const double sc = up ? 0.5 : 1.0;
-  double r = 0.0;
-#pragma unroll 1
-  for (int d = 0; d < 3; d++) {
-    const int s = d == 0 ? 1 : (d == 1 ? sy : sz), m = d == 0 ? 0 : (d == 1 ? 3 : 5);
-    const double a1 = c[-s], b1 = c[s], a2 = c[-2 * s], b2 = c[2 * s], a3 = c[-3 * s], b3 = c[3 * s];
-    d1[d] = sc * fma(8.0, b1 - a1, -(b2 - a2));
-    dd[m] = 12.0 * sc * fma(-30.0, c[0], fma(16.0, b1 + a1, -(b2 + a2)));
-    const double k = fma(15.0, b1 + a1, fma(-6.0, b2 + a2, b3 + a3)) - 20.0 * c[0];
-    const double o = fma(21.0, b1 - a1, fma(-6.0, b2 - a2, b3 - a3));
-    r = fma(wd[d], neg[d] ? k - o : k + o, r);
-    r = fma(wd[3], k, r);
-  }
-#pragma unroll 1
-  for (int m = 0; m < 3; m++) {  // xy, xz, yz
-    const int sa = m < 2 ? 1 : sy, sb = m == 0 ? sy : sz;
-    double l[4];
-#pragma unroll 1
-    for (int q = 0; q < 4; q++) {
-      const double* p = c + (q < 2 ? q - 2 : q - 1) * sa;
-      l[q] = fma(8.0, p[sb] - p[-sb], -(p[2 * sb] - p[-2 * sb]));
-    }
-    dd[m == 0 ? 1 : 2 * m] = sc * fma(8.0, l[2] - l[1], -(l[3] - l[0]));
-  }
-  return r;
 }
 
 // Box points of thread tid (of Sh::THREADS) as offsets from the box's start, for
@@ -185,20 +142,25 @@ __device__ __forceinline__ void fx_points(const Grid& g, int tid, int ii0, int j
   }
 }
 
-// Fixed-point weights of a point: advection and dissipation (|beta^d| / (24h) and
-// eps / (32h), for half the axes' KO sum), and gt^kl, doubled off the diagonal,
-// times the 3 that the pure sums leave out on it.
-__device__ __forceinline__ FxWeights<4> fx_tile_adv(const Grid& g, const double* __restrict__ c0, int neg[3]) {
-  double wd[4];
-  fx_adv_weights(g, c0, wd, neg);
-  wd[3] *= 2.0;
-  return fx_weights(wd);
-}
-__device__ __forceinline__ FxWeights<6> fx_tile_gu(const FxMetric& M) {
-  double v[6];
+// Weights of a point into wt (stride Sh::THREADS): |beta^d| / (24h) 0-2, gt^kl
+// doubled off the diagonal 3-8; neg: signs of beta as masks.
+template <typename Sh>
+__device__ __forceinline__ bool fx_tile_weights(const Grid& g, const double* __restrict__ c0, const FxMetric& M,
+                                                double* wt, int neg[3]) {
+  bool ok = true;
+  long long x;
 #pragma unroll
-  for (int m = 0; m < 6; m++) v[m] = ((m == 0 || m == 3 || m == 5) ? 3.0 : 2.0) * M.gu[m];
-  return fx_weights(v);
+  for (int d = 0; d < 3; d++) {
+    const double b = __ldg(c0 + (F_BETA + d) * g.fstride);
+    ok = fx_weight(fabs(b) * (0.5 * g.i12h), x) && ok;
+    wt[d * Sh::THREADS] = __longlong_as_double(x);
+    neg[d] = __double2hiint(b) >> 31;
+  }
+  ok = fx_weight(2.0 * g.kos, x) && ok;
+  wt[9 * Sh::THREADS] = __longlong_as_double(x);
+#pragma unroll
+  for (int m = 0; m < 6; m++) wt[(3 + m) * Sh::THREADS] = M.g2u(m);
+  return ok;
 }
 
 // Fields in the order of the loop, q: gt_ij, Gt^i | phi|W, alpha | beta^i, K,
@@ -211,11 +173,25 @@ __device__ __forceinline__ int fx_field(int q) {
 }
 __device__ __forceinline__ int fx_order(int q) { return (q < 6 || (q > 8 && q < 14)) ? 2 : (q < 15 ? 1 : 0); }
 __device__ __forceinline__ int fx_up(int q) { return q < 9 ? -1 : 0; }
-// component of the m-th second derivative kept of field q: all six of phi|W and
-// alpha (q = 9, 10), the three d_k d_a of beta^a (q = 11 + a)
-__device__ __forceinline__ int fx_kept(int q, int m) {
-  const int a = q - 11;
-  return q < 11 ? m : (a == 0 ? m : (m == 0 ? a : (a == 1 ? m + 2 : m + 3)));
+// Second derivatives of field q into slots: their contraction with gt^kl into
+// s0 + 3, those kept after it (all six of phi|W and alpha, q = 9 and 10; the
+// three d_k d_a of beta^a, q = 11 + a).
+template <typename Sh, typename Slots>
+__device__ __forceinline__ void fx_second(const double dd[6], int q, const double* wt, Slots S, int s0) {
+  if (q != 9) {  // phi|W's is not used
+    double t = 0.0;
+#pragma unroll
+    for (int m = 0; m < 6; m++) t = fma(wt[(3 + m) * Sh::THREADS], dd[m], t);
+    S(s0 + 3) = t;
+  }
+  if (q > 10) {
+    S(s0 + 4) = q == 11 ? dd[0] : (q == 12 ? dd[1] : dd[2]);
+    S(s0 + 5) = q == 11 ? dd[1] : (q == 12 ? dd[3] : dd[4]);
+    S(s0 + 6) = q == 11 ? dd[2] : (q == 12 ? dd[4] : dd[5]);
+  } else if (q > 8) {
+#pragma unroll
+    for (int m = 0; m < 6; m++) S(s0 + 4 + m) = dd[m];
+  }
 }
 
 // Field q's stencils at c in a box of integers (units of 2^(E - 1075 - FX_BITS)):
@@ -224,9 +200,10 @@ __device__ __forceinline__ int fx_kept(int q, int m) {
 // wt: the thread's weights, stride Sh::THREADS; neg: signs of beta as masks.
 template <typename Sh, typename Slots>
 __device__ __forceinline__ double fx_stencils(const long long* c, int q, int order, int up, int E,
-                                              const long long* wt_, int wE, int gwE, const int neg[3], Slots S, int s0) {
+                                              const double* wt, const int neg[3], Slots S, int s0) {
   constexpr int SY = Sh::SY, SZ = Sh::SZ;
-  long long a[4], s2[6];
+  const long long f0 = c[0];
+  long long s2[6], a[4];
   a[3] = 0;
 #pragma unroll
   for (int d = 0; d < 3; d++) {
@@ -239,17 +216,16 @@ __device__ __forceinline__ double fx_stencils(const long long* c, int q, int ord
       df[m] = hi - lo;
     }
     if (order >= 1) S(s0 + d) = fx_to(8 * df[0] - df[1], E + up);
-    s2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = 16 * sp[0] - sp[1] - 30 * c[0];  // 12 h^2 d_d d_d
-    const long long kd = 15 * sp[0] - 6 * sp[1] + sp[2] - 20 * c[0], o = 21 * df[0] - 6 * df[1] + df[2];
+    s2[d == 0 ? 0 : (d == 1 ? 3 : 5)] = 16 * sp[0] - sp[1] - 30 * f0;  // 12 h^2 d_d d_d
+    const long long kh = (15 * sp[0] - 6 * sp[1] + sp[2] - 20 * f0) >> 1, oh = (21 * df[0] - 6 * df[1] + df[2]) >> 1;
     const long long sg = neg[d];
-    a[d] = kd + ((o ^ sg) - sg);
-    a[3] += kd >> 1;
+    a[d] = kh + ((oh ^ sg) - sg);
+    a[3] += kh >> 1;
   }
-  FxWeights<4> wt;
+  long long w[4];
 #pragma unroll
-  for (int m = 0; m < 4; m++) wt.w[m] = wt_[m * Sh::THREADS];
-  wt.E = wE;
-  const double r = fx_dot(a, E, wt);
+  for (int m = 0; m < 4; m++) w[m] = __double_as_longlong(wt[(m < 3 ? m : 9) * Sh::THREADS]);
+  const double r = fx_dot(a, E + 1, w);
   if (order == 2) {
 #pragma unroll
     for (int m = 0; m < 3; m++) {  // xy, xz, yz
@@ -260,59 +236,41 @@ __device__ __forceinline__ double fx_stencils(const long long* c, int q, int ord
         const long long* p = c + (n < 2 ? n - 2 : n - 1) * sa;
         l[n] = 8 * (p[sb] - p[-sb]) - (p[2 * sb] - p[-2 * sb]);
       }
-      // a quarter of 8 (l1 - l-1) - (l2 - l-2): 36 h^2 d_a d_b
-      s2[m == 0 ? 1 : 2 * m] = 2 * (l[2] - l[1]) - ((l[3] - l[0]) >> 2);
+      // an eighth of 8 (l1 - l-1) - (l2 - l-2): 18 h^2 d_a d_b
+      s2[m == 0 ? 1 : 2 * m] = (l[2] - l[1]) - ((l[3] - l[0]) >> 3);
     }
-    {
-      FxWeights<6> t;
+    double dd[6];
 #pragma unroll
-      for (int m = 0; m < 6; m++) t.w[m] = wt_[(4 + m) * Sh::THREADS];
-      t.E = gwE;
-      S(s0 + 3) = fx_dot(s2, E + 2 + up, t);
+    for (int m = 0; m < 6; m++) {
+      const bool pure = m == 0 || m == 3 || m == 5;  // 12 v = 16 (v - v/4)
+      dd[m] = fx_to(pure ? s2[m] - (s2[m] >> 2) : s2[m], E + (pure ? 4 : 3) + up);
     }
-    if (q > 8) {
-      const int n = q < 11 ? 6 : 3;
-#pragma unroll 1
-      for (int m = 0; m < n; m++) {
-        const int ab = fx_kept(q, m);
-        long long v = s2[0];
-#pragma unroll
-        for (int t = 1; t < 6; t++) v = ab == t ? s2[t] : v;
-        const bool pure = ab == 0 || ab == 3 || ab == 5;  // 12 v = 16 (v - v/4)
-        S(s0 + 4 + m) = fx_to(v - (pure ? v >> 2 : 0), E + (pure ? 4 : 2));
-      }
-    }
+    fx_second<Sh>(dd, q, wt, S, s0);
   }
   return r;
 }
 
-// The same from a box of float64 values (cold).
+// The same from the register, each stencil aligned to its own largest value or,
+// outside the integers' range, summed in float64 (rhs_fx.cuh), the products in
+// float64: for boxes and weights outside the range.  A call of its own, so that
+// its code stays out of the loop's.
 template <typename Sh, typename Slots>
-__device__ __forceinline__ double fx_stencils_f64(const Grid& g, const double* __restrict__ c0, const FxMetric& M,
-                                                  const double* c, int q, int order, int up, Slots S, int s0) {
-  double d1[3], dd[6], wd[4];
-  int neg[3];
-  fx_adv_weights(g, c0, wd, neg);
-  const double r = fx_field_f64(c, Sh::SY, Sh::SZ, wd, neg, up, d1, dd);
+__device__ __noinline__ double fx_stencils_own(const double* __restrict__ c0, long long fs, long long sy, long long sz,
+                                               double i12h, double kap, int q, int order, int up, const double* wt,
+                                               Slots S, int s0) {
+  const double* p = c0 + fx_field(q) * fs;
+  const FxAdv w = fx_adv(c0, fs, i12h, kap);
+  double d1[3], dd[3];
+  const double r = fx_axes(p, sy, sz, w, order, up, d1, dd);
   if (order >= 1) {
 #pragma unroll
     for (int d = 0; d < 3; d++) S(s0 + d) = d1[d];
   }
   if (order == 2) {
-    double t = 0.0;
-#pragma unroll 1
-    for (int m = 0; m < 6; m++) {
-      double v = M.gu[0];
-#pragma unroll
-      for (int n = 1; n < 6; n++) v = m == n ? M.g2u(n) : v;
-      t = fma(v, dd[m], t);
-    }
-    S(s0 + 3) = t;
-    if (q > 8) {
-      const int n = q < 11 ? 6 : 3;
-#pragma unroll 1
-      for (int m = 0; m < n; m++) S(s0 + 4 + m) = dd[fx_kept(q, m)];
-    }
+    double dm[3];
+    fx_mixed3(p, sy, sz, up, dm);
+    const double d6[6] = {dd[0], dm[0], dm[1], dd[1], dm[2], dd[2]};
+    fx_second<Sh>(d6, q, wt, S, s0);
   }
   return r;
 }
@@ -341,16 +299,11 @@ __device__ __forceinline__ bool rhs_fx_tile(const void* map, const Grid& g, cons
   static_assert(Sh::PER * Sh::THREADS * sizeof(int) <= sizeof(sm.box[1]), "");
   fx_points<Sh>(g, tid, ii0, jj0, kk0, cen, sc);
   int neg[3];
-  const FxWeights<4> aw = fx_tile_adv(g, c0, neg);
   FxMetric M;
   fx_metric(g, c0, M);
-  const FxWeights<6> gw = fx_tile_gu(M);
-  const bool wok = __syncthreads_and(aw.ok && gw.ok);  // (and the barriers are initialised)
-  const int wE = aw.E, gwE = gw.E;
-#pragma unroll
-  for (int m = 0; m < 4; m++) sm.wt[m][tid] = aw.w[m];
-#pragma unroll
-  for (int m = 0; m < 6; m++) sm.wt[4 + m][tid] = gw.w[m];
+  const double* wt = &sm.wt[0][tid];
+  const bool wok = fx_tile_weights<Sh>(g, c0, M, &sm.wt[0][tid], neg);
+  __syncthreads();  // the barriers are initialised
   int at[Sh::PER];
 #pragma unroll
   for (int e = 0; e < Sh::PER; e++) at[e] = sc[e * Sh::THREADS];
@@ -389,12 +342,12 @@ __device__ __forceinline__ bool rhs_fx_tile(const void* map, const Grid& g, cons
 #pragma unroll
     for (int n = 1; n < Sh::WARPS; n++) top = max(top, sm.top[n]);
     // a box of zeros takes any exponent; top does not see low words of subnormals
-    bool ok = fx_ok(top) && wok;
+    bool ok = fx_ok(top);
     if (top == 0) {
       unsigned lo = 0;
 #pragma unroll
       for (int e = 0; e < Sh::PER; e++) lo |= (unsigned)__double2loint(x[e]);
-      ok = !__syncthreads_or(lo != 0) && wok;
+      ok = !__syncthreads_or(lo != 0);
     }
     const int E = max((int)(top >> 20), 256) + FX_BITS - FX_TILE_BITS;  // the integers' unit is 2^(E - 1075 - FX_BITS)
     // (points that several threads share: the same value)
@@ -404,11 +357,11 @@ __device__ __forceinline__ bool rhs_fx_tile(const void* map, const Grid& g, cons
     }
     __syncthreads();
     const int f = fx_field(q);
-    double r;
-    if (ok)
-      r = fx_stencils<Sh>(c, q, order, up, E, &sm.wt[0][tid], wE, gwE, neg, S, s0);
+    double r = 0.0;
+    if (ok && wok)
+      r = fx_stencils<Sh>(c, q, order, up, E, wt, neg, S, s0);
     else
-      r = fx_stencils_f64<Sh>(g, c0, M, reinterpret_cast<const double*>(c), q, order, up, S, s0);
+      r = fx_stencils_own<Sh>(c0, fs, g.pitch, g.plane, g.i12h, g.kos, q, order, up, wt, S, s0);
     out[f] = f < nf ? r : 0.0;
 
     if (q == 8) {

@@ -56,3 +56,29 @@ def test_large_values_three_points_away(n, axis, form):
     want, mag = O.rhs_points_ext(cfg, st, ijk).T, O.rhs_points_mag(cfg, st, ijk)[1].T
     got = _rhs(c, st, form == "point")[:, ijk[:, 2], ijk[:, 1], ijk[:, 0]]
     assert (np.abs(got - want) <= 1e-12 * mag).all(), (np.abs(got - want) / mag).max(axis=1)
+
+
+@pytest.mark.parametrize("n", GRIDS)
+@pytest.mark.parametrize("across,along,ko", [(0.3, 1e-9, 0.0), (0.3, 1e-30, 0.0), (0.0, 1e-20, 0.0), (0.3, 1e-42, 0.0),
+                                              (1e-60, 1e-50, 0.0), (0.0, 1e-9, 0.2)])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_small_shift_beside_a_large_one(n, across, along, ko, axis):
+    """A lapse that varies along one axis, where the shift is much smaller than
+    along the others, K = 0: d_0 alpha is the small shift's advection (and the
+    dissipation), to a few roundings of its own products: eight of 2^-53 of
+    |beta| / 24h times the upwind sum's 76 max|alpha|, and of eps / 64h times the
+    dissipation's 64."""
+    h = 0.11
+    c = dict(n=n, xmin=(-0.9, -1.1, -0.7), h=h, boundary="sommerfeld", ko_eps=ko)
+    cfg = T.oracle_cfg(c)
+    st = O.initial_data(cfg, "flat", [])
+    shape = [1, 1, 1]
+    shape[2 - axis] = -1
+    st[17] = (1.0 + 0.3 * np.sin(1.7 * cfg.coords(axis))).reshape(shape)
+    for d in range(3):
+        st[18 + d] = along if d == axis else across
+    ijk = _interior(n)
+    want = O.rhs_points_ext(cfg, st, ijk)[:, 17]
+    got = _rhs(c, st)[17][ijk[:, 2], ijk[:, 1], ijk[:, 0]]
+    bar = 8 * 2.0 ** -53 * 1.3 * (along * 76 / (24 * h) + ko * 3 * 64 / (64 * h))
+    assert np.abs(got - want).max() <= bar and np.abs(want).max() > 1e3 * bar
