@@ -4,7 +4,7 @@
 // Bound: the float64 pipe (some 870 instructions of 64 cycles for a warp's
 // points), the integer stencils beside it.  Shape and occupancy: six blocks of 128
 // threads per SM (80 registers, 33 KB of shared memory each).  A step at 128^3
-// 15.7 ms; one point at a time 19.7, before that with float64 stencils 33.1.
+// 15.8 ms; one point at a time 19.7, before that with float64 stencils 33.1.
 // Found with slightly cheaper sums (a stage then 3.51-3.65 ms): with 4, 5, 7, 8
 // blocks 4.1, 3.8, 3.6, 3.7; tiles of 16 x 4 x 2 3.65, 16 x 2 x 4 3.68, 8 x 8 x 2
 // 3.60, 8 x 8 x 4 3.95, 32 x 2 x 2 4.4 (a flatter tile converts more box points per
@@ -158,9 +158,9 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
     group_and(1 + grp, T, true);
     const int f = fx_field(q);
     double r = 0.0;
-    if (ok && wok)
-      r = fx_stencils<Sh>(c, q, order, up, E, wt, neg, S, s0);
-    else
+    bool near = false;
+    if (ok) r = fx_stencils<Sh>(c, q, order, up, E, wt, neg, S, s0, near);
+    if (!(near && wok) && !(ok && top == 0))
       r = fx_stencils_own<Sh>(c0, fs, g.pitch, g.plane, g.i12h, g.kos, q, order, up, wt, S, s0);
     sm.out[f][tid] = f < nf ? r : 0.0;
   }

@@ -19,6 +19,12 @@
 //    products with weights of the point, kept as integers too (fx_weight,
 //    fx_dot); the contraction gt^kl d_k d_l is float64: some 870 float64
 //    instructions a point.
+//  - Where the box's largest value is much more than what a thread's star holds,
+//    the box's integers have fewer bits than the thread's own values.  That thread
+//    takes the field's stencils one point at a time from the register (FX_NEAR,
+//    fx_stencils_own), so that every point is as exact as rhs_fx.cuh makes it: a
+//    field that falls off steeply inside a tile, a small value beside a large one.
+//    On smooth data some percent of the warps or fewer do.
 //  - The algebra runs inside the loop as soon as its fields are there, so that
 //    few results wait at a time (33 local slots).
 // The stencil code exists once: the instruction cache holds 128 KB, and a
@@ -34,6 +40,24 @@
 namespace bssn {
 
 constexpr int FX_TILE_BITS = 4;
+
+// A thread whose star -- the point and those one and two away along each axis: the
+// values of its pure derivatives -- reaches no 2^(FX_NEAR - 1) units at the point
+// or two away (an eighth of the box's largest exponent) takes its own alignment:
+// an integer's rounding, half a unit, is then at most 2^-54 of the star's largest
+// value, the bound of rhs_fx.cuh.  (Shift and B^i as Gaussians of width 1 at h =
+// 0.25, relative error of the shift's right-hand side at each point, 90th and
+// 99th percentile: 3e-16 and 9e-16; without this rule 2e-11 and 4e-9; float64
+// stencils 1e-15 and 3e-15.)  A step at 128^3 takes 15.7 -> 15.8 ms for it, 75 x
+// 53 x 61 2.58 -> 2.69, 24^3 0.206 -> 0.220: the threads that take their own
+// alignment hold up their block.  With three bits below the box's last (and a
+// quarter in place of an eighth) 15.8, 2.74, 0.222.
+constexpr int FX_NEAR = 54;
+// a bound on |v|'s high word, whose leading bit is that of |v| (or of |v| - 1)
+__device__ __forceinline__ int fx_mag(long long v) {
+  const int hi = (int)(v >> 32);
+  return hi ^ (hi >> 31);
+}
 
 // Tile of TX x TY x TZ interior points, one per thread, and its box: the tile
 // plus three points on every side.  TX and the box's x extent are even (tensor
@@ -198,13 +222,15 @@ __device__ __forceinline__ void fx_second(const double dd[6], int q, const doubl
 // returns advection and dissipation; its first derivatives into slots s0 ..
 // s0 + 2, its contracted second derivative into s0 + 3, those kept after it.
 // wt: the thread's weights, stride Sh::THREADS; neg: signs of beta as masks.
+// near: the point's value or one two away has FX_NEAR bits or more.
 template <typename Sh, typename Slots>
 __device__ __forceinline__ double fx_stencils(const long long* c, int q, int order, int up, int E,
-                                              const double* wt, const int neg[3], Slots S, int s0) {
+                                              const double* wt, const int neg[3], Slots S, int s0, bool& near) {
   constexpr int SY = Sh::SY, SZ = Sh::SZ;
   const long long f0 = c[0];
   long long s2[6], a[4];
   a[3] = 0;
+  int big = fx_mag(f0);
 #pragma unroll
   for (int d = 0; d < 3; d++) {
     const int s = d == 0 ? 1 : (d == 1 ? SY : SZ);
@@ -212,6 +238,7 @@ __device__ __forceinline__ double fx_stencils(const long long* c, int q, int ord
 #pragma unroll
     for (int m = 0; m < 3; m++) {
       const long long lo = c[-(m + 1) * s], hi = c[(m + 1) * s];
+      if (m == 1) big |= fx_mag(lo) | fx_mag(hi);
       sp[m] = hi + lo;
       df[m] = hi - lo;
     }
@@ -222,6 +249,7 @@ __device__ __forceinline__ double fx_stencils(const long long* c, int q, int ord
     a[d] = kh + ((oh ^ sg) - sg);
     a[3] += kh >> 1;
   }
+  near = big >> (FX_NEAR - 1 - 32) != 0;
   long long w[4];
 #pragma unroll
   for (int m = 0; m < 4; m++) w[m] = __double_as_longlong(wt[(m < 3 ? m : 9) * Sh::THREADS]);
@@ -252,8 +280,8 @@ __device__ __forceinline__ double fx_stencils(const long long* c, int q, int ord
 
 // The same from the register, each stencil aligned to its own largest value or,
 // outside the integers' range, summed in float64 (rhs_fx.cuh), the products in
-// float64: for boxes and weights outside the range.  A call of its own, so that
-// its code stays out of the loop's.
+// float64: also for boxes and weights outside the range.  A call of its own, so
+// that its code stays out of the loop's.
 template <typename Sh, typename Slots>
 __device__ __noinline__ double fx_stencils_own(const double* __restrict__ c0, long long fs, long long sy, long long sz,
                                                double i12h, double kap, int q, int order, int up, const double* wt,
@@ -358,9 +386,9 @@ __device__ __forceinline__ bool rhs_fx_tile(const void* map, const Grid& g, cons
     __syncthreads();
     const int f = fx_field(q);
     double r = 0.0;
-    if (ok && wok)
-      r = fx_stencils<Sh>(c, q, order, up, E, wt, neg, S, s0);
-    else
+    bool near = false;
+    if (ok) r = fx_stencils<Sh>(c, q, order, up, E, wt, neg, S, s0, near);
+    if (!(near && wok) && !(ok && top == 0))
       r = fx_stencils_own<Sh>(c0, fs, g.pitch, g.plane, g.i12h, g.kos, q, order, up, wt, S, s0);
     out[f] = f < nf ? r : 0.0;
 

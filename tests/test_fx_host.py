@@ -76,9 +76,10 @@ int h_stencils(const double* box, int q, const double* w4, const double* g6, con
   }
   for (int m = 0; m < 6; m++) wt[(3 + m) * Sh::THREADS] = g6[m];
   const long long* c = ib + ((k + GH) * Sh::BY + j + GH) * Sh::BX + i + GH;
+  bool near = false;
   auto S = [&](int n) -> double& { return out[1 + n]; };
-  out[0] = fx_stencils<Sh>(c, q, fx_order(q), fx_up(q), E, wt, neg, S, 0);
-  return 0;
+  out[0] = fx_stencils<Sh>(c, q, fx_order(q), fx_up(q), E, wt, neg, S, 0, near);
+  return near;
 }
 }
 """
@@ -206,11 +207,15 @@ def test_stencils_in_a_box(lib, kind):
         g6 = [float(x) for x in rng.uniform(0.5, 1.5, 6)]
         out = (ctypes.c_double * 16)()
         flat = np.ascontiguousarray(box)
+        star = np.array([box[k + 3, j + 3, i + 3]] + [box[k + 3 + m * (a == 2), j + 3 + m * (a == 1), i + 3 + m * (a == 0)]
+                                                      for a in range(3) for m in (-2, 2)])
         biggest = float(np.abs(box).max())
         u = unit(int(np.frexp(biggest)[1]) - 53 - bits)  # a unit of the box's integers
         for q in (0, 7, 9, 12, 14, 20):
-            assert lib.h_stencils(flat.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), q, (ctypes.c_double * 4)(*bh, 2 * kap),
-                                   (ctypes.c_double * 6)(*g6), (ctypes.c_int * 3)(*neg), i, j, k, out) == 0
+            near = lib.h_stencils(flat.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), q, (ctypes.c_double * 4)(*bh, 2 * kap),
+                                  (ctypes.c_double * 6)(*g6), (ctypes.c_int * 3)(*neg), i, j, k, out)
+            # near: some star value of 2^53 units or more (a value one unit below may round up to it)
+            assert near == (float(np.abs(star).max()) >= float(2 ** 53 * u)) or kind == "wide"
             r, d1, dd = _exact(box, q, (k + 3, j + 3, i + 3), bh, kap, neg)
             order, up = (2 if q < 6 or 8 < q < 14 else (1 if q < 15 else 0)), (Fr(1, 2) if q < 9 else 1)
             # r: 38 taps in half sums a weight and the quarters dropped, each half a unit

@@ -1,6 +1,7 @@
 """The float64 right-hand side is as exact beside large values as without them:
-aligning a stencil's values to the largest among several (csrc/fx.cuh) must not
-cost a derivative the bits by which values that it does not use exceed its own.
+aligning a stencil's values to the largest among several (csrc/fx.cuh) or in a
+tile's whole box (csrc/rhs_fx_tile.cuh) must not cost a derivative the bits by
+which values that it does not use exceed its own.
 
 Bars.  A stencil's values are held to 2^-54 of their largest or better and its sums
 to a few 2^-53, so a point's right-hand side is off by some hundred times 2^-53 M,
@@ -40,7 +41,7 @@ def _interior(n):
                     dtype=np.int32)
 
 
-@pytest.mark.parametrize("form", ["point"])
+@pytest.mark.parametrize("form", ["point", "tiles"])
 @pytest.mark.parametrize("n", GRIDS[:2])
 @pytest.mark.parametrize("axis", [0, 1, 2])
 def test_large_values_three_points_away(n, axis, form):
@@ -82,3 +83,36 @@ def test_small_shift_beside_a_large_one(n, across, along, ko, axis):
     got = _rhs(c, st)[17][ijk[:, 2], ijk[:, 1], ijk[:, 0]]
     bar = 8 * 2.0 ** -53 * 1.3 * (along * 76 / (24 * h) + ko * 3 * 64 / (64 * h))
     assert np.abs(got - want).max() <= bar and np.abs(want).max() > 1e3 * bar
+
+
+@pytest.mark.parametrize("n", GRIDS)
+@pytest.mark.parametrize("conformal,precision", [("W", "fp64"), ("phi", "fp64"), ("W", "ff")])
+def test_small_values_beside_large_ones(n, conformal, precision):
+    """Fields of size 1e-9 with cubes of size 0.05 (three points) here and there:
+    every point none of whose stencils reaches a cube, against the oracle in
+    extended precision."""
+    c = dict(n=n, xmin=(-0.9, -1.1, -0.7), h=0.11, boundary="sommerfeld", conformal=conformal, precision=precision)
+    st = inputs.random_state(41, n, c["xmin"], c["h"], amp=0.05)
+    if conformal == "phi":
+        st[0] = -0.5 * np.log(st[0])
+    big = np.zeros(st.shape[1:], dtype=bool)
+    for k in range(7, n[2], 11):
+        for j in range(5, n[1], 11):
+            for i in range(6, n[0], 12):
+                big[k:k + 3, j:j + 3, i:i + 3] = True
+    for f in (2, 7, 8, 10, 13, 14, 16, 18, 19, 20, 22, 23):
+        st[f] *= 2e-8
+        st[f][big] += 0.05
+    reach = np.zeros_like(big)
+    offs = [(0, 0, m) for m in range(-3, 4)]
+    offs = {tuple(np.roll(o, r)) for o in offs for r in range(3)}
+    offs |= {tuple(np.roll((0, a, b), r)) for a in range(-2, 3) for b in range(-2, 3) for r in range(3)}
+    for o in offs:
+        reach |= np.roll(big, o, (0, 1, 2))
+    ijk = np.array([q for q in _interior(n) if not reach[q[2], q[1], q[0]]], dtype=np.int32)
+    assert 0.2 * np.prod(n) < len(ijk) < 0.95 * np.prod(n)
+    cfg = T.oracle_cfg(c)
+    want = O.rhs_points_ext(cfg, st, ijk).T
+    mag = O.rhs_points_mag(cfg, st, ijk)[1].T
+    got = _rhs(c, st)[:, ijk[:, 2], ijk[:, 1], ijk[:, 0]]
+    assert (np.abs(got - want) <= 1e-12 * mag).all(), (np.abs(got - want) / mag).max(axis=1)
