@@ -183,7 +183,10 @@ bssn_status bssn_set_punctures(bssn_ctx* ctx, const double* p, int32_t npunct);
  * centred stencils, upwinded advection, KO dissipation), ghost points by the
  * Sommerfeld condition (or 0 when periodic).  d_state: a float64 register in
  * the layout above (NULL = the context's y_n); d_rhs: a float64 register the
- * caller owns.  Ghost values of d_state must be valid (periodic: filled). */
+ * caller owns.  Ghost values of d_state must be valid (periodic: filled).
+ * Float64 and double-word contexts write only d_rhs, so captured calls on other
+ * registers may be replayed beside one another and beside the context's steps;
+ * mixed ones round the state into a stage buffer of the context. */
 bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs);
 
 /* Advance y_n by nsteps classical RK4 steps of size dt (t += nsteps dt).

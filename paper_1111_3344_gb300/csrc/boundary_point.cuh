@@ -166,9 +166,23 @@ __device__ __forceinline__ void ghost_table_fill(const Grid& g, unsigned q, doub
   itab[q] = (long long)G.I[0] | ((long long)G.I[1] << 21) | ((long long)G.I[2] << 42);
 }
 
-// float64 path from the table, after the anchor pass: ghost point q, fields
-// [F0, F1) (a group of the 24 per thread, their loads in flight together).
-template <int F0, int F1>
+// The anchor's factors (nas, ira) as ghost_geo forms them.
+__device__ __forceinline__ double anchor_geo(const Grid& g, const int A[3], double nas[3]) {
+  double xa[3];
+#pragma unroll
+  for (int d = 0; d < 3; d++) xa[d] = coordv(g, d, A[d]);
+  const double ira = 1.0 / sqrt(xa[0] * xa[0] + xa[1] * xa[1] + xa[2] * xa[2]);
+#pragma unroll
+  for (int d = 0; d < 3; d++) nas[d] = (xa[d] * ira) * g.i2h;
+  return ira;
+}
+
+// float64 path from the table: ghost point q, fields [F0, F1) (a group of the 24
+// per thread, their loads in flight together).  A stage: after the anchor pass,
+// from the k - rad that it left in kanchor.  OWN (a right-hand side alone, which
+// has no memory but its output to leave anything in): the k of the output, and
+// the anchor's radiative term formed here.
+template <int F0, int F1, bool OWN = false>
 __device__ __forceinline__ void sommerfeld_point_fp64_tab(const Grid& g, const StageArgs& a,
                                                           const double* __restrict__ kanchor,
                                                           const double* __restrict__ tab,
@@ -194,7 +208,17 @@ __device__ __forceinline__ void sommerfeld_point_fp64_tab(const Grid& g, const S
   for (int n = 0; n < N; n++) {
     o[n] = (F0 + n) * fs + ib;
     v[n].load(a.src + o[n], tb);
-    ka[n] = kanchor[(F0 + n) * fs + ia];
+    if (!OWN) ka[n] = kanchor[(F0 + n) * fs + ia];
+  }
+  if constexpr (OWN) {
+    double nas[3];
+    const double ira = anchor_geo(g, A, nas);
+    const RadTaps ta = rad_taps_inside(g);
+#pragma unroll
+    for (int n = 0; n < N; n++) {
+      const long long oa = (F0 + n) * fs + ia;
+      ka[n] = a.rhs[oa] - rad_at<double, double>(g, a.src + oa, F0 + n, ta, nas, ira);
+    }
   }
   if (tb.edge()) {
 #pragma unroll
@@ -208,7 +232,7 @@ __device__ __forceinline__ void sommerfeld_point_fp64_tab(const Grid& g, const S
 
 // float64 path, anchor pass: interior point q of the boundary shell, fields
 // [F0, F1): k - rad at the anchor, in place of the k the stage kernel left in
-// kanchor (MODE_RHS: in rhs) (the same operations the ghost points of that anchor would repeat,
+// kanchor (the same operations the ghost points of that anchor would repeat,
 // one to three layers and up to eight neighbours over; see sommerfeld_point_fp64).
 template <int F0 = 0, int F1 = NF>
 __device__ __forceinline__ void sommerfeld_anchor_fp64(const Grid& g, const StageArgs& a,
@@ -216,24 +240,16 @@ __device__ __forceinline__ void sommerfeld_anchor_fp64(const Grid& g, const Stag
   int ii, jj, kk;
   shell_decode(g, q, ii, jj, kk);
   const int A[3] = {ii + GH, jj + GH, kk + GH};
-  double xa[3];
-#pragma unroll
-  for (int d = 0; d < 3; d++) xa[d] = coordv(g, d, A[d]);
-  // as ghost_geo forms the anchor's factors
-  const double ra = sqrt(xa[0] * xa[0] + xa[1] * xa[1] + xa[2] * xa[2]);
-  const double ira = 1.0 / ra;
   double nas[3];
-#pragma unroll
-  for (int d = 0; d < 3; d++) nas[d] = (xa[d] * ira) * g.i2h;
+  const double ira = anchor_geo(g, A, nas);
   const long long ia = lin(g, A[0], A[1], A[2]);
   const long long fs = g.fstride;
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
   const RadTaps ta = rad_taps_inside(g);
-  const double* ks = a.mode == MODE_RHS ? a.rhs : kanchor;
   double k[F1 - F0];  // every load before the stores
 #pragma unroll
   for (int f = F0; f < F1; f++)
-    if (f < nf) k[f - F0] = ks[f * fs + ia] - rad_at<double, double>(g, a.src + f * fs + ia, f, ta, nas, ira);
+    if (f < nf) k[f - F0] = kanchor[f * fs + ia] - rad_at<double, double>(g, a.src + f * fs + ia, f, ta, nas, ira);
 #pragma unroll
   for (int f = F0; f < F1; f++)
     if (f < nf) kanchor[f * fs + ia] = k[f - F0];

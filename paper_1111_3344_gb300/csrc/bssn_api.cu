@@ -547,7 +547,7 @@ bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs) {
     e = launch_stage_fp64(ctx->g, a, ctx->stream, fp64_cfg(ctx, ctx->tile), map, ctx->err);
     if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs interior");
     if (!ctx->g.periodic) {
-      e = launch_sommerfeld(ctx->g, a, ctx->ksh, ctx->stream, ctx->gtab);
+      e = launch_sommerfeld(ctx->g, a, nullptr, ctx->stream, ctx->gtab);
       if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs boundary");
     }
     return BSSN_OK;

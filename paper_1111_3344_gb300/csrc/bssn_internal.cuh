@@ -346,8 +346,8 @@ int split_config_count();
 const char* split_config_name(int v);
 cudaError_t launch_stage_mixed_split(const Grid& g, const StageArgsMixed& a, float* dr, cudaStream_t s,
                                      int variant);
-// kanchor: scratch register (the anchors' k of a stage; MODE_RHS: overwritten);
-// table: the ghost-geometry table (launch_ghost_table)
+// kanchor: the register with the anchors' k of a stage (MODE_RHS: not used, the k
+// of the output is read); table: the ghost-geometry table (launch_ghost_table)
 cudaError_t launch_sommerfeld(const Grid& g, const StageArgs& a, double* kanchor, cudaStream_t s,
                               const void* table);
 size_t ghost_table_size(const Grid& g);

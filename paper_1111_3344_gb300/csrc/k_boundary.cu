@@ -36,18 +36,19 @@ __global__ void sommerfeld_anchor_fp64_kernel(Grid g, StageArgs a, double* __res
 // one branch for the group, for the float64 pipe bounds it (computed for every
 // point and selected: 328 us at 128^3 against 293; one field after another: 38 us
 // at 24^3, 74 at 48^3, 299 at 128^3; so 29, 61, 293).
+template <bool OWN>
 __global__ void sommerfeld_fp64_tab_kernel(Grid g, StageArgs a, const double* __restrict__ kanchor,
                                            const double* __restrict__ tab, const long long* __restrict__ itab) {
   after_previous();
   const unsigned q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= ghost_count(g)) return;
   switch (blockIdx.y) {  // six groups of four fields
-    case 0: sommerfeld_point_fp64_tab<0, 4>(g, a, kanchor, tab, itab, q); break;
-    case 1: sommerfeld_point_fp64_tab<4, 8>(g, a, kanchor, tab, itab, q); break;
-    case 2: sommerfeld_point_fp64_tab<8, 12>(g, a, kanchor, tab, itab, q); break;
-    case 3: sommerfeld_point_fp64_tab<12, 16>(g, a, kanchor, tab, itab, q); break;
-    case 4: sommerfeld_point_fp64_tab<16, 20>(g, a, kanchor, tab, itab, q); break;
-    default: sommerfeld_point_fp64_tab<20, NF>(g, a, kanchor, tab, itab, q); break;
+    case 0: sommerfeld_point_fp64_tab<0, 4, OWN>(g, a, kanchor, tab, itab, q); break;
+    case 1: sommerfeld_point_fp64_tab<4, 8, OWN>(g, a, kanchor, tab, itab, q); break;
+    case 2: sommerfeld_point_fp64_tab<8, 12, OWN>(g, a, kanchor, tab, itab, q); break;
+    case 3: sommerfeld_point_fp64_tab<12, 16, OWN>(g, a, kanchor, tab, itab, q); break;
+    case 4: sommerfeld_point_fp64_tab<16, 20, OWN>(g, a, kanchor, tab, itab, q); break;
+    default: sommerfeld_point_fp64_tab<20, NF, OWN>(g, a, kanchor, tab, itab, q); break;
   }
 }
 
@@ -102,21 +103,25 @@ __global__ void periodic_fill_kernel(Grid g, S* __restrict__ y, double* __restri
   periodic_point<S>(g, y, w, q);
 }
 
-// The anchor pass (one thread per shell point) forms k - rad at the anchors once
-// into kanchor, then the ghost points each form only their own radiative term
-// (a right-hand side of 80^3: 1.13 ms with both terms and the geometry at every
-// ghost point, 1.03 so).
+// A stage: the anchor pass (one thread per shell point) turns the k at the anchors
+// into k - rad once, then the ghost points each form only their own radiative
+// term.  A right-hand side alone: every ghost point forms both, so that the call
+// writes nothing but its output (captured calls of one context may run on
+// several streams); a right-hand side of 80^3 takes 1.139 ms, 1.088 with the
+// anchor pass into memory of the context.
 cudaError_t launch_sommerfeld(const Grid& g, const StageArgs& a, double* kanchor, cudaStream_t s,
                               const void* table) {
   const unsigned total = ghost_count(g), ns = shell_count(g);
   const int bs = 128;
-  cudaError_t e = launch_after(sommerfeld_anchor_fp64_kernel, dim3((ns + bs - 1) / bs, 4), bs, 0, s, fx_launch_early(g), g, a,
-                               kanchor);
-  if (e != cudaSuccess) return e;
   const double* tab = (const double*)table;
   const long long* itab = (const long long*)(tab + (size_t)GEO_DOUBLES * total);
-  return launch_after(sommerfeld_fp64_tab_kernel, dim3((total + bs - 1) / bs, 6), bs, 0, s, fx_launch_early(g), g, a,
-                      kanchor, tab, itab);
+  const dim3 blocks((total + bs - 1) / bs, 6);
+  const bool early = fx_launch_early(g);
+  if (a.mode == MODE_RHS)
+    return launch_after(sommerfeld_fp64_tab_kernel<true>, blocks, bs, 0, s, early, g, a, nullptr, tab, itab);
+  cudaError_t e = launch_after(sommerfeld_anchor_fp64_kernel, dim3((ns + bs - 1) / bs, 4), bs, 0, s, early, g, a, kanchor);
+  if (e != cudaSuccess) return e;
+  return launch_after(sommerfeld_fp64_tab_kernel<false>, blocks, bs, 0, s, early, g, a, kanchor, tab, itab);
 }
 cudaError_t launch_sommerfeld_mixed(const Grid& g, const StageArgsMixed& a, const float* kanchor,
                                     cudaStream_t s) {
