@@ -186,7 +186,10 @@ bssn_status bssn_set_punctures(bssn_ctx* ctx, const double* p, int32_t npunct);
  * caller owns.  Ghost values of d_state must be valid (periodic: filled).
  * Float64 and double-word contexts write only d_rhs, so captured calls on other
  * registers may be replayed beside one another and beside the context's steps;
- * mixed ones round the state into a stage buffer of the context. */
+ * mixed ones round the state into a stage buffer of the context.  A tensor-load
+ * wait that gives up (bounded) leaves points of d_rhs unwritten: a caller that
+ * steps by this call alone sees it as BSSN_ETIMEOUT from bssn_wait_state (or the
+ * next bssn_get_state or bssn_constraints). */
 bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs);
 
 /* Advance y_n by nsteps classical RK4 steps of size dt (t += nsteps dt).
@@ -416,10 +419,10 @@ bssn_status bssn_batch_set_tile(bssn_batch* b, int32_t cfg);
  * the configurations the batch cannot use. */
 bssn_status bssn_batch_autotune(bssn_batch* b, int32_t reps, int32_t* best, double* ms_per_cfg);
 /* Test hook of the bounded wait (no counterpart in the paper), as
- * bssn_test_stall_tma for the batch's TMA-staged stage kernel: polls > 0 makes
- * every block issue no tile copy and give up after that many polls; the next
- * bssn_batch_get_state or bssn_batch_constraints returns BSSN_ETIMEOUT (and
- * clears the error word).  The member tables are re-uploaded in stream order;
+ * bssn_test_stall_tma for the batch's TMA-staged stage kernels (float64 batches:
+ * the per-member configurations): polls > 0 makes every block issue no tile copy
+ * and give up after that many polls; the next bssn_batch_get_state or
+ * bssn_batch_constraints returns BSSN_ETIMEOUT (and clears the error word).  The member tables are re-uploaded in stream order;
  * the captured graph is kept, except under the per-member configurations,
  * whose launches carry the arguments themselves: their graph is captured
  * again at the next step.  polls in [0, 2^20]; 0 restores normal operation. */
@@ -491,9 +494,14 @@ bssn_status bssn_profile(bssn_ctx* ctx, int32_t enable, double out[4]);
  * the next synchronising call (bssn_get_state, bssn_wait_state,
  * bssn_constraints) returns BSSN_ETIMEOUT and clears the error word; the
  * context stays usable.  polls in [0, 2^20]; 0 (the default) restores normal
- * operation.  Affects only the TMA-staged configurations of mixed contexts
- * (the float64 tiles' waits have the same limit and report the same way). */
+ * operation.  Affects the TMA-staged configurations of mixed contexts and the
+ * float64 and double-word stage where it runs in tiles ("32x4x1/1"). */
 bssn_status bssn_test_stall_tma(bssn_ctx* ctx, int32_t polls);
+/* The same where one copy among many does not arrive: the float64 tiles load one
+ * field after another, on grids of few tiles in four groups of threads.  The copy
+ * left out is that of one group (0-3; larger grids have only group 0) and round
+ * (0-23; the four groups: 0-2 and, but for group 0, 3-6; others leave out none). */
+bssn_status bssn_test_stall_tile(bssn_ctx* ctx, int32_t polls, int32_t group, int32_t round);
 
 /* Measured arithmetic peak of the current GPU (no counterpart in the paper:
  * it is the denominator of the roofline on which the stage kernels are

@@ -153,6 +153,7 @@ _SIGS = [
                                   ctypes.POINTER(ctypes.c_double), ctypes.c_int32, ctypes.c_void_p,
                                   ctypes.POINTER(ctypes.c_double)], ctypes.c_int),
     ("bssn_test_stall_tma", [ctypes.c_void_p, ctypes.c_int32], ctypes.c_int),
+    ("bssn_test_stall_tile", [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32], ctypes.c_int),
     ("bssn_peak_probe", [ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
                          ctypes.POINTER(ctypes.c_double)], ctypes.c_int),
 ]
@@ -371,6 +372,11 @@ def bssn_test_stall_tma(ctx: int, polls: int):
     """Test hook: TMA-staged stage kernels issue no copy and give up waiting
     after `polls` polls (0: normal operation); see include/bssn.h."""
     _check(load().bssn_test_stall_tma(ctypes.c_void_p(ctx), int(polls)))
+
+
+def bssn_test_stall_tile(ctx: int, polls: int, group: int, round: int):
+    """Test hook: one copy of the float64 tiles left out; see include/bssn.h."""
+    _check(load().bssn_test_stall_tile(ctypes.c_void_p(ctx), int(polls), int(group), int(round)))
 
 
 def bssn_batch_test_stall_tma(batch: int, polls: int):

@@ -182,7 +182,7 @@ struct bssn_ctx {
   CUtensorMap fmap[3];  // float64: tensor maps of y_n, s1, s2 (tile form of the stage)
   bool fmap_ok;
   int* err;             // device error word (bounded waits that gave up)
-  int stall_polls;      // test hook of the TMA-staged kernels (bssn_test_stall_tma)
+  int stall_polls, stall_at;  // test hook of the TMA-staged kernels (bssn_test_stall_tma, bssn_test_stall_tile)
   double* part;
   double* out16;
   double t;
@@ -338,6 +338,7 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
   ctx->prof = false;
   ctx->err = (int*)(ctx->mem + c.err);
   ctx->stall_polls = 0;
+  ctx->stall_at = -1;
   ctx->trk = (double*)(ctx->mem + c.trk);
   ctx->tracking = false;
   ctx->trk_stale = false;
@@ -536,6 +537,8 @@ bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs) {
     a.src = src;
     a.rhs = out;
     a.mode = MODE_RHS;
+    a.stall_polls = ctx->stall_polls;
+    a.stall_at = ctx->stall_at;
     // a caller's register is described here, where its address allows it (also
     // while the stream is captured; the query binds the thread's context)
     CUtensorMap made;
@@ -591,6 +594,8 @@ static bssn_status run_stage(bssn_ctx* ctx, const double* src, int mode, double*
   a.a_dtf = (float)a_dt;
   a.b_dt = b_dt;
   a.mode = mode;
+  a.stall_polls = ctx->stall_polls;
+  a.stall_at = ctx->stall_at;
   cudaError_t e;
   if (ctx->prof && (e = prof_mark(ctx, ctx->ev_stage)) != cudaSuccess) return cuda_fail(e, "profile");
   e = launch_stage_fp64(ctx->g, a, ctx->stream, fp64_cfg(ctx, ctx->tile), fx_map(ctx, src), ctx->err);
@@ -1058,7 +1063,15 @@ bssn_status bssn_test_stall_tma(bssn_ctx* ctx, int32_t polls) {
   if (!ctx) return fail(BSSN_EINVAL, "ctx is NULL");
   if (polls < 0 || polls > (1 << 20)) return fail(BSSN_EINVAL, "polls must be in [0, 2^20]");
   ctx->stall_polls = polls;
+  ctx->stall_at = -1;
   return BSSN_OK;
+}
+
+bssn_status bssn_test_stall_tile(bssn_ctx* ctx, int32_t polls, int32_t group, int32_t round) {
+  if (group < 0 || group > 3 || round < 0 || round > 23) return fail(BSSN_EINVAL, "group must be in [0, 3], round in [0, 23]");
+  const bssn_status s = bssn_test_stall_tma(ctx, polls);
+  if (s == BSSN_OK) ctx->stall_at = 32 * group + round;
+  return s;
 }
 
 bssn_status bssn_profile(bssn_ctx* ctx, int32_t enable, double out[4]) {

@@ -202,6 +202,8 @@ void fill_member_dev(bssn_batch* b, int id) {
       a.a_dt = a_dt[s];
       a.b_dt = b_dt[s];
       a.mode = mode[s];
+      a.stall_polls = b->stall_polls;
+      a.stall_at = -1;
       if (make_fx_tensor_map(M.g, a.src, &D.tmap[s]) != cudaSuccess) M.fmap_ok = false;
     }
   } else {

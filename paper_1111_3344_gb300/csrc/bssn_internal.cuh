@@ -294,8 +294,11 @@ struct StageArgsT {
   int mode;
   // test hook of the TMA-staged kernels: > 0 issues no tile copy and gives up
   // waiting after this many polls, so that the bounded-wait path runs with
-  // nothing in flight; 0 in normal operation
+  // nothing in flight; 0 in normal operation.  Float64 tiles load one field
+  // after another: the copy left out is the first of every group of threads
+  // (stall_at < 0) or that of one group's round (group * 32 + round)
   int stall_polls;
+  int stall_at;
 };
 using StageArgs = StageArgsT<double>;
 using StageArgsMixed = StageArgsT<float>;

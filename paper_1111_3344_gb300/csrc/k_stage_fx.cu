@@ -12,7 +12,8 @@
 //
 // The waits for the tensor loads are bounded: a block whose wait runs out sets
 // the error word (read back by the host as BSSN_ETIMEOUT), waits once more,
-// boundedly, for its own copy, and returns without writing results.
+// boundedly, for its own copy, and returns without writing results.  (A test hook
+// leaves out one copy and polls a given number of times.)
 #include "rhs_fx_tile.cuh"
 #include "stage_point.cuh"
 
@@ -29,7 +30,7 @@ __global__ void __launch_bounds__(FxT::THREADS, 6)
   // threads past the grid work on the nearest point inside it; their results are dropped
   const int i = min(ii, g.n0 - 1) + GH, j = min(jj, g.n1 - 1) + GH, k = min(kk, g.n2 - 1) + GH;
   double r[NF];
-  if (!rhs_fx_tile<FxT>(&map, g, a.src, sm, tid, ii0, jj0, kk0, i, j, k, r)) {
+  if (!rhs_fx_tile<FxT>(&map, g, a.src, sm, tid, ii0, jj0, kk0, i, j, k, r, fx_stall_round(a, 0), a.stall_polls)) {
     if (tid == 0) atomicExch(err, 1);
     return;
   }
@@ -91,8 +92,9 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
   const int cen = fx_center<Sh>(ii0, jj0, kk0, i, j, k);
   int* sc = reinterpret_cast<int*>(sm.box[grp][1]) + tid;
   fx_points<Sh>(g, tid, ii0, jj0, kk0, cen, sc);
+  const int stall = fx_stall_round(a, grp);
   after_previous();
-  if (tid == 0) fx_issue<Sh>(&map, sm.box[grp][0], bar0, ii0, jj0, kk0, fx_field(grp));
+  if (tid == 0 && stall != 0) fx_issue<Sh>(&map, sm.box[grp][0], bar0, ii0, jj0, kk0, fx_field(grp));
   FxMetric M;  // the first group's
   if (grp == 0) {
     int neg[3];
@@ -125,20 +127,21 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
     long long* box = sm.box[grp][rd & 1];
     const long long* c = box + cen;
     const unsigned bar = rd & 1 ? bar1 : bar0;
-    const bool there = mbar_wait(bar, (rd >> 1) & 1, WAIT_LIMIT);
+    const bool there = mbar_wait(bar, (rd >> 1) & 1, rd == stall ? a.stall_polls : WAIT_LIMIT);
     double x[Sh::PER];
 #pragma unroll
     for (int e = 0; e < Sh::PER; e++) x[e] = __longlong_as_double(box[at[e]]);
     const unsigned wtop = __reduce_max_sync(0xffffffffu, fx_top(x));
     if ((tid & 31) == 0) sm.top[grp][tid >> 5] = wtop;
     if (!group_and(1 + grp, T, there)) {
-      mbar_wait(bar, (rd >> 1) & 1, WAIT_LIMIT);  // the group's one copy in flight lands before the block exits
+      // the group's one copy in flight lands before the block exits
+      if (rd != stall) mbar_wait(bar, (rd >> 1) & 1, WAIT_LIMIT);
       sm.fail = 1;
       if (rd < 3) __syncthreads();
       break;
     }
     const int next = rd + 1 < 3 ? q + GROUPS : (rd == 2 ? (grp ? 11 + grp : NF) : q + GROUPS - 1);
-    if (tid == 0 && next < NF)
+    if (tid == 0 && next < NF && rd + 1 != stall)
       fx_issue<Sh>(&map, sm.box[grp][(rd + 1) & 1], rd & 1 ? bar0 : bar1, ii0, jj0, kk0, fx_field(next));
     unsigned top = sm.top[grp][0];
 #pragma unroll

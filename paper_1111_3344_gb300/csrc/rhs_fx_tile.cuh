@@ -303,14 +303,23 @@ __device__ __noinline__ double fx_stencils_own(const double* __restrict__ c0, lo
   return r;
 }
 
+// Test hook (StageArgsT::stall_polls): the round whose copy group grp leaves out, -1
+// for none.
+template <typename A>
+__device__ __forceinline__ int fx_stall_round(const A& a, int grp) {
+  if (a.stall_polls <= 0) return -1;
+  return a.stall_at < 0 ? 0 : (a.stall_at / 32 == grp ? a.stall_at % 32 : -1);
+}
+
 // The right-hand side of all 24 fields at this thread's point (i, j, k) (stored
 // indices, inside the grid) of the tile whose first interior point is (ii0,
 // jj0, kk0), from the float64 register st, which map describes (its box that
-// of Sh); every thread of the block calls it.  False: a wait ran out.
+// of Sh); every thread of the block calls it.  False: a wait ran out (at once in
+// round stall, after polls, its copy left out).
 template <typename Sh>
 __device__ __forceinline__ bool rhs_fx_tile(const void* map, const Grid& g, const double* __restrict__ st,
                                             FxShared<Sh>& sm, int tid, int ii0, int jj0, int kk0, int i, int j, int k,
-                                            double out[NF]) {
+                                            double out[NF], int stall, int polls) {
   const long long fs = g.fstride, id = lin(g, i, j, k);
   const double* c0 = st + id;
   const int nf = g.shift == BSSN_SHIFT_FROZEN ? F_BETA : NF;
@@ -319,7 +328,7 @@ __device__ __forceinline__ bool rhs_fx_tile(const void* map, const Grid& g, cons
 
   if (tid == 0) {
     for (int b = 0; b < 2; b++) mbar_init(smem_addr(&sm.bar[b]));
-    fx_issue<Sh>(map, sm.box[0], smem_addr(&sm.bar[0]), ii0, jj0, kk0, fx_field(0));
+    if (stall != 0) fx_issue<Sh>(map, sm.box[0], smem_addr(&sm.bar[0]), ii0, jj0, kk0, fx_field(0));
   }
   const int cen = fx_center<Sh>(ii0, jj0, kk0, i, j, k);
   // (through the second buffer, which is still free)
@@ -353,7 +362,7 @@ __device__ __forceinline__ bool rhs_fx_tile(const void* map, const Grid& g, cons
     asm volatile("" : "+r"(order), "+r"(up), "+r"(s0));  // one copy of the code below, not one per value
     long long* box = sm.box[q & 1];
     const long long* c = box + cen;
-    const bool there = mbar_wait(smem_addr(&sm.bar[q & 1]), (q >> 1) & 1, WAIT_LIMIT);
+    const bool there = mbar_wait(smem_addr(&sm.bar[q & 1]), (q >> 1) & 1, q == stall ? polls : WAIT_LIMIT);
     double x[Sh::PER];
 #pragma unroll
     for (int e = 0; e < Sh::PER; e++) x[e] = __longlong_as_double(box[at[e]]);
@@ -361,10 +370,11 @@ __device__ __forceinline__ bool rhs_fx_tile(const void* map, const Grid& g, cons
     if ((tid & 31) == 0) sm.top[tid >> 5] = wtop;
     // the maxima are there, and the previous field's box is free
     if (!__syncthreads_and(there)) {
-      mbar_wait(smem_addr(&sm.bar[q & 1]), (q >> 1) & 1, WAIT_LIMIT);  // the one copy in flight lands before the block exits
+      // the one copy in flight lands before the block exits
+      if (q != stall) mbar_wait(smem_addr(&sm.bar[q & 1]), (q >> 1) & 1, WAIT_LIMIT);
       return false;
     }
-    if (tid == 0 && q + 1 < NF)
+    if (tid == 0 && q + 1 < NF && q + 1 != stall)
       fx_issue<Sh>(map, sm.box[(q + 1) & 1], smem_addr(&sm.bar[(q + 1) & 1]), ii0, jj0, kk0, fx_field(q + 1));
     unsigned top = sm.top[0];
 #pragma unroll
