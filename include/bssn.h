@@ -336,8 +336,9 @@ bssn_status bssn_set_tile(bssn_ctx* ctx, int32_t cfg);
  * the next step overwrites the stage buffers and k-sum they write), select the
  * fastest for the context and return it in *best; ms_per_cfg (may be NULL,
  * else bssn_tile_count() entries) receives the mean milliseconds per stage
- * launch (INFINITY for configurations this context cannot use).  Synchronises
- * the stream. */
+ * launch (INFINITY for configurations this context cannot use; the names of
+ * double-word precision are one kernel, measured once, and the first of them is
+ * the choice).  Synchronises the stream. */
 bssn_status bssn_autotune(bssn_ctx* ctx, int32_t reps, int32_t* best, double* ms_per_cfg);
 
 /* ------------------------------------------------------------ batches
@@ -416,7 +417,8 @@ bssn_status bssn_batch_set_tile(bssn_batch* b, int32_t cfg);
  * the batch's live members (launches of the first two stages, which leave y_n
  * unchanged) and selects the fastest; ms_per_cfg (bssn_batch_tile_count
  * entries, may be NULL) gets the mean milliseconds per stage launch, -1 for
- * the configurations the batch cannot use. */
+ * the configurations the batch cannot use; double-word batches' own names get
+ * that of "members" and are never the choice. */
 bssn_status bssn_batch_autotune(bssn_batch* b, int32_t reps, int32_t* best, double* ms_per_cfg);
 /* Test hook of the bounded wait (no counterpart in the paper), as
  * bssn_test_stall_tma for the batch's TMA-staged stage kernels (float64 batches:
