@@ -540,12 +540,10 @@ bssn_status bssn_rhs(bssn_ctx* ctx, const void* d_state, void* d_rhs) {
     a.stall_polls = ctx->stall_polls;
     a.stall_at = ctx->stall_at;
     // a caller's register is described here, where its address allows it (also
-    // while the stream is captured; the query binds the thread's context)
+    // while the stream is captured)
     CUtensorMap made;
     const CUtensorMap* map = fx_map(ctx, src);
-    cudaStreamCaptureStatus cap;
-    if (!map && ctx->fmap_ok && (uintptr_t)src % 16 == 0 && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess &&
-        make_fx_tensor_map(ctx->g, src, &made, true) == cudaSuccess)
+    if (!map && ctx->fmap_ok && (uintptr_t)src % 16 == 0 && make_fx_tensor_map(ctx->g, src, &made) == cudaSuccess)
       map = &made;
     e = launch_stage_fp64(ctx->g, a, ctx->stream, fp64_cfg(ctx, ctx->tile), map, ctx->err);
     if (e != cudaSuccess) return cuda_fail(e, "bssn_rhs interior");

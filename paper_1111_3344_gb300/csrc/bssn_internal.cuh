@@ -319,7 +319,7 @@ cudaError_t launch_stage_fp64(const Grid& g, const StageArgs& a, cudaStream_t s,
                               const CUtensorMap* map = nullptr, int* err = nullptr);
 bool fx_tile_fits(const Grid& g);
 bool fx_launch_early(const Grid& g);  // the kernels of a step are short: their launches overlap (launch_after)
-cudaError_t make_fx_tensor_map(const Grid& g, const double* base, CUtensorMap* out, bool bound = false);
+cudaError_t make_fx_tensor_map(const Grid& g, const double* base, CUtensorMap* out);
 cudaError_t launch_stage_fx(const Grid& g, const StageArgs& a, const CUtensorMap& map, int* err, cudaStream_t s);
 cudaError_t launch_stage_mixed(const Grid& g, const StageArgsMixed& a, cudaStream_t s, int cfg = 0);
 cudaError_t launch_stage_mixed_ks64(const Grid& g, const StageArgsMixed& a, cudaStream_t s);
@@ -331,9 +331,8 @@ const char* tile_config_name(int c);
 // stage buffer that is the stencil source.
 // Tensor map of a register as [field][z][y][x] (elem bytes: 4 float, 8 float64)
 // with a box of bx x by x bz points of one field.
-// bound: the calling thread has made a runtime call that binds its context.
-cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out,
-                              bool bound = false);
+// (Allowed while the calling thread captures a stream.)
+cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out);
 // Tensor map of a float stage buffer for TMA-staged variant v (0: 32 x 4 x 1
 // tiles, 1: 32 x 8 x 1, 2: 32 x 2 x 4; the box is the tile plus three ghost layers).
 cudaError_t make_stage_tensor_map(const Grid& g, const float* base, CUtensorMap* out, int variant = 0);

@@ -208,11 +208,11 @@ __global__ void __launch_bounds__(GROUPS * FxT::THREADS, 1)
 
 // (and the shared-memory limit of the kernel that may read through the map, so
 // that launches under capture need no other call)
-cudaError_t make_fx_tensor_map(const Grid& g, const double* base, CUtensorMap* out, bool bound) {
+cudaError_t make_fx_tensor_map(const Grid& g, const double* base, CUtensorMap* out) {
   static std::atomic<unsigned> done{0};
   const cudaError_t e = smem_optin(stage_fx_wide_kernel, sizeof(FxWideShared<FxT>), done);
   if (e != cudaSuccess) return e;
-  return encode_tensor_map(g, base, 8, FxT::BX, FxT::BY, FxT::BZ, out, bound);
+  return encode_tensor_map(g, base, 8, FxT::BX, FxT::BY, FxT::BZ, out);
 }
 
 // Up to three tiles per SM one after another: ms a stage with groups, without:

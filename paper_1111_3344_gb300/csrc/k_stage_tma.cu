@@ -87,14 +87,18 @@ bool half_tiles(const Grid& g) {
 }
 }
 
-cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out,
-                              bool bound) {
+cudaError_t encode_tensor_map(const Grid& g, const void* base, int elem, int bx, int by, int bz, CUtensorMap* out) {
   // the encoding is a driver call and needs a current context: a thread whose
   // first CUDA call this is has none until a runtime call binds the primary
-  // context of its device (cudaFree(nullptr) does, and frees nothing; it is no
-  // call for a stream capture: bound says that one has been made)
-  cudaError_t ce = bound ? cudaSuccess : cudaFree(nullptr);
+  // context of its device (cudaFree(nullptr) does, and frees nothing).  A stream
+  // capture of this thread forbids that call and would be lost by it, unless the
+  // thread's mode is relaxed meanwhile.
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t ce = cudaThreadExchangeStreamCaptureMode(&mode);
   if (ce != cudaSuccess) return ce;
+  ce = cudaFree(nullptr);
+  const cudaError_t ce2 = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (ce != cudaSuccess || ce2 != cudaSuccess) return ce != cudaSuccess ? ce : ce2;
   if (!g_encode) {
     cudaDriverEntryPointQueryResult q;
     cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", (void**)&g_encode, 12000,
