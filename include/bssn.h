@@ -326,7 +326,10 @@ bssn_status bssn_set_staging(bssn_ctx* ctx, void* d_mem, size_t bytes);
  * The "ff..." configurations (last) are those of double-word precision, and the
  * same kernel.
  * Every configuration evaluates the same per-point arithmetic, so results agree
- * to rounding and each configuration is reproducible bit for bit. */
+ * to rounding and each configuration is reproducible bit for bit.  (In float64
+ * "32x4x1/1" has two forms, equal to rounding: in tiles, and one point at a time
+ * where tiles fit the grid badly and for bssn_rhs of a register that is not
+ * 16-byte aligned.  The others always go one point at a time.) */
 int32_t bssn_tile_count(void);
 const char* bssn_tile_name(int32_t cfg); /* e.g. "32x8x1/1"; "" when out of range */
 bssn_status bssn_set_tile(bssn_ctx* ctx, int32_t cfg);
@@ -355,8 +358,11 @@ bssn_status bssn_autotune(bssn_ctx* ctx, int32_t reps, int32_t* best, double* ms
  *    kernels, one launch chain per member, the chains side by side on 16, 4
  *    or 1 auxiliary streams inside the graph, which is captured again when
  *    the membership changes.
- * A member computes the same bits as the same evolution run alone through a
- * bssn_ctx.  All device memory comes from the caller's pool: the batch tables
+ * A member computes the same bits whichever other members share the batch; under
+ * the per-member configurations also the bits of the same evolution run alone
+ * through a bssn_ctx on the same tile configuration (the defaults of both).
+ * The work-list configurations of float64 go one point at a time and equal that
+ * to rounding.  All device memory comes from the caller's pool: the batch tables
  * (bssn_batch_table_bytes) at its start, then member registers carved by a
  * first-fit sub-allocator (bssn_batch_member_bytes each). */
 #define BSSN_BATCH_MAX_MEMBERS 256
