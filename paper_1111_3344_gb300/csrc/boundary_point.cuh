@@ -8,14 +8,6 @@
 
 namespace bssn {
 
-__device__ __forceinline__ void x0v0(const Grid& g, int f, double& X0, double& v0) {
-  X0 = 0.0;
-  v0 = 1.0;
-  if (f == F_ALP || (f == F_CHI && g.use_w) || f == F_GT + 0 || f == F_GT + 3 || f == F_GT + 5)
-    X0 = 1.0;
-  if (f == F_ALP || f == F_TRK) v0 = 1.4142135623730951;
-}
-
 __device__ __forceinline__ double coordv(const Grid& g, int d, int i) {
   const double xm = d == 0 ? g.xmin0 : (d == 1 ? g.xmin1 : g.xmin2);
   return xm + (i - GH + 0.5) * g.h;

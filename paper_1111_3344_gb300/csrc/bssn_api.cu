@@ -354,7 +354,7 @@ bssn_status bssn_alloc(const bssn_params* p, void* d_mem, size_t bytes, void* cu
     // the 11-field TMA stage: the same bits as the fused kernels and the
     // fastest configuration at every size measured (one step, against the fused
     // 32x8x1, which took 0.145 ms at 24^3, 0.48 at 48^3, 5.37 at 128^3, 43.2 at
-    // 256^3: 0.13, 0.34, 3.71, 27.7)
+    // 256^3: 0.13, 0.30, 3.71, 27.7)
     if (ok) ctx->tile = tile_config_count() + 2;
   }
   ctx->cstream = ctx->istream = nullptr;

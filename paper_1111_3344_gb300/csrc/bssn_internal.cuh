@@ -74,14 +74,6 @@ inline void grid_constants(Grid& g) {
   g.xminf[2] = (float)g.xmin2;
 }
 
-// Pick the float64 or float copy of a constant.
-template <typename T>
-__host__ __device__ __forceinline__ T gc(double d, float f);
-template <>
-__host__ __device__ __forceinline__ double gc<double>(double d, float) { return d; }
-template <>
-__host__ __device__ __forceinline__ float gc<float>(double, float f) { return f; }
-
 // Raise kernel's dynamic shared-memory limit to bytes on the current device,
 // once per device: the attribute belongs to the kernel as loaded in that
 // device's context.  done holds one bit per device (devices 32 and up set the
@@ -137,8 +129,6 @@ __device__ __forceinline__ void after_previous() {
 
 template <typename T>
 constexpr bool is_f32 = std::is_same<T, float>::value;
-template <typename T>
-constexpr bool is_f64 = std::is_same<T, double>::value;
 
 // Matter projections of T_{mu nu} at linear index id (Sec. "Spacetime Curvature
 // Evolution"): E = (T_00 - 2 beta^i T_0i + beta^i beta^j T_ij)/alpha^2,

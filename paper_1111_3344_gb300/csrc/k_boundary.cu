@@ -13,7 +13,8 @@
 //   rhs_b = rad_b + (r_a / r_b)^2 (rhs_a - rad_a),
 // so each ghost point is independent: one thread per ghost point, no layer
 // ordering.  X0 = 1 for alpha, W and the diagonal of gt, else 0; v0 = sqrt 2
-// for alpha and K, else 1.  The boundary arithmetic is float64 on both paths.
+// for alpha and K, else 1.  On the mixed path the boundary arithmetic is float,
+// W's float64.
 #include "boundary_point.cuh"
 
 namespace bssn {
@@ -67,10 +68,9 @@ cudaError_t launch_ghost_table(const Grid& g, void* table, cudaStream_t s) {
 }
 size_t ghost_table_size(const Grid& g) { return ghost_table_bytes(g); }
 
-// one thread per ghost point, every field (geometry formed once)
-// mixed: blockIdx.y picks one of four field groups (W and gt_ij; K and
-// At_ij but its last; the rest of At_ij, Gt^i, alpha; beta^i and B^i), each
-// a few unrolled fields per thread.  Bound by load latency: every load of a
+// Mixed: one thread per ghost point and field group; blockIdx.y picks one of four
+// groups (W and gt_ij; K and At_ij but its last; the rest of At_ij, Gt^i, alpha;
+// beta^i and B^i), each a few unrolled fields per thread.  Bound by load latency: every load of a
 // group comes before its stores and under no branch (loads and stores of one
 // field after another, the neighbours of each under its own branches: 34 us
 // at 48^3, 175 at 128^3; so 25 and 139).  Interleaving the groups' blocks (31 at

@@ -123,17 +123,11 @@ __device__ __forceinline__ double up_coef(bool pos, int m) {
   const double cn[7] = {1.0, -6.0, 18.0, -10.0, -3.0, 0.0, 0.0};
   return pos ? cp[m + 3] : cn[m + 3];
 }
-// the same weight in the arithmetic type T (float: from the float constants,
-// which hold these small integers exactly)
-template <typename T>
-__device__ __forceinline__ T up_coefT(bool pos, int m) {
-  if constexpr (is_f64<T>) {
-    return up_coef(pos, m);
-  } else {
-    const float cp[7] = {0.0f, 0.0f, -3.0f, -10.0f, 18.0f, -6.0f, 1.0f};
-    const float cn[7] = {1.0f, -6.0f, 18.0f, -10.0f, -3.0f, 0.0f, 0.0f};
-    return T(pos ? cp[m + 3] : cn[m + 3]);
-  }
+// the same weight in float (which holds these small integers exactly)
+__device__ __forceinline__ float up_coeff(bool pos, int m) {
+  const float cp[7] = {0.0f, 0.0f, -3.0f, -10.0f, 18.0f, -6.0f, 1.0f};
+  const float cn[7] = {1.0f, -6.0f, 18.0f, -10.0f, -3.0f, 0.0f, 0.0f};
+  return pos ? cp[m + 3] : cn[m + 3];
 }
 
 // Background value X0 of field f (1 for W, the diagonal of gt and alpha; 0
@@ -151,9 +145,9 @@ __host__ __device__ __forceinline__ double background(const Grid& g, int f) {
 template <typename T, typename S, bool DEV, typename A>
 __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i, int j, int k,
                                               T out[NF]) {
-  const T i12h = gc<T>(g.i12h, g.i12hf);
-  const T i12h2 = gc<T>(g.i12h2, g.i12h2f);
-  const T i144h2 = gc<T>(g.i144h2, g.i144h2f);
+  const T i12h = g.i12hf;
+  const T i12h2 = g.i12h2f;
+  const T i144h2 = g.i144h2f;
 #define PF(f) acc.ptr(f)
 #define SD(f, d) acc.s((f), (d))
 #define LD(f, p) acc.template ld<T>((f), (p))
@@ -189,7 +183,7 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
     T det = gt[0] * c00 + gt[1] * c01 + gt[2] * c02;
     T idet;
     if (g.use_w) {
-      const T wf = gc<T>(g.w_floor, g.w_floorf);
+      const T wf = g.w_floorf;
       const T Wd = chi > wf ? chi : wf;
       const T r = T(1) / (det * Wd);
       idet = Wd * r;
@@ -567,7 +561,7 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       out[F_BETA + a] = T(0.75) * Bv[a];
-      out[F_B + a] = gam_rhs[a] - gc<T>(g.eta, g.etaf) * q * Bv[a];
+      out[F_B + a] = gam_rhs[a] - g.etaf * q * Bv[a];
     }
   }
 
@@ -581,7 +575,7 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
     for (int f = 0; f < NF; f++)
       if (f < nf) out[f] += acc.template advko<T>(f);
   } else {
-    const T kap = gc<T>(g.kos, g.kosf);
+    const T kap = g.kosf;
     T f0s[NF];  // centre values as stored (float: the stencil is applied to f_m - f0)
     T bh[3];
 #pragma unroll
@@ -609,7 +603,7 @@ __device__ __forceinline__ void rhs_point_acc(const Grid& g, const A& acc, int i
       T w[7];
 #pragma unroll
       for (int m = -3; m <= 3; m++)
-        if (m != 0) w[m + 3] = fmaT<T>(bh[d], up_coefT<T>(pos, m), kap * cko[m + 3]);
+        if (m != 0) w[m + 3] = fmaT<T>(bh[d], up_coeff(pos, m), kap * cko[m + 3]);
 #pragma unroll
       for (int f = 0; f < NF; f++) {
         if (f >= nf) break;

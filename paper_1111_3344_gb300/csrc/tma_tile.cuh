@@ -78,8 +78,8 @@ using TileAcc = TileAccT<TmaDefault>;
 
 // Thread 0: arm the barrier for the staged bytes and issue one tensor load per
 // staged field, box origin (x0, y0, z0) in stored coordinates (the interior
-// start of the tile minus the ghost width; x0 a multiple of 32, so the
-// innermost offset is a multiple of 16 bytes).  The tensor map's box is
+// start of the tile minus the ghost width; x0 a multiple of the
+// tile's x extent, 16 or 32, so the innermost offset is a multiple of 16 bytes).  The tensor map's box is
 // Sh::BX x Sh::BY x Sh::BZ.
 template <typename Sh = TmaDefault>
 __device__ __forceinline__ void issue_staged_loads(const void* tmap, unsigned bar, float* smem, int x0, int y0,
