@@ -43,16 +43,17 @@ constexpr int FX_TILE_BITS = 4;
 
 // A thread whose star -- the point and those one and two away along each axis: the
 // values of its pure derivatives -- reaches no 2^(FX_NEAR - 1) units at the point
-// or two away (an eighth of the box's largest exponent) takes its own alignment:
-// an integer's rounding, half a unit, is then at most 2^-54 of the star's largest
-// value, the bound of rhs_fx.cuh.  (Shift and B^i as Gaussians of width 1 at h =
-// 0.25, relative error of the shift's right-hand side at each point, 90th and
-// 99th percentile: 3e-16 and 9e-16; without this rule 2e-11 and 4e-9; float64
-// stencils 1e-15 and 3e-15.)  A step at 128^3 takes 15.7 -> 15.8 ms for it, 75 x
-// 53 x 61 2.58 -> 2.69, 24^3 0.206 -> 0.220: the threads that take their own
-// alignment hold up their block.  With three bits below the box's last (and a
-// quarter in place of an eighth) 15.8, 2.74, 0.222.
-constexpr int FX_NEAR = 54;
+// or two away (a sixteenth of the box's largest exponent) takes its own alignment:
+// an integer's rounding, half a unit, is then at most 2^-53 of the star's largest
+// value, as float64 rounds that value itself.  (Shift and B^i as Gaussians of
+// width 1 at h = 0.25, relative error of the shift's right-hand side at each
+// point, 90th and 99th percentile: 4e-16 and 2e-15; without this rule 2e-11 and
+// 4e-9; float64 stencils 1e-15 and 3e-15.)  A step at 128^3 takes 15.72 -> 15.78 ms
+// for it, 75 x 53 x 61 2.58 -> 2.61, 24^3 0.208 -> 0.210: the threads that take
+// their own alignment hold up their block.  One bit more 15.82, 2.69 and 0.222,
+// for 3e-16 and 9e-16; three threads sharing a point's three axes 16.1, 2.70 and
+// 0.218.
+constexpr int FX_NEAR = 53;
 // a bound on |v|'s high word, whose leading bit is that of |v| (or of |v| - 1)
 __device__ __forceinline__ int fx_mag(long long v) {
   const int hi = (int)(v >> 32);

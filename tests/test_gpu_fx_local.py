@@ -3,7 +3,7 @@ aligning a stencil's values to the largest among several (csrc/fx.cuh) or in a
 tile's whole box (csrc/rhs_fx_tile.cuh) must not cost a derivative the bits by
 which values that it does not use exceed its own.
 
-Bars.  A stencil's values are held to 2^-54 of their largest or better and its sums
+Bars.  A stencil's values are held to 2^-53 of their largest or better and its sums
 to a few 2^-53, so a point's right-hand side is off by some hundred times 2^-53 M,
 M the oracle's magnitude of the same expression at the same point: 1e-12 M has
 a factor of 30 to spare.  The grids run both forms of the stage in tiles (up to
