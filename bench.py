@@ -54,12 +54,12 @@ DOMAIN = 8.0
 ALG_BYTES_PER_POINT_STEP = {"fp64": 3072.0, "mixed": 2496.0, "ff": 3072.0}
 # Float64 work the stage kernels execute per interior point per launch
 # (right-hand side plus RK4 combine), from ncu instruction counts at 96^3
-# (DADD + DMUL + 2 DFMA): the tile form (configuration 32x4x1/1) 62 DADD + 119
-# DMUL + 631 DFMA; the point form 114 DADD + 156 DMUL + 796 DFMA.
-FLOP_PER_POINT_RHS = 1443.0
-DPINST_PER_POINT_RHS = 812.0
-FLOP_PER_POINT_RHS_POINT = 1862.0
-DPINST_PER_POINT_RHS_POINT = 1066.0
+# (DADD + DMUL + 2 DFMA): the tile form (configuration 32x4x1/1) 62 DADD + 116
+# DMUL + 691 DFMA; the point form 114 DADD + 156 DMUL + 844 DFMA.
+FLOP_PER_POINT_RHS = 1560.0
+DPINST_PER_POINT_RHS = 869.0
+FLOP_PER_POINT_RHS_POINT = 1958.0
+DPINST_PER_POINT_RHS_POINT = 1114.0
 # Operations of one right-hand side at an interior point in the oracle's
 # printed arrangement (its instrumented build, W variant, Gamma-driver shift:
 # 5395 additions, 7874 multiplications, 299 divisions).  The arrangement
@@ -75,7 +75,7 @@ ORACLE_FLOP_PER_POINT_RHS = 5395 + 7874 + 299
 # (where the share of ghosts, padding and L2 hits differs), reports null.
 TRAFFIC_N = 128
 STAGE_TRAFFIC_PER_POINT = {
-    ("fp64", "32x4x1/1"): 4195.0,       # stage_fx_kernel: 35190.8 MB per step, most of it local memory
+    ("fp64", "32x4x1/1"): 4221.5,       # stage_fx_kernel: 35412.6 MB per step, most of it local memory
     ("mixed", "tma32x4x1/2"): 565.3,   # stage_mixed_tma_kernel, 8 staged fields: 4741.9 MB per step
     ("mixed", "tma11_32x8x1/1"): 569.3,  # stage_mixed_tma_kernel, 11 staged fields: 4775.7 MB per step
 }
@@ -83,7 +83,7 @@ STAGE_TRAFFIC_PER_POINT = {
 # from ncu instruction counts at 96^3).  psi4 and constraints include the
 # ADM-field pass that precedes them (36 flop per stored point, 44 per
 # interior point at 96^3).
-ANALYSIS_FLOP_PER_POINT = {"psi4": 3409.0 + 44.0, "adm_integrals": 1771.9, "constraints": 1999.0 + 44.0}
+ANALYSIS_FLOP_PER_POINT = {"psi4": 735.0 + 44.0, "adm_integrals": 895.3, "constraints": 520.3 + 44.0}
 
 
 def _measured_hbm_gbs(default=6764.0):
