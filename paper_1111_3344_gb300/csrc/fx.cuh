@@ -10,8 +10,10 @@
 //    sixteen) are aligned to the largest exponent E among them: a value becomes
 //    its 53-bit significand times 2^FX_BITS (sign applied), shifted right by E
 //    minus its own exponent;
-//  - the sums of these integers are exact; FX_BITS = 2 leaves the headroom for
-//    the largest coefficient sum, 192 (|sum| < 192 2^55 < 2^63);
+//  - the sums of these integers are exact (an axis' sums that the third
+//    neighbours enter are shifted right first where those are larger, and lose a
+//    unit of theirs at most); FX_BITS = 2 leaves the headroom for the largest
+//    coefficient sum, 192 (|sum| < 192 2^55 < 2^63);
 //  - the result is rounded to float64 once.
 // The only other error is the bits shifted out of the values whose magnitude
 // is below a quarter of the largest: at most 2^-54 of that largest value each, a

@@ -1,10 +1,10 @@
 // Float64 fused stage in tiles (rhs_fx_tile.cuh): one block per tile of 8 x 4 x 4
 // interior points, one thread per point.
 //
-// Bound: the float64 pipe (some 870 instructions of 64 cycles for a warp's
+// Bound: the float64 pipe (869 instructions of 64 cycles for a warp's
 // points), the integer stencils beside it.  Shape and occupancy: six blocks of 128
 // threads per SM (80 registers, 33 KB of shared memory each).  A step at 128^3
-// 15.8 ms; one point at a time 19.7, before that with float64 stencils 33.1.
+// 15.8 ms; one point at a time 20, before that with float64 stencils 33.1.
 // Found with slightly cheaper sums (a stage then 3.51-3.65 ms): with 4, 5, 7, 8
 // blocks 4.1, 3.8, 3.6, 3.7; tiles of 16 x 4 x 2 3.65, 16 x 2 x 4 3.68, 8 x 8 x 2
 // 3.60, 8 x 8 x 4 3.95, 32 x 2 x 2 4.4 (a flatter tile converts more box points per
@@ -225,11 +225,14 @@ static long long fx_tiles(const Grid& g) {
 }
 bool fx_launch_early(const Grid& g) { return fx_tiles(g) <= 2 * 152; }
 
-// A tile takes as long with points past the grid as without, 0.73 of the time
+// A tile takes as long with points past the grid as without, 0.75 of the time
 // of the same points one at a time (k_stage.cu: blocks of consecutive points, no
 // padding).  Measured, ms a stage, tile against point form, with the share of
-// threads that have a point: 121^3 0.90 3.23 / 4.23; 41^3 0.74 0.210 / 0.222;
-// 33^3 0.69 0.157 / 0.145; 9 x 200 x 200 0.56 1.11 / 0.97: tiles from 0.72 on.
+// threads that have a point: 121^3 0.90 3.18 / 3.71; 73^3 0.84 0.808 / 0.867; 50^3
+// 0.83 0.310 / 0.334; 41^3 0.74 0.197 / 0.209; 33^3 0.69 0.157 / 0.145; 9 x 200 x
+// 200 0.56 1.11 / 0.97: tiles from 0.72 on.  (On smooth data; while a puncture's
+// fields still fall off steeply and many points take their own alignment 3.34,
+// 0.889, 0.363, 0.248.)
 // With few tiles one block's latency counts, whatever the padding (129 x 5 x 5
 // 0.052 / 0.144, 33^3 with groups 0.144 / 0.147).
 bool fx_tile_fits(const Grid& g) {

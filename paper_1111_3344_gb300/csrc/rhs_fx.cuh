@@ -6,7 +6,7 @@
 // Bound: the float64 pipe, 64 cycles of an SM sub-partition for a warp
 // instruction.  With the stencils in float64 a point took 1906 of them; here
 // the stencils leave 6 per field (advection and dissipation) and none for the
-// derivatives, the algebra about 830.  The integer work, some 25,000
+// derivatives, the algebra and the combine about 970.  The integer work, some 25,000
 // instructions a point, runs beside the float64 pipe.
 //
 // Advection: the lopsided stencil is the mean of the KO sum K and the odd sum O =

@@ -4,7 +4,7 @@
 //
 // One point at a time (rhs_fx.cuh), every stencil aligns its own 19 to 67
 // values: some 25,000 integer instructions a point, as long as the float64
-// pipe is busy (1016 instructions of 64 cycles for a warp).  Here a block loops
+// pipe is busy (1114 instructions of 64 cycles for a warp).  Here a block loops
 // over the fields:
 //  - A tensor load brings the field's box (the tile and three points on every
 //    side) into one of two buffers while the other's field is worked on.
@@ -17,20 +17,25 @@
 //  - A thread then reads its taps (67 for a twice-differenced field) with fixed
 //    offsets and no conversion.  Advection and dissipation are one sum of four
 //    products with weights of the point, kept as integers too (fx_weight,
-//    fx_dot); the contraction gt^kl d_k d_l is float64: some 870 float64
+//    fx_dot); the contraction gt^kl d_k d_l is float64: 869 float64
 //    instructions a point.
 //  - Where the box's largest value is much more than what a thread's star holds,
 //    the box's integers have fewer bits than the thread's own values.  That thread
 //    takes the field's stencils one point at a time from the register (FX_NEAR,
 //    fx_stencils_own), so that every point is as exact as rhs_fx.cuh makes it: a
 //    field that falls off steeply inside a tile, a small value beside a large one.
-//    On smooth data some percent of the warps or fewer do.
+//    On smooth data some percent of the warps or fewer do.  In the first tens of
+//    steps of a puncture, whose shift, B^i and Gt^i start from zero and fall off
+//    steeply, one to two of a warp's 24 fields at 64^3, 0.16 at 128^3: a step of
+//    64^3 takes 2.75 ms then, 2.58 after 150 steps, 2.46 without (the rule's own
+//    code and the loop's together exceed the instruction cache).
 //  - The algebra runs inside the loop as soon as its fields are there, so that
 //    few results wait at a time (33 local slots).
 // The stencil code exists once: the instruction cache holds 128 KB, and a
 // float64 instruction takes five instruction slots.  Neither part alone fills
-// the time (128^3, cycles of an SM sub-partition for a warp's points: algebra
-// 58-61 thousand, the loop without it 56, together 68; per-point form 88).
+// the time (128^3, cycles of an SM sub-partition for a warp's points, with sums
+// that took 57 float64 instructions fewer: algebra 58-61 thousand, the loop
+// without it 56, together 68; per-point form 88; now 71).
 #pragma once
 #include "fx.cuh"
 #include "fx_algebra.cuh"
